@@ -93,7 +93,7 @@ def draw(rng):
                      "broadening": 2.0, "omegas": rng.randint(50, 400), "axis": rng.randint(0, 2)})
     else:
         n = rng.choice([16, 20, 24, 27, 32, 40, 48, 64])
-        case = {"kind": "fno", "n": n, "width": rng.randint(4, 32), "modes": rng.randint(2, min(12, n // 2)),
+        case = {"kind": "fno", "n": n, "width": 2 * rng.randint(2, 16), "modes": rng.randint(2, min(12, n // 2)),
                 "layers": rng.randint(1, 4), "batch": rng.randint(1, 4), "train": rng.random() < 0.5}
     return case
 
