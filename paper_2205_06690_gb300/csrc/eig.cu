@@ -1,13 +1,14 @@
 // Lowest eigenvalues of the real symmetric Tamm-Dancoff matrix A (Eq. 1), in FP64 on the device:
-// Householder reduction to tridiagonal form (one block, matrix in global memory / L2) followed by
-// Sturm-sequence bisection, one thread per requested eigenvalue.
+// Householder reduction to tridiagonal form (one thread-block cluster, the matrix in its distributed
+// shared memory) followed by Sturm-sequence multisection, one warp per requested eigenvalue.
+#include <cooperative_groups.h>
 #include <math.h>
 
 #include "kernels.h"
 
 namespace sbse {
 
-constexpr int kEigThreads = 1024;
+namespace cg = cooperative_groups;
 
 __device__ double block_sum(double v, double *red) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -25,27 +26,141 @@ __device__ double block_sum(double v, double *red) {
   return red[32];
 }
 
-// A (n x n, row-major, overwritten) -> diagonal dg[n] and off-diagonal of[n-1].
-// H = I - beta v v^T maps A[k+1:, k] onto alpha e_1; the trailing block becomes
-// A' - v w^T - w v^T with p = beta A' v, K = beta v.p / 2, w = p - K v.
-// INSMEM: the matrix is first copied to shared memory (small n), otherwise it stays in global
-// memory (L2-resident for the sizes of A).
+// Householder reduction of A (n x n, row-major, symmetric) to the diagonal dg[n] and off-diagonal
+// of[n-1] by one thread-block cluster. H = I - beta v v^T maps A[k+1:, k] onto alpha e_1; the trailing
+// block becomes A' - v w^T - w v^T with p = beta A' v, K = beta v.p / 2, w = p - K v.
+// Rows are dealt to the CTAs in turn (row i to CTA i mod size: even shares while the trailing block
+// shrinks) and stay in their shared memory (INSMEM; else in global memory, L2-resident, overwritten).
+// Two exchanges a step, each CTA writing its entries into every CTA's copy through distributed shared
+// memory: the column x, from which all CTAs form v alike, and p. The rank-2 update of step k - 1 is
+// applied in the sweep that forms p of step k, so a row is read once per step.
+// Bound: 3 m^2 FP64 multiply-adds per step over the cluster's SMs (1.6 per clock and SM) and the latency
+// of two cluster barriers and two block sums. One block of 1024 threads took 64.2 ms at n = 512 and
+// 2.58 ms at n = 128; the cluster of 16 takes 4.96 ms and 0.58 ms. A grid-wide barrier over all SMs
+// would cut the arithmetic further but costs several times a cluster barrier, about what it saves.
 // refl != null: the Householder vector of step k is stored in row k of refl (entries k+1 .. n-1)
 // and its beta in betas[k] (0 where the step is the identity), for the back-transformation of
 // eigenvectors.
+// An FP64 instruction holds its SM sub-partition for about 64 clocks whatever the warp's active lanes, so
+// the scalars (square root, division) are formed by one thread and the sums by one warp per
+// sub-partition.
+constexpr int kTriThreads = 512;
+
+__host__ __device__ inline int tri_rows(int n, int cs) { return (n + cs - 1) / cs; }
+// shared memory beyond the rows: x, v, the previous v and w, p (n each) and the scalars
+__host__ __device__ inline size_t tri_vec_doubles(int n) { return 5 * (size_t)n + 8; }
+
+// partial sums of a_i b_i, o <= i < n, into red[0..3] (first four warps); the caller synchronises
+__device__ __forceinline__ void tri_dot(const double *a, const double *b, int o, int n, double *red) {
+  if (threadIdx.x < 128) {
+    double s = 0.0;
+    for (int i = o + threadIdx.x; i < n; i += 128) s = fma(a[i], b[i], s);
+    for (int q = 16; q > 0; q >>= 1) s += __shfl_xor_sync(0xffffffffu, s, q);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  }
+}
+
 template <bool INSMEM>
+__global__ void __launch_bounds__(kTriThreads)
+    k_tridiag(const double *Ain, double *Ag, int n, double *dg, double *of, double *refl, double *betas) {
+  extern __shared__ double sm[];
+  cg::cluster_group cl = cg::this_cluster();
+  const int cs = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  double *x = sm, *v = x + n, *vp = v + n, *wp = vp + n, *p = wp + n, *red = p + n;  // red: 4 sums, beta, K
+  double *rows = INSMEM ? red + 8 : Ag;
+  // row i (owned: i % cs == rank)
+  auto row = [&](int i) { return INSMEM ? rows + (size_t)(i / cs) * n : rows + (size_t)i * n; };
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
+  for (int i = rank + cs * warp; i < n; i += cs * nw) {
+    double *r = row(i);
+    for (int j = lane; j < n; j += 32) r[j] = Ain[(size_t)i * n + j];
+  }
+  for (int i = tid; i < n; i += blockDim.x) vp[i] = wp[i] = 0.0;
+  cl.sync();  // (also orders the CTA's own rows)
+  for (int k = 0; k + 2 < n; ++k) {
+    const int o = k + 1;
+    const int first = o + ((rank - o) % cs + cs) % cs;  // first owned row >= o
+    // column k below the diagonal with the pending update, written to every CTA's x
+    if (warp == 0) {
+      const double vk = vp[k], wk = wp[k];
+      for (int i = first + lane * cs; i < n; i += 32 * cs) {
+        const double xi = fma(-wp[i], vk, fma(-vp[i], wk, row(i)[k]));
+        for (int dst = 0; dst < cs; ++dst) *cl.map_shared_rank(x + i, dst) = xi;
+      }
+    } else if (warp == 1 && lane == 0 && k % cs == rank) {
+      dg[k] = fma(-2.0 * vp[k], wp[k], row(k)[k]);
+    }
+    cl.sync();
+    tri_dot(x, x, o, n, red);
+    for (int i = o + tid; i < n; i += blockDim.x) v[i] = x[i];
+    __syncthreads();
+    if (tid == 0) {
+      const double sigma = (red[0] + red[1]) + (red[2] + red[3]), x0 = x[o];
+      double alpha = x0, beta = 0.0;
+      if (!(sigma - x0 * x0 <= 0.0)) {  // else the step is the identity (beta = 0)
+        alpha = x0 >= 0.0 ? -sqrt(sigma) : sqrt(sigma);
+        beta = 1.0 / (sigma - x0 * alpha);  // 2 / |v|^2
+        v[o] = x0 - alpha;
+      }
+      red[4] = beta;
+      if (rank == 0) {
+        of[k] = alpha;
+        if (betas) betas[k] = beta;
+      }
+    }
+    __syncthreads();
+    const double beta = red[4];
+    if (refl && k % cs == rank && beta != 0.0)
+      for (int i = o + tid; i < n; i += blockDim.x) refl[(size_t)k * n + i] = v[i];
+    // the pending update of the owned rows and p = beta A' v, one warp per row
+    for (int i = first + cs * warp; i < n; i += cs * nw) {
+      double *r = row(i);
+      const double vi = vp[i], wi = wp[i];
+      double s = 0.0;
+      for (int j = o + lane; j < n; j += 32) {
+        const double aij = fma(-wi, vp[j], fma(-vi, wp[j], r[j]));
+        r[j] = aij;
+        s = fma(aij, v[j], s);
+      }
+      for (int q = 16; q > 0; q >>= 1) s += __shfl_xor_sync(0xffffffffu, s, q);
+      if (lane < cs) *cl.map_shared_rank(p + i, lane) = beta * s;
+    }
+    cl.sync();
+    tri_dot(v, p, o, n, red);
+    __syncthreads();
+    if (tid == 0) red[5] = 0.5 * beta * ((red[0] + red[1]) + (red[2] + red[3]));
+    __syncthreads();
+    const double K = red[5];
+    for (int i = o + tid; i < n; i += blockDim.x) {  // a step that is the identity leaves v = w = 0 pending
+      const double vi = beta != 0.0 ? v[i] : 0.0;
+      vp[i] = vi;
+      wp[i] = fma(-K, vi, p[i]);
+    }
+    __syncthreads();
+  }
+  // the last 2 x 2 block, with the pending update
+  if (tid == 0) {
+    const int a = n - 2, b = n - 1;
+    if (a % cs == rank) dg[a] = fma(-2.0 * vp[a], wp[a], row(a)[a]);
+    if (b % cs == rank) {
+      dg[b] = fma(-2.0 * vp[b], wp[b], row(b)[b]);
+      of[a] = fma(-wp[b], vp[a], fma(-vp[b], wp[a], row(b)[a]));
+    }
+  }
+  cl.sync();  // no CTA leaves while another may still write into its shared memory
+}
+
+// The same reduction by one block with the matrix in global memory, for sizes whose five vectors do not
+// fit the shared memory of a cluster's CTAs (n > kTriMaxN).
+constexpr int kEigThreads = 1024;
+constexpr int kTriMaxN = 5000;
+
 __global__ void __launch_bounds__(kEigThreads)
-    k_tridiag(double *Ag, int n, double *dg, double *of, double *refl, double *betas) {
+    k_tridiag_block(double *A, int n, double *dg, double *of, double *refl, double *betas) {
   extern __shared__ double sm[];
   double *v = sm;
   double *p = v + n;
   double *red = p + n;  // 33 doubles
-  double *A = Ag;
-  if (INSMEM) {
-    A = red + 34;
-    for (long long l = threadIdx.x; l < (long long)n * n; l += blockDim.x) A[l] = Ag[l];
-    __syncthreads();
-  }
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
   for (int k = 0; k + 2 < n; ++k) {
     const int m = n - k - 1;
@@ -110,49 +225,161 @@ __global__ void __launch_bounds__(kEigThreads)
   }
 }
 
-// number of eigenvalues of the tridiagonal (dg, of) below x (Sturm count by LDL^T pivots)
-__device__ int sturm_count(const double *dg, const double *of, int n, double x, double tiny) {
-  int c = 0;
-  double q = dg[0] - x;
-  if (q == 0.0) q = -tiny;
-  if (q < 0.0) ++c;
-  for (int i = 1; i < n; ++i) {
-    q = dg[i] - x - of[i - 1] * of[i - 1] / q;
-    if (q == 0.0) q = -tiny;
-    if (q < 0.0) ++c;
+// k_tridiag on the largest cluster that its shared memory and the device allow (16 CTAs need the
+// opt-in; small matrices take fewer, with at least 8 rows each)
+static void launch_tridiag(const double *A, double *Aw, int n, double *dg, double *of, double *refl, double *betas,
+                           cudaStream_t s) {
+  if (n > kTriMaxN) {
+    const size_t sm = (2 * (size_t)n + 34) * sizeof(double);
+    raise_smem_limit((const void *)k_tridiag_block, sm);
+    cudaMemcpyAsync(Aw, A, (size_t)n * n * sizeof(double), cudaMemcpyDeviceToDevice, s);
+    k_tridiag_block<<<1, kEigThreads, sm, s>>>(Aw, n, dg, of, refl, betas);
+    count_launch(1);
+    return;
   }
+  for (int cs = 16; cs >= 1; cs >>= 1) {
+    if (cs > 1 && n < 8 * cs) continue;
+    const size_t vec = tri_vec_doubles(n) * sizeof(double);
+    const size_t full = vec + (size_t)tri_rows(n, cs) * n * sizeof(double);
+    const bool in = full <= 200 * 1024;
+    const void *fn = in ? (const void *)k_tridiag<true> : (const void *)k_tridiag<false>;
+    const size_t smem = in ? full : vec;
+    if (smem > 48 * 1024) raise_smem_limit(fn, smem);
+    if (cs > 8 && cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+      cudaGetLastError();
+      continue;
+    }
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)cs);
+    cfg.blockDim = dim3(kTriThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)cs;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int fit = 0;
+    if (cs > 1 && (cudaOccupancyMaxActiveClusters(&fit, fn, &cfg) != cudaSuccess || fit < 1)) {
+      cudaGetLastError();
+      continue;
+    }
+    if (in)
+      cudaLaunchKernelEx(&cfg, k_tridiag<true>, A, Aw, n, dg, of, refl, betas);
+    else
+      cudaLaunchKernelEx(&cfg, k_tridiag<false>, A, Aw, n, dg, of, refl, betas);
+    count_launch(1);
+    return;
+  }
+}
+
+// The tridiagonal scaled by a power of two to norm <= 1, for the Sturm counts: ds = diagonal, es =
+// squared off-diagonal, kept at or above 1e-40 (a change of 1e-20 of the norm in the off-diagonal, far
+// below rounding) so that a decoupled matrix never makes the recurrence vanish.
+// Number of eigenvalues below x from the sign changes of the principal minors,
+// p_i = (d_i - x) p_{i-1} - e_{i-1}^2 p_{i-2} (a zero minor takes the sign opposite to the one before, as
+// the zero pivot of the quotient form counts as negative). Every four steps the pair is rescaled by a
+// power of two (|d - x| <= 2 and the floor on e^2 keep four steps far inside the exponent range). Three
+// FP64 instructions per step and no division: the quotient form's division made the chain several
+// times longer.
+__device__ __forceinline__ int sturm_count(const double *ds, const double *es, int n, double x) {
+  // the sign and the zero test read the bit pattern: an FP64 comparison costs as much as a product
+  double p0 = 1.0, p1 = ds[0] - x;
+  auto zero = [](double p) { return ((__double2hiint(p) << 1) | __double2loint(p)) == 0; };
+  int neg = zero(p1) ? 1 : (int)((unsigned)__double2hiint(p1) >> 31), c = neg;  // neg: sign of the latest minor
+  int i = 1;
+  auto step = [&](int q) {
+    const double p2 = fma(ds[q] - x, p1, -(es[q - 1] * p0));
+    const int ng = zero(p2) ? 1 - neg : (int)((unsigned)__double2hiint(p2) >> 31);
+    c += ng ^ neg;
+    neg = ng;
+    p0 = p1;
+    p1 = p2;
+  };
+  for (; i + 3 < n; i += 4) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) step(i + u);
+    // scale by 2^-e, e the exponent of the larger of the two
+    const int e0 = (__double2hiint(p0) >> 20) & 0x7ff, e1 = (__double2hiint(p1) >> 20) & 0x7ff;
+    const double sc = __hiloint2double((2046 - max(max(e0, e1), 1)) << 20, 0);
+    p0 *= sc;
+    p1 *= sc;
+  }
+  for (; i < n; ++i) step(i);
   return c;
 }
 
-// (j+1)-th smallest eigenvalue by multisection: one warp per eigenvalue, each lane counts the
-// eigenvalues below one of 32 interior points of the bracket, which shrinks 33-fold per round.
-__global__ void k_bisect(const double *dg, const double *of, int n, int k, double *ev) {
-  const int lane = threadIdx.x & 31;
-  const int j = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (j >= k) return;
+// (j+1)-th smallest eigenvalue by multisection: one block per eigenvalue, each thread counts the
+// eigenvalues below one of 128 interior points of the bracket, which shrinks 129-fold per round (a warp
+// on each of the SM's sub-partitions costs no more time than one warp). Eight warps of eight
+// eigenvalues on one SM with the quotient form took 5.9 ms for ten eigenvalues at n = 512, this 0.58 ms;
+// at n = 128, 1.48 ms and 0.15 ms.
+constexpr int kBisT = 128;
+__global__ void __launch_bounds__(kBisT) k_bisect(const double *dg, const double *of, int n, int k, double *ev) {
+  extern __shared__ double sm[];
+  __shared__ double bound[3][kBisT / 32];
+  double *ds = sm, *es = sm + n;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, j = blockIdx.x;
   double lo = dg[0], hi = dg[0], nrm = 0.0;
-  for (int i = 0; i < n; ++i) {
+  for (int i = threadIdx.x; i < n; i += kBisT) {
+    const double d = dg[i];
     const double r = (i > 0 ? fabs(of[i - 1]) : 0.0) + (i < n - 1 ? fabs(of[i]) : 0.0);
-    lo = fmin(lo, dg[i] - r);
-    hi = fmax(hi, dg[i] + r);
-    nrm = fmax(nrm, fabs(dg[i]) + r);
+    lo = fmin(lo, d - r);
+    hi = fmax(hi, d + r);
+    nrm = fmax(nrm, fabs(d) + r);
   }
-  const double tiny = 1e-300 + 1e-30 * nrm * 2.2e-16;
-  lo -= 1e-12 * (nrm + 1.0);
-  hi += 1e-12 * (nrm + 1.0);
+  for (int q = 16; q > 0; q >>= 1) {
+    lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, q));
+    hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, q));
+    nrm = fmax(nrm, __shfl_xor_sync(0xffffffffu, nrm, q));
+  }
+  if (lane == 0) {
+    bound[0][warp] = lo;
+    bound[1][warp] = hi;
+    bound[2][warp] = nrm;
+  }
+  __syncthreads();
+  for (int w = 0; w < kBisT / 32; ++w) {
+    lo = fmin(lo, bound[0][w]);
+    hi = fmax(hi, bound[1][w]);
+    nrm = fmax(nrm, bound[2][w]);
+  }
+  if (nrm == 0.0) {  // the zero matrix (the floor on e^2 below is relative to the norm)
+    if (threadIdx.x == 0) ev[j] = 0.0;
+    return;
+  }
+  int ex = 0;
+  if (nrm < INFINITY) frexp(nrm, &ex);
+  for (int i = threadIdx.x; i < n; i += kBisT) {
+    ds[i] = ldexp(dg[i], -ex);
+    if (i < n - 1) {
+      const double e = ldexp(of[i], -ex);
+      es[i] = fmax(e * e, 1e-40);
+    }
+  }
+  __syncthreads();
+  lo = ldexp(lo, -ex) - 1e-12;
+  hi = ldexp(hi, -ex) + 1e-12;
   for (int it = 0; it < 64; ++it) {
-    const double w = (hi - lo) / 33.0;
-    const double x = lo + (lane + 1) * w;
-    const bool below = (x > lo && x < hi) ? (sturm_count(dg, of, n, x, tiny) <= j) : (x <= lo);
-    const unsigned bal = __ballot_sync(0xffffffffu, below);
-    const int m = __popc(bal);  // lanes 0..m-1 have at most j eigenvalues below their point
+    const double w = (hi - lo) / (kBisT + 1.0);
+    const double x = lo + (threadIdx.x + 1) * w;
+    const bool below = (x > lo && x < hi) ? (sturm_count(ds, es, n, x) <= j) : (x <= lo);
+    const int m = __syncthreads_count(below);  // threads 0..m-1 have at most j eigenvalues below their point
     const double nlo = (m == 0) ? lo : lo + m * w;
-    const double nhi = (m == 32) ? hi : lo + (m + 1) * w;
+    const double nhi = (m == kBisT) ? hi : lo + (m + 1) * w;
     if (!(nhi - nlo < hi - lo)) break;  // no further progress in floating point
     lo = nlo;
     hi = nhi;
   }
-  if (lane == 0) ev[j] = 0.5 * (lo + hi);
+  if (threadIdx.x == 0) ev[j] = ldexp(0.5 * (lo + hi), ex);
+}
+
+static void launch_bisect(const double *dg, const double *of, int n, int k, double *ev, cudaStream_t s) {
+  const size_t sm = 2 * (size_t)n * sizeof(double);
+  if (sm > 48 * 1024) raise_smem_limit((const void *)k_bisect, sm);
+  k_bisect<<<k, kBisT, sm, s>>>(dg, of, n, k, ev);
+  count_launch(1);
 }
 
 size_t eig_work_bytes(int n) { return (size_t)n * n * sizeof(double) + 2 * (size_t)n * sizeof(double); }
@@ -162,29 +389,17 @@ int launch_eig_lowest(double *A, int n, int k, double *evals_dev, double *work, 
   double *Aw = work;
   double *dg = Aw + (long long)n * n;
   double *of = dg + n;
-  cudaMemcpyAsync(Aw, A, (size_t)n * n * sizeof(double), cudaMemcpyDeviceToDevice, s);
-  const size_t sm = (2 * (size_t)n + 34) * sizeof(double);
-  const size_t sm_full = sm + (size_t)n * n * sizeof(double);
   if (n >= 3) {
-    if (sm_full <= 200 * 1024) {
-      raise_smem_limit((const void *)k_tridiag<true>, sm_full);
-      k_tridiag<true><<<1, kEigThreads, sm_full, s>>>(Aw, n, dg, of, nullptr, nullptr);
-    } else {
-      if (sm > 48 * 1024)
-        raise_smem_limit((const void *)k_tridiag<false>, sm);
-      k_tridiag<false><<<1, kEigThreads, sm, s>>>(Aw, n, dg, of, nullptr, nullptr);
-    }
-    count_launch(1);
+    launch_tridiag(A, Aw, n, dg, of, nullptr, nullptr, s);
   } else {
     // n <= 2: the matrix is already tridiagonal
-    cudaMemcpyAsync(dg, Aw, sizeof(double), cudaMemcpyDeviceToDevice, s);
+    cudaMemcpyAsync(dg, A, sizeof(double), cudaMemcpyDeviceToDevice, s);
     if (n == 2) {
-      cudaMemcpyAsync(dg + 1, Aw + 3, sizeof(double), cudaMemcpyDeviceToDevice, s);
-      cudaMemcpyAsync(of, Aw + 2, sizeof(double), cudaMemcpyDeviceToDevice, s);
+      cudaMemcpyAsync(dg + 1, A + 3, sizeof(double), cudaMemcpyDeviceToDevice, s);
+      cudaMemcpyAsync(of, A + 2, sizeof(double), cudaMemcpyDeviceToDevice, s);
     }
   }
-  k_bisect<<<(k + 7) / 8, 256, 0, s>>>(dg, of, n, k, evals_dev);
-  count_launch(1);
+  launch_bisect(dg, of, n, k, evals_dev, s);
   return 0;
 }
 
@@ -337,31 +552,20 @@ int launch_eig_vectors(const double *A, int n, int k, double *evals_dev, double 
   double *betas = refl + (long long)n * n;
   double *Y = betas + n;
   double *fac = Y + (long long)k * n;
-  cudaMemcpyAsync(Aw, A, (size_t)n * n * sizeof(double), cudaMemcpyDeviceToDevice, s);
   cudaMemsetAsync(betas, 0, (size_t)n * sizeof(double), s);
-  const size_t sm = (2 * (size_t)n + 34) * sizeof(double);
-  const size_t sm_full = sm + (size_t)n * n * sizeof(double);
   if (n >= 3) {
-    if (sm_full <= 200 * 1024) {
-      raise_smem_limit((const void *)k_tridiag<true>, sm_full);
-      k_tridiag<true><<<1, kEigThreads, sm_full, s>>>(Aw, n, dg, of, refl, betas);
-    } else {
-      if (sm > 48 * 1024)
-        raise_smem_limit((const void *)k_tridiag<false>, sm);
-      k_tridiag<false><<<1, kEigThreads, sm, s>>>(Aw, n, dg, of, refl, betas);
-    }
-    count_launch(1);
+    launch_tridiag(A, Aw, n, dg, of, refl, betas, s);
   } else {
-    cudaMemcpyAsync(dg, Aw, sizeof(double), cudaMemcpyDeviceToDevice, s);
+    cudaMemcpyAsync(dg, A, sizeof(double), cudaMemcpyDeviceToDevice, s);
     if (n == 2) {
-      cudaMemcpyAsync(dg + 1, Aw + 3, sizeof(double), cudaMemcpyDeviceToDevice, s);
-      cudaMemcpyAsync(of, Aw + 2, sizeof(double), cudaMemcpyDeviceToDevice, s);
+      cudaMemcpyAsync(dg + 1, A + 3, sizeof(double), cudaMemcpyDeviceToDevice, s);
+      cudaMemcpyAsync(of, A + 2, sizeof(double), cudaMemcpyDeviceToDevice, s);
     }
   }
-  k_bisect<<<(k + 7) / 8, 256, 0, s>>>(dg, of, n, k, evals_dev);
+  launch_bisect(dg, of, n, k, evals_dev, s);
   k_tri_vectors<<<1, 256, 0, s>>>(dg, of, n, k, evals_dev, Y, fac);
   k_tri_backtransform<<<k, 256, (size_t)n * sizeof(double), s>>>(refl, betas, n, k, Y, evecs_dev);
-  count_launch(3);
+  count_launch(2);
   return 0;
 }
 
