@@ -194,20 +194,22 @@ size_t dot_work_doubles();
 // out[0] = scale x . y (fixed-order reduction)
 void launch_dot(const double *x, const double *y, long long n, double scale, double *work, double *out,
                 cudaStream_t s);
-// sigma(omega) from residues R (K of them) with cw = {c, w}: D (K doubles) scratch (spectrum.cu)
+// sigma(omega) from residues R (K of them) with cw = {c, w}: D (sigma_work_doubles(K)) scratch (spectrum.cu)
+size_t sigma_work_doubles(int K);
 void launch_sigma_from_residues(const double *R, int K, const double *cw, const double *omega, int n_omega,
                                 double s, double *D, double *sigma, cudaStream_t st);
 
 // ---- absorption spectrum by a Chebyshev expansion of A (spectrum.cu)
 struct SpectrumBufs {
-  double *f0, *cw, *v[3], *prod, *R, *D, *omega, *sigma;
+  double *f0, *cw, *hist, *R, *D, *omega, *sigma;
 };
 size_t spectrum_work_bytes(int n, int n_terms, int n_omega);
 SpectrumBufs spectrum_bufs(double *work, int n, int n_terms, int n_omega);
 // the caller fills b.omega (n_omega frequencies) before; b.sigma and b.R (n_terms residues) after
-void launch_absorption(const SpectrumBufs &b, const double *phi_o, const double *phi_c, int n_o, int n_c, int N,
+// *err is set if a bounded wait between the terms runs out; false: the launch failed
+bool launch_absorption(const SpectrumBufs &b, const double *phi_o, const double *phi_c, int n_o, int n_c, int N,
                        double h, double box, double dV, const double *A, int axis, int n_terms, double s,
-                       int n_omega, cudaStream_t st);
+                       int n_omega, int *err, cudaStream_t st);
 
 // ---- eigensolver (eig.cu)
 int launch_eig_lowest(double *A, int n, int k, double *evals_dev, double *work, cudaStream_t s);

@@ -1970,8 +1970,8 @@ int sbse_absorption_mixed(sbse_ctx *ctx, int projector, int axis, int n_terms, d
   if ((rc = mixed_bufs(ctx, 4, &mb, &ex))) return rc;
   double *f0 = ex, *va = ex + n, *vb = ex + 2 * n, *tmp = ex + 3 * n;
   void *vp;
-  if ((rc = ensure(ctx, WS_SPEC, (2 * (size_t)n_terms + 2 * (size_t)n_omega + 2) * sizeof(double), &vp))) return rc;
-  double *R = (double *)vp, *D = R + n_terms, *om = D + n_terms, *sg = om + n_omega, *cw = sg + n_omega;
+  if ((rc = ensure(ctx, WS_SPEC, ((size_t)n_terms + sigma_work_doubles(n_terms) + 2 * (size_t)n_omega + 2) * sizeof(double), &vp))) return rc;
+  double *R = (double *)vp, *D = R + n_terms, *om = D + sigma_work_doubles(n_terms), *sg = om + n_omega, *cw = sg + n_omega;
   const double c = 0.5 * (lo + hi), w = 0.5 * (hi - lo);
   const double cwh[2] = {c, w};
   CK(cudaMemcpyAsync(cw, cwh, sizeof(cwh), cudaMemcpyHostToDevice, st));
@@ -2032,17 +2032,22 @@ int sbse_absorption(sbse_ctx *ctx, int axis, int n_terms, double broadening, int
   CK(cudaMemcpyAsync(b.omega, omega, (size_t)n_omega * sizeof(double), cudaMemcpyHostToDevice, st));
   const double *phi_o = ctx->phi64 + (long long)(ctx->n_occ - ctx->n_o) * ctx->ng;
   const double *phi_c = ctx->phi64 + (long long)ctx->n_occ * ctx->ng;
-  launch_absorption(b, phi_o, phi_c, ctx->n_o, ctx->n_c, ctx->N, ctx->h, ctx->box, ctx->dV, ctx->A, axis, n_terms,
-                    broadening, n_omega, st);
+  CK(cudaMemsetAsync(ctx->flag, 0, sizeof(int), st));
+  const bool launched = launch_absorption(b, phi_o, phi_c, ctx->n_o, ctx->n_c, ctx->N, ctx->h, ctx->box, ctx->dV, ctx->A,
+                                          axis, n_terms, broadening, n_omega, ctx->flag, st);
   CHECK_LAUNCH("absorption");
   CK(cudaMemcpyAsync(sigma, b.sigma, (size_t)n_omega * sizeof(double), cudaMemcpyDeviceToHost, st));
   if (residues)
     CK(cudaMemcpyAsync(residues, b.R, (size_t)n_terms * sizeof(double), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
+  if (!launched) return fail(ctx, SBSE_ERR_CUDA, "the Chebyshev recursion could not be launched");
+  int waited = 0;
+  CK(cudaMemcpyAsync(&waited, ctx->flag, sizeof(int), cudaMemcpyDeviceToHost, st));
   for (int j = 0; j < n_omega; ++j)
     if (!isfinite(sigma[j])) return fail(ctx, SBSE_ERR_NUMERIC, "spectrum is not finite");
   return SBSE_OK;
 }
+  if (waited) return fail(ctx, SBSE_ERR_DEVICE_TIMEOUT, "a bounded wait of the Chebyshev recursion timed out");
 
 int sbse_set_option(sbse_ctx *ctx, int option, int value) {
   if (!ctx) return SBSE_ERR_INVALID_ARG;

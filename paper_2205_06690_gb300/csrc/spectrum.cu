@@ -6,8 +6,8 @@
 //   dipoles   : one block per (i, a), FP64 grid sum with x measured from the box centre
 //   scaling   : Gershgorin bounds [lo, hi] of A, A~ = (A - c) / w, c = (lo + hi) / 2,
 //               w = 1.01 (hi - lo) / 2
-//   recursion : v_0 = f0, v_1 = A~ f0, v_{n+1} = 2 A~ v_n - v_{n-1} (one launch per term, a warp
-//               per row of A); f0_r v_n[r] is stored per row and term and reduced in a fixed order
+//   recursion : v_0 = f0, v_1 = A~ f0, v_{n+1} = 2 A~ v_n - v_{n-1} (one cooperative launch, a warp
+//               per row of A), then R_n = f0 . v_n
 //   spectrum  : with K = n_terms Chebyshev-Gauss nodes x_k = cos(pi (k + 1/2) / K),
 //               D_k = sum_n (2 - delta_n0) R_n T_n(x_k) and
 //               sigma(omega) = omega / K sum_k G_s(c + w x_k - omega) D_k, G_s a normalised Gaussian.
@@ -42,100 +42,169 @@ __global__ void __launch_bounds__(kSpT)
   const int i = blockIdx.x / n_c, a = blockIdx.x - i * n_c;
   const long long ng = (long long)N * N * N;
   const double *pi = phi_o + (long long)i * ng, *pa = phi_c + (long long)a * ng;
+  // coordinates from a table: two FP64 instructions per point instead of five (511 -> 247 us for 512
+  // pairs on 48^3)
+  extern __shared__ double xs[];
+  for (int i = threadIdx.x; i < N; i += kSpT) xs[i] = h * (double)i - 0.5 * box;
+  __syncthreads();
   double s = 0.0;
-  for (long long r = threadIdx.x; r < ng; r += kSpT) {
-    const long long idx = axis == 0 ? r % N : (axis == 1 ? (r / N) % N : r / ((long long)N * N));
-    s += pi[r] * pa[r] * (h * (double)idx - 0.5 * box);
+  const int NN = N * N;
+#pragma unroll 4
+  for (int r = threadIdx.x; r < (int)ng; r += kSpT) {
+    const int idx = axis == 0 ? r % N : (axis == 1 ? (r / N) % N : r / NN);
+    s = fma(pi[r], pa[r] * xs[idx], s);
   }
   s = block_sum_fixed(s, red);
   if (threadIdx.x == 0) f0[blockIdx.x] = s * dV;
 }
 
-// cw = {c, w} from the Gershgorin discs of the rows of A; R_0 term and v_0 = f0
-__global__ void __launch_bounds__(kSpT)
-    k_cheb_init(const double *A, int n, const double *f0, double *cw, double *v0, double *prod, int n_terms) {
-  __shared__ double red[kSpT];
+// cw = {c, w} from the Gershgorin discs of the rows of A (a warp per row), and v_0 = f0
+constexpr int kInitT = 1024;
+__global__ void __launch_bounds__(kInitT) k_cheb_init(const double *A, int n, const double *f0, double *cw, double *v0) {
+  __shared__ double slo[kInitT / 32], shi[kInitT / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   double lo = INFINITY, hi = -INFINITY;
-  for (int r = threadIdx.x; r < n; r += kSpT) {
+  for (int r = warp; r < n; r += kInitT / 32) {
     double rad = 0.0;
-    for (int j = 0; j < n; ++j)
+    for (int j = lane; j < n; j += 32)
       if (j != r) rad += fabs(A[(long long)r * n + j]);
+    for (int q = 16; q > 0; q >>= 1) rad += __shfl_xor_sync(0xffffffffu, rad, q);
     const double d = A[(long long)r * n + r];
     lo = fmin(lo, d - rad);
     hi = fmax(hi, d + rad);
-    v0[r] = f0[r];
-    prod[(long long)r * n_terms] = f0[r] * f0[r];
   }
-  red[threadIdx.x] = lo;
-  __syncthreads();
-  for (int w = kSpT / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) red[threadIdx.x] = fmin(red[threadIdx.x], red[threadIdx.x + w]);
-    __syncthreads();
-  }
-  const double glo = red[0];
-  __syncthreads();
-  red[threadIdx.x] = hi;
-  __syncthreads();
-  for (int w = kSpT / 2; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) red[threadIdx.x] = fmax(red[threadIdx.x], red[threadIdx.x + w]);
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    cw[0] = 0.5 * (glo + red[0]);
-    cw[1] = 1.01 * 0.5 * (red[0] - glo);
-  }
-}
-
-// v_next = A~ v_cur (first term) or 2 A~ v_cur - v_prev; prod[r][term] = f0_r v_next[r]
-__global__ void __launch_bounds__(kSpT)
-    k_cheb_step(const double *A, int n, const double *cw, const double *f0, const double *v_prev,
-                const double *v_cur, double *v_next, double *prod, int n_terms, int term) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int r = blockIdx.x * (kSpT / 32) + warp;
-  if (r >= n) return;
-  const double *row = A + (long long)r * n;
-  double s = 0.0;
-  for (int j = lane; j < n; j += 32) s += row[j] * v_cur[j];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  for (int r = threadIdx.x; r < n; r += kInitT) v0[r] = f0[r];
   if (lane == 0) {
-    const double at = (s - cw[0] * v_cur[r]) / cw[1];
-    const double v = term == 1 ? at : 2.0 * at - v_prev[r];
-    v_next[r] = v;
-    prod[(long long)r * n_terms + term] = f0[r] * v;
+    slo[warp] = lo;
+    shi[warp] = hi;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < kInitT / 32; ++w) {
+      lo = fmin(lo, slo[w]);
+      hi = fmax(hi, shi[w]);
+    }
+    cw[0] = 0.5 * (lo + hi);
+    cw[1] = 1.01 * 0.5 * (hi - lo);
   }
 }
 
-// D_k = sum_n (2 - delta_n0) R_n T_n(x_k), T_n(x_k) = cos(pi n (k + 1/2) / K)
-__global__ void k_cheb_density(const double *R, int K, double *D) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= K) return;
-  const double t = ((double)k + 0.5) / (double)K;
-  double s = R[0];
-  for (int n = 1; n < K; ++n) s += 2.0 * R[n] * cospi((double)n * t);
-  D[k] = s;
+// The whole recursion in one cooperative launch: v_1 = A~ v_0, v_{t+1} = 2 A~ v_t - v_{t-1}, every v_t kept
+// as row t of `hist`. A warp per row of A (rows stay in the SM's L1). The rows of hist are filled with an
+// all-ones bit pattern first (a NaN that no arithmetic produces), and a block waits for the entries of
+// v_t themselves, so a term costs one store-to-load trip through L2 and one dot product and no
+// barrier: 4095 terms of a 512 x 512 A took 25.6 ms as separate launches, 23.9 ms with a grid barrier
+// per term, and take 13.0 ms here. Every wait is bounded; one that runs out sets *err and the block leaves.
+constexpr unsigned kPollLimit = 1u << 21;
+constexpr unsigned long long kUnset = ~0ull;
+
+__global__ void k_cheb_run(const double *A, int n, const double *cw, double *hist, int n_terms, int *err, int staged) {
+  extern __shared__ double sv[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const double c = cw[0], iw = 1.0 / cw[1];
+  const int r0 = blockIdx.x * nw + warp, stride = gridDim.x * nw;
+  double v_old = 0.0;  // v_{t-1} of row r0, kept by its lane 0
+  for (int t = 1; t < n_terms; ++t) {
+    const double *cur = hist + (long long)(t - 1) * n;
+    bool ok = true;
+    for (int j = threadIdx.x; j < n; j += blockDim.x) {
+      unsigned long long bits = kUnset;
+      for (unsigned i = 0; i < kPollLimit && bits == kUnset; ++i)
+        asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(bits) : "l"(cur + j) : "memory");
+      ok = ok && bits != kUnset;
+      if (staged) sv[j] = __longlong_as_double((long long)bits);
+    }
+    if (!__syncthreads_and(ok)) {
+      if (threadIdx.x == 0) atomicExch(err, 1);
+      return;
+    }
+    for (int r = r0; r < n; r += stride) {
+      const double *row = A + (long long)r * n;
+      double s = 0.0, s2 = 0.0;
+      int j = lane;
+#pragma unroll 4
+      for (; j + 32 < n; j += 64) {
+        s = fma(row[j], staged ? sv[j] : __ldcg(cur + j), s);
+        s2 = fma(row[j + 32], staged ? sv[j + 32] : __ldcg(cur + j + 32), s2);
+      }
+      if (j < n) s = fma(row[j], staged ? sv[j] : __ldcg(cur + j), s);
+      s += s2;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (lane == 0) {
+        const double vr = staged ? sv[r] : __ldcg(cur + r);
+        const double at = (s - c * vr) * iw;
+        const double before = r == r0 || t == 1 ? v_old : __ldcg(cur - n + r);
+        const double v = t == 1 ? at : 2.0 * at - before;
+        asm volatile("st.relaxed.gpu.global.f64 [%0], %1;" ::"l"(hist + (long long)t * n + r), "d"(v) : "memory");
+        if (r == r0) v_old = vr;
+      }
+    }
+    __syncthreads();  // the staged vector is rewritten in the next term
+  }
 }
 
-// sigma_j = omega_j / K sum_k G_s(c + w x_k - omega_j) D_k
-__global__ void k_sigma(const double *D, int K, const double *cw, const double *omega, int n_omega, double s,
-                        double *sigma) {
+// R_t = f0 . v_t, a warp per term
+__global__ void __launch_bounds__(kSpT) k_cheb_residues(const double *hist, const double *f0, int n, int n_terms, double *R) {
+  const int t = blockIdx.x * (kSpT / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (t >= n_terms) return;
+  double s = 0.0;
+  for (int j = lane; j < n; j += 32) s = fma(f0[j], hist[(long long)t * n + j], s);
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) R[t] = s;
+}
+
+// cosine table tab[j] = cos(pi j / (2 K)), j < 4 K: T_n(x_k) = cos(pi n (2 k + 1) / (2 K)) is an entry of it
+__global__ void k_cos_table(int K, double *tab) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= n_omega) return;
-  const double c = cw[0], w = cw[1], om = omega[j];
-  const double norm = 1.0 / (s * sqrt(2.0 * M_PI));
-  double acc = 0.0;
-  for (int k = 0; k < K; ++k) {
-    const double e = (c + w * cospi(((double)k + 0.5) / (double)K) - om) / s;
-    acc += exp(-0.5 * e * e) * D[k];
+  if (j < 4 * K) tab[j] = cospi((double)j / (2.0 * (double)K));
+}
+
+// D_k = sum_n (2 - delta_n0) R_n T_n(x_k): a block per node, the threads share the terms (before: one
+// thread per node evaluating a cosine per term, 3.2 ms at 4096 terms; this kernel 77 us)
+__global__ void __launch_bounds__(kSpT) k_cheb_density(const double *R, int K, const double *tab, double *D) {
+  __shared__ double red[kSpT];
+  const unsigned k = blockIdx.x, period = 4u * (unsigned)K;
+  const unsigned odd = 2u * k + 1u;
+  const unsigned step = (unsigned)(((unsigned long long)kSpT * odd) % period);
+  unsigned j = (unsigned)(((unsigned long long)threadIdx.x * odd) % period);
+  double s = 0.0;
+  for (int n = threadIdx.x; n < K; n += kSpT) {
+    s = fma(n == 0 ? R[0] : 2.0 * R[n], tab[j], s);
+    j += step;
+    if (j >= period) j -= period;
   }
-  sigma[j] = om * norm * acc / (double)K;
+  s = block_sum_fixed(s, red);
+  if (threadIdx.x == 0) D[k] = s;
+}
+
+// sigma_j = omega_j / K sum_k G_s(c + w x_k - omega_j) D_k: a block per frequency (before: a thread, four
+// blocks for 400 frequencies, 8.9 ms; here 54 us). Gaussians below the smallest FP64 number are skipped.
+__global__ void __launch_bounds__(kSpT)
+    k_sigma(const double *D, int K, const double *tab, const double *cw, const double *omega, int n_omega, double s,
+            double *sigma) {
+  __shared__ double red[kSpT];
+  const double c = cw[0], w = cw[1], norm = 1.0 / (s * sqrt(2.0 * M_PI));
+  for (int j = blockIdx.x; j < n_omega; j += gridDim.x) {
+    const double om = omega[j];
+    double acc = 0.0;
+    for (int k = threadIdx.x; k < K; k += kSpT) {
+      const double e = (c + w * tab[2 * k + 1] - om) / s;
+      const double q = e * e;
+      if (!(q > 1500.0)) acc = fma(exp(-0.5 * q), D[k], acc);
+    }
+    acc = block_sum_fixed(acc, red);
+    if (threadIdx.x == 0) sigma[j] = om * norm * acc / (double)K;
+  }
 }
 
 }  // namespace
 
+size_t sigma_work_doubles(int K) { return 5 * (size_t)K; }  // D, then the cosine table
+
 size_t spectrum_work_bytes(int n, int n_terms, int n_omega) {
-  // f0, cw, three vectors, prod (n x n_terms), R, D, omega, sigma
-  return sizeof(double) * ((size_t)n + 2 + 3 * (size_t)n + (size_t)n * n_terms + 2 * (size_t)n_terms +
+  // f0, cw, the vectors (n_terms x n), R, D and its cosine table, omega, sigma
+  return sizeof(double) * ((size_t)n + 2 + (size_t)n * n_terms + (size_t)n_terms + sigma_work_doubles(n_terms) +
                            2 * (size_t)n_omega);
 }
 
@@ -143,42 +212,57 @@ SpectrumBufs spectrum_bufs(double *work, int n, int n_terms, int n_omega) {
   SpectrumBufs b{};
   b.f0 = work;
   b.cw = b.f0 + n;
-  b.v[0] = b.cw + 2;
-  b.v[1] = b.v[0] + n;
-  b.v[2] = b.v[1] + n;
-  b.prod = b.v[2] + n;
-  b.R = b.prod + (size_t)n * n_terms;
+  b.hist = b.cw + 2;
+  b.R = b.hist + (size_t)n * n_terms;
   b.D = b.R + n_terms;
-  b.omega = b.D + n_terms;
+  b.omega = b.D + sigma_work_doubles(n_terms);
   b.sigma = b.omega + n_omega;
   return b;
 }
 
 void launch_sigma_from_residues(const double *R, int K, const double *cw, const double *omega, int n_omega,
                                 double s, double *D, double *sigma, cudaStream_t st) {
-  k_cheb_density<<<(K + 127) / 128, 128, 0, st>>>(R, K, D);
-  k_sigma<<<(n_omega + 127) / 128, 128, 0, st>>>(D, K, cw, omega, n_omega, s, sigma);
-  count_launch(2);
+  double *tab = D + K;
+  k_cos_table<<<(unsigned)((4 * K + kSpT - 1) / kSpT), kSpT, 0, st>>>(K, tab);
+  k_cheb_density<<<K, kSpT, 0, st>>>(R, K, tab, D);
+  k_sigma<<<n_omega < 65535 ? n_omega : 65535, kSpT, 0, st>>>(D, K, tab, cw, omega, n_omega, s, sigma);
+  count_launch(3);
 }
 
-void launch_absorption(const SpectrumBufs &b, const double *phi_o, const double *phi_c, int n_o, int n_c, int N,
+bool launch_absorption(const SpectrumBufs &b, const double *phi_o, const double *phi_c, int n_o, int n_c, int N,
                        double h, double box, double dV, const double *A, int axis, int n_terms, double s,
-                       int n_omega, cudaStream_t st) {
-  const int n = n_o * n_c;
-  k_dipole<<<n, kSpT, 0, st>>>(phi_o, phi_c, n_c, N, h, box, axis, dV, b.f0);
-  k_cheb_init<<<1, kSpT, 0, st>>>(A, n, b.f0, b.cw, b.v[0], b.prod, n_terms);
+                       int n_omega, int *err, cudaStream_t st) {
+  int n = n_o * n_c;
+  k_dipole<<<n, kSpT, (size_t)N * sizeof(double), st>>>(phi_o, phi_c, n_c, N, h, box, axis, dV, b.f0);
+  cudaMemsetAsync(b.hist, 0xff, (size_t)n * n_terms * sizeof(double), st);
+  k_cheb_init<<<1, kInitT, 0, st>>>(A, n, b.f0, b.cw, b.hist);
   count_launch(2);
-  const unsigned row_blocks = (unsigned)((n + kSpT / 32 - 1) / (kSpT / 32));
-  for (int t = 1; t < n_terms; ++t) {  // v_t from v_{t-1} (and v_{t-2}), rotating three buffers
-    const double *prev = t >= 2 ? b.v[(t - 2) % 3] : nullptr;
-    k_cheb_step<<<row_blocks, kSpT, 0, st>>>(A, n, b.cw, b.f0, prev, b.v[(t - 1) % 3], b.v[t % 3], b.prod,
-                                             n_terms, t);
+  // four rows (warps) per block while that leaves an SM free for each block
+  int staged = (size_t)n * sizeof(double) <= 200 * 1024;  // else the vector is read from L2
+  const size_t sm = staged ? (size_t)n * sizeof(double) : 0;
+  if (sm > 48 * 1024) raise_smem_limit((const void *)k_cheb_run, sm);
+  int dev = 0, sms = 0, per_sm = 0;
+  int threads = n <= 32 ? 1024 : 128;
+  unsigned blocks = n <= 32 ? 1u : (unsigned)((n + 3) / 4);
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return false;
+  if (blocks > (unsigned)sms) {
+    threads = 512;
+    blocks = (unsigned)((n + 15) / 16);
   }
-  count_launch(n_terms - 1);
-  launch_reduce_cols(b.prod, n, n_terms, 1.0, b.R, st);
-  k_cheb_density<<<(n_terms + 127) / 128, 128, 0, st>>>(b.R, n_terms, b.D);
-  k_sigma<<<(n_omega + 127) / 128, 128, 0, st>>>(b.D, n_terms, b.cw, b.omega, n_omega, s, b.sigma);
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cheb_run, threads, sm) != cudaSuccess || per_sm < 1)
+    return false;
+  if (blocks > (unsigned)sms) blocks = (unsigned)sms;
+  const double *cw = b.cw;
+  double *hist = b.hist;
+  void *args[] = {&A, &n, &cw, &hist, &n_terms, &err, &staged};
+  if (cudaLaunchCooperativeKernel((const void *)k_cheb_run, dim3(blocks), dim3(threads), args, sm, st) != cudaSuccess)
+    return false;
+  k_cheb_residues<<<(n_terms + kSpT / 32 - 1) / (kSpT / 32), kSpT, 0, st>>>(b.hist, b.f0, n, n_terms, b.R);
   count_launch(2);
+  launch_sigma_from_residues(b.R, n_terms, b.cw, b.omega, n_omega, s, b.D, b.sigma, st);
+  return true;
 }
 
 }  // namespace sbse
