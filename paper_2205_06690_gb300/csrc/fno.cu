@@ -12,9 +12,9 @@
 #include <stdint.h>
 
 #include <string>
+#include <utility>
 #include <vector>
 
-#include "gemm_nt.cuh"
 #include "kernels.h"
 #include "sbse.h"
 
@@ -47,10 +47,14 @@ __device__ __forceinline__ float gelu_grad_f(float x) {
   return 0.5f * (1.f + erff(x * 0.70710678118654752f)) + x * expf(-0.5f * x * x) * 0.39894228040143268f;
 }
 
+}  // namespace
+#include "fno_kernels.cuh"
+namespace {
+
 // FFT index kept at position j of a full axis: 0..m-1, N-m..N-1
 __device__ __forceinline__ int kept(int j, int m, int N) { return j < m ? j : N - 2 * m + j; }
 
-// ---- truncated transforms ----------------------------------------------------------------------
+// ---- truncated transforms by direct sums, for planes that do not fit in shared memory ---------------
 
 // forward along x, real -> complex: out[row][kx] = sum_x in[row][x] e^{-2 pi i kx x / N}, kx < m
 __global__ void k_dft_x(const float *in, float2 *out, long long rows, int N, int m, const float2 *tw) {
@@ -112,52 +116,6 @@ __global__ void k_idft_x(const float2 *in, float *out, long long rows, int N, in
   out[t] = scale * s;
 }
 
-// G[b][co][mode] = sum_ci F[b][ci][mode] R[mode][ci][co]       (transpose = 0)
-// dF[b][ci][mode] = sum_co conj(R[mode][ci][co]) dG[b][co][mode] (transpose = 1)
-// with an optional per-kx factor on the input modes (kxscale[mode % m], null = 1)
-__global__ void k_fno_mix(const float2 *in, const __nv_bfloat162 *R, float2 *out, int B, int C, int modes,
-                          int m, int transpose, const float *kxscale) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (long long)B * C * modes) return;
-  const int mode = (int)(t % modes);
-  const long long r = t / modes;
-  const int c = (int)(r % C);
-  const int b = (int)(r / C);
-  const float ks = kxscale ? kxscale[mode % m] : 1.f;
-  float re = 0.f, im = 0.f;
-  for (int k = 0; k < C; ++k) {
-    const float2 x = in[((long long)b * C + k) * modes + mode];
-    const float2 w = transpose ? __bfloat1622float2(R[((long long)mode * C + c) * C + k])
-                               : __bfloat1622float2(R[((long long)mode * C + k) * C + c]);
-    if (transpose) {  // conj(w) x
-      re += w.x * x.x + w.y * x.y;
-      im += w.x * x.y - w.y * x.x;
-    } else {
-      re += x.x * w.x - x.y * w.y;
-      im += x.x * w.y + x.y * w.x;
-    }
-  }
-  out[t] = make_float2(ks * re, ks * im);
-}
-
-// dR[mode][ci][co] = sum_b conj(F[b][ci][mode]) dG[b][co][mode]  (written as float2 pairs)
-__global__ void k_fno_dR(const float2 *F, const float2 *dG, float2 *dR, int B, int C, int modes) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (long long)modes * C * C) return;
-  const int co = (int)(t % C);
-  const long long r = t / C;
-  const int ci = (int)(r % C);
-  const int mode = (int)(r / C);
-  float re = 0.f, im = 0.f;
-  for (int b = 0; b < B; ++b) {
-    const float2 f = F[((long long)b * C + ci) * modes + mode];
-    const float2 g = dG[((long long)b * C + co) * modes + mode];
-    re += f.x * g.x + f.y * g.y;
-    im += f.x * g.y - f.y * g.x;
-  }
-  dR[t] = make_float2(re, im);
-}
-
 // ---- pointwise parts ---------------------------------------------------------------------------
 
 // V0[b][c][r] = sum_i Wl[c][i] x[b][i][r] + bl[c]
@@ -169,27 +127,6 @@ __global__ void k_fno_lift(const float *x, const float *Wl, const float *bl, flo
   const long long r = t - (long long)b * ng;
   const float x0 = x[((long long)b * 2) * ng + r], x1 = x[((long long)b * 2 + 1) * ng + r];
   for (int c = 0; c < C; ++c) V0[((long long)b * C + c) * ng + r] = Wl[2 * c] * x0 + Wl[2 * c + 1] * x1 + bl[c];
-}
-
-// U[b][co][r] = S[b][co][r] + sum_ci W[co][ci] V[b][ci][r] + bias[co]; Vn = GELU(U) or U
-__global__ void k_fno_pointwise(const float *S, const float *V, const __nv_bfloat16 *W, const float *bias,
-                                float *U, float *Vn, int B, int C, long long ng, int act) {
-  extern __shared__ float ws[];
-  for (int i = threadIdx.x; i < C * C; i += blockDim.x) ws[i] = __bfloat162float(W[i]);
-  __syncthreads();
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (long long)B * ng) return;
-  const int b = (int)(t / ng);
-  const long long r = t - (long long)b * ng;
-  float v[64];
-  for (int ci = 0; ci < C; ++ci) v[ci] = V[((long long)b * C + ci) * ng + r];
-  for (int co = 0; co < C; ++co) {
-    float s = bias[co] + S[((long long)b * C + co) * ng + r];
-    for (int ci = 0; ci < C; ++ci) s += ws[co * C + ci] * v[ci];
-    const long long o = ((long long)b * C + co) * ng + r;
-    U[o] = s;
-    Vn[o] = act ? gelu_f(s) : s;
-  }
 }
 
 // y[b][r] = sum_c w[c] V[b][c][r] + bias
@@ -205,40 +142,11 @@ __global__ void k_fno_project(const float *V, const float *w, const float *bias,
 }
 
 // dV[b][c][r] = w[c] dy[b][r]
-__global__ void k_fno_project_back(const float *dy, const float *w, float *dV, int B, int C, long long ng) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (long long)B * C * ng) return;
-  const long long r = t % ng;
-  const long long bc = t / ng;
-  const int c = (int)(bc % C);
-  const int b = (int)(bc / C);
-  dV[t] = w[c] * dy[(long long)b * ng + r];
-}
-
-// dU = dVn * GELU'(U) (or dVn), in place into dU
-__global__ void k_fno_act_back(const float *dVn, const float *U, float *dU, long long n, int act) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n) return;
-  dU[t] = act ? dVn[t] * gelu_grad_f(U[t]) : dVn[t];
-}
-
-// dV[b][ci][r] = sum_co W[co][ci] dU[b][co][r] + dVspec[b][ci][r]
-__global__ void k_fno_pointwise_back(const float *dU, const __nv_bfloat16 *W, const float *dVspec, float *dV,
-                                     int B, int C, long long ng) {
-  extern __shared__ float ws[];
-  for (int i = threadIdx.x; i < C * C; i += blockDim.x) ws[i] = __bfloat162float(W[i]);
-  __syncthreads();
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (long long)B * ng) return;
-  const int b = (int)(t / ng);
-  const long long r = t - (long long)b * ng;
-  float g[64];
-  for (int co = 0; co < C; ++co) g[co] = dU[((long long)b * C + co) * ng + r];
-  for (int ci = 0; ci < C; ++ci) {
-    float s = dVspec[((long long)b * C + ci) * ng + r];
-    for (int co = 0; co < C; ++co) s += ws[co * C + ci] * g[co];
-    dV[((long long)b * C + ci) * ng + r] = s;
-  }
+__global__ void k_fno_project_back(const float *dy, const float *w, float *dV, int C, long long ng) {
+  const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x, b = blockIdx.y;
+  if (r >= ng) return;
+  const float v = dy[b * ng + r];
+  for (int c = 0; c < C; ++c) dV[(b * C + c) * ng + r] = w[c] * v;
 }
 
 // loss = 0.5 sum (y - t)^2 / count, dy = (y - t) / count; per-block partial losses (FP64)
@@ -276,25 +184,6 @@ __global__ void k_to_bf16(const float *src, __nv_bfloat16 *dst, long long n) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) dst[i] = __float2bfloat16_rn(src[i]);
 }
-
-__global__ void k_d2f(const double *src, float *dst, long long n) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) dst[i] = (float)src[i];
-}
-
-// loaders for the split-K weight-gradient sums over (b, r): K index k = b * ng + r
-struct LoadChan {  // X(row = c, k) = A[b][c][r]
-  const float *A;
-  int C;
-  long long ng;
-  __device__ float operator()(int c, long long k) const {
-    const long long b = k / ng;
-    return A[(b * C + c) * ng + (k - b * ng)];
-  }
-};
-struct LoadOne {
-  __device__ float operator()(int, long long) const { return 1.f; }
-};
 
 inline unsigned nblk(long long n) { return (unsigned)((n + kT - 1) / kT); }
 
@@ -356,16 +245,6 @@ __global__ void k_resample(const float *src, int ns, float *dst, int nd, long lo
   dst[t] = acc;
 }
 
-// a[i] *= s[i % m]: the per-kx factor c_kx / N^3 of the spectral gradient (kx is the fastest mode index)
-__global__ void k_fno_scale_kx(float2 *a, long long n, int m, const float *s) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float f = s[i % m];
-  a[i].x *= f;
-  a[i].y *= f;
-}
-
-
 }  // namespace
 
 // ================================================================================================
@@ -385,13 +264,14 @@ struct sbse_fno {
   std::vector<long long> off_spec, off_w, off_b;
   long long adam_t = 0;
   // tables and activations
-  float2 *tw = nullptr;
+  float2 *tw = nullptr, *fold = nullptr;
   float *kx_herm = nullptr;  // c_kx / N^3
-  float *V = nullptr, *U = nullptr, *S = nullptr, *T1 = nullptr, *dV = nullptr, *dU = nullptr;
+  float *V = nullptr, *U = nullptr, *S = nullptr, *dV = nullptr, *dU = nullptr;
   float2 *F = nullptr, *C1 = nullptr, *C2b = nullptr, *G = nullptr;
   float *y = nullptr, *dy = nullptr;
   double *red = nullptr, *gpart = nullptr, *gout = nullptr;
   size_t gpart_cap = 0;
+  bool folded = false;  // the plane kernels' shared memory fits (else direct sums)
 };
 
 namespace {
@@ -418,62 +298,130 @@ template <typename X> int falloc(sbse_fno *f, X **p, size_t bytes) {
   return SBSE_OK;
 }
 
-// spectral transform of `rows` real rows grouped as [bc][z][y][x] -> F[bc][kz][ky][kx]
+// shared memory of the plane kernels beyond which the direct sums are used (planes of edge 200 and more)
+constexpr size_t kFoSmemMax = 200 * 1024;
+
+// spectral transform of the real fields [bc][z][y][x] -> F[bc][kz][ky][kx]
 void fwd_spectrum(sbse_fno *f, const float *in, float2 *out, long long bc) {
-  const int N = f->N, m = f->m;
+  const int N = f->N, m = f->m, inner = 2 * m * m;
+  if (f->folded) {
+    const long long cols = bc * inner;
+    k_fo_fwd_xy<<<(unsigned)(bc * N), kFoT, fo_fwd_smem(N, m), f->stream>>>(in, f->C2b, N, m, f->fold);
+    dim3 g((unsigned)((cols + kFoT - 1) / kFoT), (unsigned)((m + 1 + kZk - 1) / kZk));
+    k_fo_fwd_z<<<g, kFoT, 0, f->stream>>>(f->C2b, out, cols, inner, N, m, f->fold);
+    count_launch(2);
+    return;
+  }
   const long long rows = bc * N * N;
   k_dft_x<<<nblk(rows * m), kT, 0, f->stream>>>(in, f->C1, rows, N, m, f->tw);  // [bc][z][y][kx]
   // y: [bc*N (z)][N (y)][m] -> [bc*N][2m][m]
   k_dft_mid<<<nblk(bc * N * 2 * m * m), kT, 0, f->stream>>>(f->C1, f->C2b, bc * N, N, 2 * m, m, N, m, 0, -1, f->tw);
   // z: [bc][N (z)][2m*m] -> [bc][2m][2m*m]
-  k_dft_mid<<<nblk(bc * 2 * m * 2 * m * m), kT, 0, f->stream>>>(f->C2b, out, bc, N, 2 * m, 2 * m * m, N, m, 0, -1,
-                                                               f->tw);
+  k_dft_mid<<<nblk(bc * 2 * m * inner), kT, 0, f->stream>>>(f->C2b, out, bc, N, 2 * m, inner, N, m, 0, -1, f->tw);
   count_launch(3);
 }
 
 // inverse of the kept modes: in[bc][kz][ky][kx] -> real out[bc][z][y][x]
 void inv_spectrum(sbse_fno *f, const float2 *in, float *out, long long bc, int hermitian, float scale) {
-  const int N = f->N, m = f->m;
-  k_dft_mid<<<nblk(bc * N * 2 * m * m), kT, 0, f->stream>>>(in, f->C2b, bc, 2 * m, N, 2 * m * m, N, m, 1, +1, f->tw);
+  const int N = f->N, m = f->m, inner = 2 * m * m;
+  if (f->folded) {
+    const long long cols = bc * inner;
+    dim3 g((unsigned)((cols + kFoT - 1) / kFoT), (unsigned)((N / 2 + 1 + kZz - 1) / kZz));
+    k_fo_inv_z<<<g, kFoT, 0, f->stream>>>(in, f->C2b, cols, inner, N, m, f->fold);
+    k_fo_inv_xy<<<(unsigned)(bc * N), kFoT, fo_inv_smem(N, m), f->stream>>>(f->C2b, out, N, m, hermitian, scale,
+                                                                           f->fold);
+    count_launch(2);
+    return;
+  }
+  k_dft_mid<<<nblk(bc * N * inner), kT, 0, f->stream>>>(in, f->C2b, bc, 2 * m, N, inner, N, m, 1, +1, f->tw);
   k_dft_mid<<<nblk(bc * N * N * m), kT, 0, f->stream>>>(f->C2b, f->C1, bc * N, 2 * m, N, m, N, m, 1, +1, f->tw);
   k_idft_x<<<nblk(bc * N * N * N), kT, 0, f->stream>>>(f->C1, out, bc * N * N, N, m, hermitian, scale, f->tw);
   count_launch(3);
+}
+
+// batch entries whose spectra (two tiles of a block) fit in 96 KB of shared memory
+int mix_batch(int B, int C) {
+  const int fit = (int)(96 * 1024 / (2 * mix_tile_bytes(1, C)));
+  return B < fit ? B : (fit < 1 ? 1 : fit);
+}
+
+void mix_forward(sbse_fno *f, const float2 *F, const __nv_bfloat16 *R, float2 *G, int B) {
+  const int C = f->C, Bg = mix_batch(B, C);
+  for (int b0 = 0; b0 < B; b0 += Bg) {
+    const int nb = B - b0 < Bg ? B - b0 : Bg;
+    const long long o = (long long)b0 * C * f->modes;
+    k_fo_mix<<<(unsigned)((f->modes + kMxModes - 1) / kMxModes), kMxT, 2 * mix_tile_bytes(nb, C), f->stream>>>(
+        F + o, R, G + o, nb, C, f->modes, (uintptr_t)R % sizeof(__nv_bfloat162) == 0);
+    count_launch(1);
+  }
+}
+
+// dR and dF (written over the forward spectra F, which no later layer needs) from dG
+void mix_backward(sbse_fno *f, float2 *F, const float2 *dG, const __nv_bfloat16 *R, float *dR, int B) {
+  const int C = f->C, Bg = mix_batch(B, C);
+  for (int b0 = 0; b0 < B; b0 += Bg) {
+    const int nb = B - b0 < Bg ? B - b0 : Bg;
+    const long long o = (long long)b0 * C * f->modes;
+    const size_t sm = 2 * mix_tile_bytes(nb, C) + (size_t)kMxModes * C * (C + 1) * sizeof(__nv_bfloat162);
+    k_fo_mix_back<<<(unsigned)((f->modes + kMxModes - 1) / kMxModes), kMxT, sm, f->stream>>>(
+        F + o, dG + o, R, dR, F + o, nb, C, f->modes, f->m, f->kx_herm, b0 > 0,
+        (uintptr_t)R % sizeof(__nv_bfloat162) == 0, (uintptr_t)dR % sizeof(float2) == 0);
+    count_launch(1);
+  }
+}
+
+template <int CP>
+void pointwise_launch(sbse_fno *f, bool back, const float *S, const float *V, const __nv_bfloat16 *W, const float *bias,
+                      const float *Uprev, float *U, float *out, int B, int act) {
+  dim3 g((unsigned)((f->ng + kPwT * kPw - 1) / (kPwT * kPw)), (unsigned)B);
+  if (back)
+    k_fo_pointwise_back<CP><<<g, kPwT, 0, f->stream>>>(V, W, S, Uprev, out, f->C, f->ng);
+  else
+    k_fo_pointwise<CP><<<g, kPwT, 0, f->stream>>>(S, V, W, bias, U, out, f->C, f->ng, act);
+  count_launch(1);
+}
+
+// the compiled channel count at or above C
+void pointwise(sbse_fno *f, bool back, const float *S, const float *V, const __nv_bfloat16 *W, const float *bias,
+               const float *Uprev, float *U, float *out, int B, int act) {
+  const int C = f->C;
+  if (C <= 8) pointwise_launch<8>(f, back, S, V, W, bias, Uprev, U, out, B, act);
+  else if (C <= 16) pointwise_launch<16>(f, back, S, V, W, bias, Uprev, U, out, B, act);
+  else if (C <= 24) pointwise_launch<24>(f, back, S, V, W, bias, Uprev, U, out, B, act);
+  else if (C <= 32) pointwise_launch<32>(f, back, S, V, W, bias, Uprev, U, out, B, act);
+  else if (C <= 48) pointwise_launch<48>(f, back, S, V, W, bias, Uprev, U, out, B, act);
+  else pointwise_launch<64>(f, back, S, V, W, bias, Uprev, U, out, B, act);
 }
 
 float *Vl(sbse_fno *f, int l, int B) { return f->V + (long long)l * B * f->C * f->ng; }
 float *Ul(sbse_fno *f, int l, int B) { return f->U + (long long)l * B * f->C * f->ng; }
 float2 *Fl(sbse_fno *f, int l, int B) { return f->F + (long long)l * B * f->C * f->modes; }
 
-void forward_impl(sbse_fno *f, int B, const float *x) {
+// keep_u: the pre-activations are stored for a backward pass
+void forward_impl(sbse_fno *f, int B, const float *x, bool keep_u) {
   const int C = f->C;
   const long long ng = f->ng;
   const float *par = f->par;
   k_fno_lift<<<nblk(B * ng), kT, 0, f->stream>>>(x, par + f->off_lw, par + f->off_lb, Vl(f, 0, B), B, C, ng);
   count_launch(1);
-  const __nv_bfloat162 *R16;
   for (int l = 0; l < f->L; ++l) {
     fwd_spectrum(f, Vl(f, l, B), Fl(f, l, B), (long long)B * C);
-    R16 = reinterpret_cast<const __nv_bfloat162 *>(f->par16 + f->off_spec[l]);
-    k_fno_mix<<<nblk((long long)B * C * f->modes), kT, 0, f->stream>>>(Fl(f, l, B), R16, f->G, B, C, f->modes, f->m,
-                                                                       0, nullptr);
-    count_launch(1);
+    mix_forward(f, Fl(f, l, B), f->par16 + f->off_spec[l], f->G, B);
     inv_spectrum(f, f->G, f->S, (long long)B * C, 1, 1.f / (float)(ng));
-    k_fno_pointwise<<<nblk(B * ng), kT, C * C * sizeof(float), f->stream>>>(
-        f->S, Vl(f, l, B), f->par16 + f->off_w[l], par + f->off_b[l], Ul(f, l, B), Vl(f, l + 1, B), B, C, ng,
-        l < f->L - 1 ? 1 : 0);
-    count_launch(1);
+    const bool act = l < f->L - 1;
+    pointwise(f, false, f->S, Vl(f, l, B), f->par16 + f->off_w[l], par + f->off_b[l], nullptr,
+              keep_u && act ? Ul(f, l, B) : nullptr, Vl(f, l + 1, B), B, act ? 1 : 0);
   }
   k_fno_project<<<nblk(B * ng), kT, 0, f->stream>>>(Vl(f, f->L, B), par + f->off_pw, par + f->off_pb, f->y, B,
                                                     C, ng);
   count_launch(1);
 }
 
-// weight gradient: out[M][Nn] = sum_{b,r} A[b][row][r] Bm[b][col][r]  (Bm = null: ones)
-int wgrad(sbse_fno *f, const float *A, int M, const float *Bm, int Nn, int B, float *out) {
-  const long long K = (long long)B * f->ng;
-  const long long kc = gemm_kchunk(K);
-  const long long chunks = (K + kc - 1) / kc;
-  const size_t need = (size_t)chunks * M * Nn * sizeof(double);
+// weight gradient w[M][Nn] = sum_{b,r} A[b][row][r] Bm[b][col][r], and bias[M] = sum_{b,r} A (if not null)
+int wgrad(sbse_fno *f, const float *A, int M, const float *Bm, int Nn, int B, float *w, float *bias) {
+  const long long chunks_b = (f->ng + kWgChunk - 1) / kWgChunk, chunks = chunks_b * B;
+  const int cols = M * (Nn + 1);
+  const size_t need = (size_t)chunks * cols * sizeof(double);
   if (need > f->gpart_cap) {
     if (f->gpart) cudaFree(f->gpart);
     f->gpart = nullptr;
@@ -482,60 +430,38 @@ int wgrad(sbse_fno *f, const float *A, int M, const float *Bm, int Nn, int B, fl
     if (rc) return rc;
     f->gpart_cap = need;
   }
-  dim3 grid((unsigned)chunks, (M + kGemmBM - 1) / kGemmBM, (Nn + kGemmBN - 1) / kGemmBN);
-  if (Bm)
-    k_gemm_nt_part<float><<<grid, kGemmThreads, 0, f->stream>>>(M, Nn, K, kc, LoadChan{A, M, f->ng},
-                                                                LoadChan{Bm, Nn, f->ng}, f->gpart);
-  else
-    k_gemm_nt_part<float><<<grid, kGemmThreads, 0, f->stream>>>(M, Nn, K, kc, LoadChan{A, M, f->ng}, LoadOne{},
-                                                                f->gpart);
+  k_fo_wgrad<<<(unsigned)chunks, kWgT, wg_smem(M, Nn), f->stream>>>(A, M, Bm, Nn, f->ng, chunks_b, f->gpart);
   count_launch(1);
-  launch_reduce_cols(f->gpart, (int)chunks, M * Nn, 1.0, f->gout, f->stream);
-  k_d2f<<<nblk((long long)M * Nn), kT, 0, f->stream>>>(f->gout, out, (long long)M * Nn);
+  launch_reduce_cols(f->gpart, (int)chunks, cols, 1.0, f->gout, f->stream);
+  k_fo_wgrad_out<<<nblk(cols), kT, 0, f->stream>>>(f->gout, M, Nn, w, bias);
   count_launch(1);
   return SBSE_OK;
 }
 
-// backward from dL/dy (in f->dy); fills f->grad (and dL/dx into dx when given)
+// backward from dL/dy (in f->dy); fills f->grad
 int backward_impl(sbse_fno *f, int B, const float *x) {
   const int C = f->C, L = f->L;
-  const long long ng = f->ng, n_act = (long long)B * C * ng;
+  const long long ng = f->ng;
   int rc;
-  // projection
-  if ((rc = wgrad(f, Vl(f, L, B), C, f->dy, 1, B, f->grad + f->off_pw))) return rc;
-  if ((rc = wgrad(f, f->dy, 1, nullptr, 1, B, f->grad + f->off_pb))) return rc;
-  k_fno_project_back<<<nblk(n_act), kT, 0, f->stream>>>(f->dy, f->par + f->off_pw, f->dV, B, C, ng);
+  // projection: its weights' gradient with dy as the one row, the sum of dy is the bias's
+  if ((rc = wgrad(f, f->dy, 1, Vl(f, L, B), C, B, f->grad + f->off_pw, f->grad + f->off_pb))) return rc;
+  // the last layer has no activation: dU = dV
+  k_fno_project_back<<<dim3(nblk(ng), (unsigned)B), kT, 0, f->stream>>>(f->dy, f->par + f->off_pw, f->dU, C, ng);
   count_launch(1);
   for (int l = L - 1; l >= 0; --l) {
-    k_fno_act_back<<<nblk(n_act), kT, 0, f->stream>>>(f->dV, Ul(f, l, B), f->dU, n_act, l < L - 1 ? 1 : 0);
-    count_launch(1);
-    if ((rc = wgrad(f, f->dU, C, Vl(f, l, B), C, B, f->grad + f->off_w[l]))) return rc;
-    if ((rc = wgrad(f, f->dU, C, nullptr, 1, B, f->grad + f->off_b[l]))) return rc;
-    // spectral: dG = c_kx / N^3 rfft(dU) on the kept modes (scaled inside the mix kernel input)
+    if ((rc = wgrad(f, f->dU, C, Vl(f, l, B), C, B, f->grad + f->off_w[l], f->grad + f->off_b[l]))) return rc;
+    // spectral: dG = c_kx / N^3 rfft(dU) on the kept modes (scaled as the mix reads it), dR, dF
     fwd_spectrum(f, f->dU, f->G, (long long)B * C);
-    {  // dG *= c_kx / N^3
-      const long long n = (long long)B * C * f->modes;
-      k_fno_scale_kx<<<nblk(n), kT, 0, f->stream>>>(f->G, n, f->m, f->kx_herm);
-      count_launch(1);
-    }
-    // dR[mode][ci][co] = sum_b conj(F[b][ci]) dG[b][co]
-    k_fno_dR<<<nblk((long long)f->modes * C * C), kT, 0, f->stream>>>(Fl(f, l, B), f->G,
-                                                                      reinterpret_cast<float2 *>(f->grad + f->off_spec[l]),
-                                                                      B, C, f->modes);
-    count_launch(1);
-    const __nv_bfloat162 *R16 = reinterpret_cast<const __nv_bfloat162 *>(f->par16 + f->off_spec[l]);
-    k_fno_mix<<<nblk((long long)B * C * f->modes), kT, 0, f->stream>>>(f->G, R16, reinterpret_cast<float2 *>(f->T1),
-                                                                       B, C, f->modes, f->m, 1, nullptr);
-    count_launch(1);
+    mix_backward(f, Fl(f, l, B), f->G, f->par16 + f->off_spec[l],
+                 f->grad + f->off_spec[l], B);
     // dV_spec = Re sum_k dF_k e^{+i k.r} (no Hermitian doubling, no 1/N^3)
-    inv_spectrum(f, reinterpret_cast<float2 *>(f->T1), f->S, (long long)B * C, 0, 1.f);
-    k_fno_pointwise_back<<<nblk(B * ng), kT, C * C * sizeof(float), f->stream>>>(
-        f->dU, f->par16 + f->off_w[l], f->S, f->dV, B, C, ng);
-    count_launch(1);
+    inv_spectrum(f, Fl(f, l, B), f->S, (long long)B * C, 0, 1.f);
+    // dV, times the activation's derivative of the layer below: its dU
+    pointwise(f, true, f->S, f->dU, f->par16 + f->off_w[l], nullptr, l > 0 ? Ul(f, l - 1, B) : nullptr, nullptr, f->dV, B,
+              0);
+    std::swap(f->dU, f->dV);
   }
-  if ((rc = wgrad(f, f->dV, C, x, 2, B, f->grad + f->off_lw))) return rc;
-  if ((rc = wgrad(f, f->dV, C, nullptr, 1, B, f->grad + f->off_lb))) return rc;
-  return SBSE_OK;
+  return wgrad(f, f->dU, C, x, 2, B, f->grad + f->off_lw, f->grad + f->off_lb);
 }
 
 void refresh_bf16(sbse_fno *f) {
@@ -596,11 +522,11 @@ int sbse_fno_create(sbse_fno **out, int device, int n, int width, int modes, int
   rc = rc ? rc : falloc(f, &f->vel, f->n_par * sizeof(float));
   rc = rc ? rc : falloc(f, &f->par16, f->n_par * sizeof(__nv_bfloat16));
   rc = rc ? rc : falloc(f, &f->tw, n * sizeof(float2));
+  rc = rc ? rc : falloc(f, &f->fold, fo_tab_bytes(n, modes));
   rc = rc ? rc : falloc(f, &f->kx_herm, modes * sizeof(float));
   rc = rc ? rc : falloc(f, &f->V, (layers + 1) * act * sizeof(float));
   rc = rc ? rc : falloc(f, &f->U, layers * act * sizeof(float));
   rc = rc ? rc : falloc(f, &f->S, act * sizeof(float));
-  rc = rc ? rc : falloc(f, &f->T1, act * sizeof(float));
   rc = rc ? rc : falloc(f, &f->dV, act * sizeof(float));
   rc = rc ? rc : falloc(f, &f->dU, act * sizeof(float));
   rc = rc ? rc : falloc(f, &f->F, (size_t)layers * B * width * f->modes * sizeof(float2));
@@ -610,7 +536,7 @@ int sbse_fno_create(sbse_fno **out, int device, int n, int width, int modes, int
   rc = rc ? rc : falloc(f, &f->y, B * f->ng * sizeof(float));
   rc = rc ? rc : falloc(f, &f->dy, B * f->ng * sizeof(float));
   rc = rc ? rc : falloc(f, &f->red, 4096 * sizeof(double));
-  rc = rc ? rc : falloc(f, &f->gout, ((size_t)width * width + 64) * sizeof(double));
+  rc = rc ? rc : falloc(f, &f->gout, ((size_t)width * (width + 3) + 64) * sizeof(double));
   if (rc) {
     sbse::set_thread_error(f->err);
     sbse_fno_destroy(f);
@@ -621,6 +547,23 @@ int sbse_fno_create(sbse_fno **out, int device, int n, int width, int modes, int
     const double a = -2.0 * M_PI * k / n;
     tw[k] = make_float2((float)cos(a), (float)sin(a));
   }
+  std::vector<float2> fold((size_t)(n / 2 + 1) * (modes + 1));
+  for (int p = 0; p <= n / 2; ++p)
+    for (int k = 0; k <= modes; ++k) {
+      const double a = 2.0 * M_PI * ((long long)p * k % n) / n;
+      fold[(size_t)p * (modes + 1) + k] = make_float2((float)cos(a), (float)sin(a));
+    }
+  cudaMemcpy(f->fold, fold.data(), fold.size() * sizeof(float2), cudaMemcpyHostToDevice);
+  f->folded = fo_fwd_smem(n, modes) <= kFoSmemMax && fo_inv_smem(n, modes) <= kFoSmemMax;
+  if (f->folded) {
+    raise_smem_limit((const void *)k_fo_fwd_xy, fo_fwd_smem(n, modes));
+    raise_smem_limit((const void *)k_fo_inv_xy, fo_inv_smem(n, modes));
+  }
+  raise_smem_limit((const void *)k_fo_wgrad, wg_smem(width, width > 2 ? width : 2));
+  const int mb = mix_batch(max_batch, width);
+  raise_smem_limit((const void *)k_fo_mix, 2 * mix_tile_bytes(mb, width));
+  raise_smem_limit((const void *)k_fo_mix_back, 2 * mix_tile_bytes(mb, width) +
+                                                    (size_t)kMxModes * width * (width + 1) * sizeof(__nv_bfloat162));
   std::vector<float> kh(modes);
   for (int k = 0; k < modes; ++k) kh[k] = (k == 0 ? 1.f : 2.f) / (float)f->ng;
   cudaMemcpy(f->tw, tw.data(), n * sizeof(float2), cudaMemcpyHostToDevice);
@@ -636,7 +579,7 @@ void sbse_fno_destroy(sbse_fno *f) {
   if (!f) return;
   cudaSetDevice(f->device);
   if (f->stream) cudaStreamSynchronize(f->stream);
-  void *ptrs[] = {f->par, f->grad, f->mom, f->vel, f->par16, f->tw, f->kx_herm, f->V, f->U, f->S, f->T1, f->dV,
+  void *ptrs[] = {f->par, f->grad, f->mom, f->vel, f->par16, f->tw, f->kx_herm, f->V, f->U, f->S, f->fold, f->dV,
                   f->dU, f->F, f->G, f->C1, f->C2b, f->y, f->dy, f->red, f->gpart, f->gout};
   for (void *p : ptrs)
     if (p) cudaFree(p);
@@ -671,7 +614,7 @@ int sbse_fno_get_params(sbse_fno *f, float *host, float *grad_host) {
 int sbse_fno_forward(sbse_fno *f, int batch, const float *x_dev, float *y_dev) {
   if (!f || !x_dev || !y_dev || batch < 1 || batch > f->maxB) return SBSE_ERR_INVALID_ARG;
   FCK(cudaSetDevice(f->device));
-  forward_impl(f, batch, x_dev);
+  forward_impl(f, batch, x_dev, false);
   FCK(cudaMemcpyAsync(y_dev, f->y, (size_t)batch * f->ng * sizeof(float), cudaMemcpyDeviceToDevice, f->stream));
   FCK(cudaGetLastError());
   FCK(cudaStreamSynchronize(f->stream));
@@ -681,7 +624,7 @@ int sbse_fno_forward(sbse_fno *f, int batch, const float *x_dev, float *y_dev) {
 int sbse_fno_gradients(sbse_fno *f, int batch, const float *x_dev, const float *dy_dev) {
   if (!f || !x_dev || !dy_dev || batch < 1 || batch > f->maxB) return SBSE_ERR_INVALID_ARG;
   FCK(cudaSetDevice(f->device));
-  forward_impl(f, batch, x_dev);
+  forward_impl(f, batch, x_dev, true);
   FCK(cudaMemcpyAsync(f->dy, dy_dev, (size_t)batch * f->ng * sizeof(float), cudaMemcpyDeviceToDevice, f->stream));
   int rc = backward_impl(f, batch, x_dev);
   if (rc) return rc;
@@ -693,7 +636,7 @@ int sbse_fno_gradients(sbse_fno *f, int batch, const float *x_dev, const float *
 int sbse_fno_train_step(sbse_fno *f, int batch, const float *x_dev, const float *t_dev, float lr, double *loss) {
   if (!f || !x_dev || !t_dev || batch < 1 || batch > f->maxB || !(lr > 0.f)) return SBSE_ERR_INVALID_ARG;
   FCK(cudaSetDevice(f->device));
-  forward_impl(f, batch, x_dev);
+  forward_impl(f, batch, x_dev, true);
   const long long n = (long long)batch * f->ng;
   const int blocks = 1024;
   k_fno_mse<<<blocks, kT, 0, f->stream>>>(f->y, t_dev, f->dy, n, 1.f / (float)n, f->red);
@@ -763,7 +706,7 @@ int sbse_surrogate_W(sbse_ctx *ctx, sbse_fno *f, int n_pairs, const int *pi, con
     const int nb = (n_pairs - k0) < bmax ? (n_pairs - k0) : bmax;
     rc = sbse_fno_pair_inputs(ctx, nb, pi + k0, pj + k0, s_rho, s_v, x);
     if (rc) break;
-    forward_impl(f, nb, x);
+    forward_impl(f, nb, x, false);
     for (int k = 0; k < nb; ++k) {
       const int slot = sbse::ctx_pair_slot(ctx, pi[k0 + k], pj[k0 + k]);
       k_store_w<<<nblk(f->ng), kT, 0, f->stream>>>(f->y + (long long)k * f->ng, cv.W + (long long)slot * f->ng,
