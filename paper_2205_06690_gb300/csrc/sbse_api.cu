@@ -1049,8 +1049,8 @@ struct MixedBufs {
 int mixed_bufs(sbse_ctx *ctx, int n_extra_fields, MixedBufs *mb, double **extra) {
   const long long ng = ctx->ng;
   const int n_o = ctx->n_o;
-  const int nb = std::max(ctx->n_occ, ctx->n_c);
-  const size_t pwd = project_work_doubles(n_o, nb, ng);
+  // (not monotonic in the number of basis rows: fewer rows are cut into more chunks)
+  const size_t pwd = std::max(project_work_doubles(n_o, ctx->n_occ, ng), project_work_doubles(n_o, ctx->n_c, ng));
   const size_t doubles = (size_t)n_o * ng + 2 * (size_t)ng + pwd + dot_work_doubles() + (size_t)n_extra_fields * n_o * ng;
   void *vp;
   int rc;
