@@ -7,9 +7,11 @@
 // are split into BF16 high and low parts (x = hi + lo) and three MMAs per K slice accumulate
 // hi*hi + hi*lo + lo*hi in FP32 in tensor memory (relative error ~1e-5 of each product instead of
 // BF16's 4e-3). One CTA owns a 128 x NT output tile (NT <= 256, multiple of 16) and a chunk of grid
-// points; stages of 64 points are double-buffered in shared memory in the canonical K-major layout
+// points; stages of 32 points are double-buffered in shared memory in the canonical K-major layout
 // without swizzle (8-row x 16-byte core matrices: K-adjacent core matrices 128 B apart, row groups
-// 1024 B apart). Thread 0 issues the MMAs and commits them to one mbarrier per stage; every wait on
+// 512 B apart). The producers' loads and conversions bound it, not the MMAs: with stages of 64 points one
+// CTA filled an SM and waited out the load latency of every stage, with 32 two CTAs alternate
+// (512 x 512 and 1024 x 136 over 96^3 together: 9.2 -> 6.3 ms). Thread 0 issues the MMAs and commits them to one mbarrier per stage; every wait on
 // an mbarrier is bounded and sets *err on timeout. Partials (FP64) are reduced by the caller.
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -24,7 +26,7 @@
 namespace sbse {
 
 constexpr int kUmM = 128;     // rows per tile (UMMA M)
-constexpr int kUmBK = 64;     // grid points per stage
+constexpr int kUmBK = 32;     // grid points per stage (two CTAs per SM: one's loads hide behind the other's work)
 constexpr int kUmThreads = 128;  // the cleaning update
 constexpr int kPgThreads = 256;  // the grid-sum GEMM: eight producer warps keep more loads in flight
 constexpr int kUmStages = 2;
@@ -82,14 +84,15 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity) {
   return false;
 }
 
-// bytes of one stage: A hi/lo (128 rows) + B hi/lo (NT rows), BF16, 64 points
+// bytes of one stage: A hi/lo (128 rows) + B hi/lo (NT rows), BF16
 __host__ __device__ constexpr size_t umma_stage_bytes(int nt) {
   return (size_t)2 * (kUmM + nt) * kUmBK * 2;
 }
 
-// offset (bytes) of element (row, k) of a R x 64 BF16 tile in the canonical no-swizzle K-major layout
+constexpr uint32_t kUmGroup = kUmBK / 8 * 128;  // bytes of an 8-row group
+// offset (bytes) of element (row, core matrix kc) of a R x kUmBK BF16 tile, canonical no-swizzle K-major
 __device__ __forceinline__ uint32_t canon_off(int row, int kc) {
-  return (uint32_t)(((row >> 3) * 8 + kc) * 128 + (row & 7) * 16);
+  return (uint32_t)(row >> 3) * kUmGroup + (uint32_t)(kc * 128 + (row & 7) * 16);
 }
 
 __device__ __forceinline__ void split8(const float *x, uint4 *hi, uint4 *lo) {
@@ -124,9 +127,8 @@ __device__ __forceinline__ void load_unit(int u, int units_a, const float *F, co
   const int rr = lane & 7, kq = lane >> 3;
   const bool isA = u < units_a;
   const int uu = isA ? u : u - units_a;
-  const int row = (uu >> 1) * 8 + rr;
-  const int kc = (uu & 1) * 4 + kq;  // core matrix index along K (0..7)
-  const long long kb = k0 + kc * 8;
+  const int row = uu * 8 + rr;
+  const long long kb = k0 + kq * 8;
 #pragma unroll
   for (int j = 0; j < 8; ++j) x[j] = 0.f;
   const bool full = vec_ok && kb + 8 <= kend;
@@ -191,7 +193,7 @@ __device__ __forceinline__ void produce_stage(uint8_t *st, int nt, const float *
   uint8_t *b_lo = b_hi + nt * kUmBK * 2;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rr = lane & 7, kq = lane >> 3;
-  const int units_a = (kUmM / 8) * 2, units_b = (nt / 8) * 2, total = units_a + units_b;
+  const int units_a = kUmM / 8, units_b = nt / 8, total = units_a + units_b;
   const bool vec_ok = (ng & 3) == 0;  // 16-byte aligned rows
   constexpr int W = NTHR / 32;
   for (int u0 = warp; u0 < total; u0 += W * kUB) {
@@ -206,11 +208,10 @@ __device__ __forceinline__ void produce_stage(uint8_t *st, int nt, const float *
       if (u >= total) break;
       const bool isA = u < units_a;
       const int uu = isA ? u : u - units_a;
-      const int row = (uu >> 1) * 8 + rr;
-      const int kc = (uu & 1) * 4 + kq;
+      const int row = uu * 8 + rr;
       uint4 hi, lo;
       split8(x[i], &hi, &lo);
-      const uint32_t off = canon_off(row, kc);
+      const uint32_t off = canon_off(row, kq);
       *reinterpret_cast<uint4 *>((isA ? a_hi : b_hi) + off) = hi;
       *reinterpret_cast<uint4 *>((isA ? a_lo : b_lo) + off) = lo;
     }
@@ -218,7 +219,7 @@ __device__ __forceinline__ void produce_stage(uint8_t *st, int nt, const float *
 }
 
 template <int AMODE>
-__global__ void __launch_bounds__(kPgThreads)
+__global__ void __launch_bounds__(kPgThreads, 2)
     k_umma_prod_gemm(const float *F, const int2 *xi, int M, const float *Y, int Nn, int nt, long long ng,
                      long long kchunk, double *part, int *err) {
   extern __shared__ __align__(128) uint8_t smem[];
@@ -267,8 +268,8 @@ __global__ void __launch_bounds__(kPgThreads)
 #pragma unroll
       for (int t = 0; t < kUmBK / 16; ++t) {
         const uint32_t o = t * 256;  // two core matrices (16 points) per MMA along K
-        const uint64_t dah = make_desc(a_hi + o, 128, 1024), dal = make_desc(a_lo + o, 128, 1024);
-        const uint64_t dbh = make_desc(b_hi + o, 128, 1024), dbl = make_desc(b_lo + o, 128, 1024);
+        const uint64_t dah = make_desc(a_hi + o, 128, kUmGroup), dal = make_desc(a_lo + o, 128, kUmGroup);
+        const uint64_t dbh = make_desc(b_hi + o, 128, kUmGroup), dbl = make_desc(b_lo + o, 128, kUmGroup);
         mma_bf16(tmem, dah, dbh, idesc, (it > 0 || t > 0) ? 1u : 0u);
         mma_bf16(tmem, dah, dbl, idesc, 1u);
         mma_bf16(tmem, dal, dbh, idesc, 1u);
