@@ -632,7 +632,74 @@ __global__ void __launch_bounds__(256)
 
 template <typename T> size_t clean_work_bytes(long long ng, int n_occ, int P, int L) {
   const long long n_cols = (long long)P * L;
-  const long long kc = gemm_kchunk(ng);
+// The same overlaps in FP64. FP64 arithmetic is the bound (about 1.6 multiply-adds per clock and SM), so
+// what counts is that no multiply-add is spent on padding and that every SM has work: a warp owns 4
+// columns x 4 states over one chunk of points, its lanes take consecutive points straight from global
+// memory (3 KB per 32 multiply-adds, a few bytes per clock and SM), and the 32 sums are combined by a
+// reduce-scatter over the lanes (31 additions). The 64 x 64 tile above pads a system of 4 occupied
+// states 16-fold and left it one block: one cleaning of 30 columns on 16^3 (these overlaps and the
+// update below) took 9.2 ms and takes 17 us; 100 columns x 20 states on 40^3, overlaps 8.36 -> 0.52 ms.
+constexpr int kOdC = 4, kOdS = 4, kOdWarps = 4;
+
+// points per chunk: enough chunks for about 16 warps per SM, at least 128 points (4 per lane), whole
+// warps of points
+static long long ov64_chunk(long long ng, int n_cols, int n_occ) {
+  const long long tiles = (long long)((n_cols + kOdC - 1) / kOdC) * ((n_occ + kOdS - 1) / kOdS);
+  const long long want = (152 * 16 + tiles - 1) / tiles;
+  long long c = ((ng + want - 1) / want + 31) / 32 * 32;
+  if (c > 4096) c = 4096;  // a chunk's rows of d and phi stay in L2 while every tile reads them
+  while ((ng + c - 1) / c > 4096) c *= 2;
+  return c < 128 ? 128 : c;
+}
+
+__global__ void __launch_bounds__(32 * kOdWarps)
+    k_clean_overlap64(const double2 *d, const double *phi, int n_cols, int n_occ, long long ng, long long kchunk,
+                      int tiles_c, int tiles, double *part) {
+  const int lane = threadIdx.x & 31;
+  const int tile = blockIdx.x * kOdWarps + (threadIdx.x >> 5);
+  if (tile >= tiles) return;
+  const int c0 = (tile % tiles_c) * kOdC, s0 = (tile / tiles_c) * kOdS;
+  const long long kbeg = (long long)blockIdx.y * kchunk;
+  const long long kend = (kbeg + kchunk < ng) ? kbeg + kchunk : ng;
+  const double2 *dp[kOdC];
+  const double *pp[kOdS];
+  // rows past the last column or state repeat the last one; their sums are not written
+#pragma unroll
+  for (int i = 0; i < kOdC; ++i) dp[i] = d + (long long)min(c0 + i, n_cols - 1) * ng;
+#pragma unroll
+  for (int j = 0; j < kOdS; ++j) pp[j] = phi + (long long)min(s0 + j, n_occ - 1) * ng;
+  double acc[2 * kOdC * kOdS];  // [column][re, im][state]
+#pragma unroll
+  for (int i = 0; i < 2 * kOdC * kOdS; ++i) acc[i] = 0.0;
+  for (long long k = kbeg + lane; k < kend; k += 32) {
+    double2 x[kOdC];
+    double f[kOdS];
+#pragma unroll
+    for (int i = 0; i < kOdC; ++i) x[i] = dp[i][k];
+#pragma unroll
+    for (int j = 0; j < kOdS; ++j) f[j] = pp[j][k];
+#pragma unroll
+    for (int i = 0; i < kOdC; ++i)
+#pragma unroll
+      for (int j = 0; j < kOdS; ++j) {
+        acc[(2 * i) * kOdS + j] = fma(x[i].x, f[j], acc[(2 * i) * kOdS + j]);
+        acc[(2 * i + 1) * kOdS + j] = fma(x[i].y, f[j], acc[(2 * i + 1) * kOdS + j]);
+      }
+  }
+  // reduce-scatter: after the exchange over lane bit w the lane keeps the sums whose index has that bit
+#pragma unroll
+  for (int w = 16; w > 0; w >>= 1)
+#pragma unroll
+    for (int i = 0; i < w; ++i) {
+      const bool up = (lane & w) != 0;
+      const double give = up ? acc[i] : acc[i + w], mine = up ? acc[i + w] : acc[i];
+      acc[i] = mine + __shfl_xor_sync(0xffffffffu, give, w);
+    }
+  const int c = c0 + (lane >> 3), h = (lane >> 2) & 1, s = s0 + (lane & 3);
+  if (c < n_cols && s < n_occ) part[((long long)blockIdx.y * 2 * n_cols + 2 * c + h) * n_occ + s] = acc[0];
+}
+
+  const long long kc = sizeof(T) == 8 ? ov64_chunk(ng, (int)n_cols, n_occ) : gemm_kchunk(ng);
   const long long chunks = (ng + kc - 1) / kc;
   const long long ptb = (ng + kUpPts - 1) / kUpPts;
   size_t b = 0;
@@ -656,7 +723,7 @@ const double *launch_clean(const GridTables<T> &g, const T *phi_occ, int n_occ, 
                            const uint8_t *phi_ov) {
   (void)work_bytes;
   const int n_cols = P * L;
-  const long long kc = gemm_kchunk(g.ng);
+  const long long kc = sizeof(T) == 8 ? ov64_chunk(g.ng, n_cols, n_occ) : gemm_kchunk(g.ng);
   const long long chunks = (g.ng + kc - 1) / kc;
   const long long ptb = (g.ng + kUpPts - 1) / kUpPts;
   double *part = work;
@@ -674,8 +741,14 @@ const double *launch_clean(const GridTables<T> &g, const T *phi_occ, int n_occ, 
     launch_umma_clean_overlap(reinterpret_cast<const float *>(d), n_cols,
                               reinterpret_cast<const float *>(phi_occ), n_occ, g.ng, dV, ov, part, err, s);
   } else {
-    dim3 grid((unsigned)chunks, (n_cols + kOvC - 1) / kOvC, (n_occ + kOvS - 1) / kOvS);
-    k_clean_overlap<T><<<grid, 256, 0, s>>>(d, phi_occ, n_cols, n_occ, g.ng, kc, part);
+    if constexpr (sizeof(T) == 8) {
+      const int tc = (n_cols + kOdC - 1) / kOdC, tiles = tc * ((n_occ + kOdS - 1) / kOdS);
+      dim3 grid((unsigned)((tiles + kOdWarps - 1) / kOdWarps), (unsigned)chunks);
+      k_clean_overlap64<<<grid, 32 * kOdWarps, 0, s>>>(d, phi_occ, n_cols, n_occ, g.ng, kc, tc, tiles, part);
+    } else {
+      dim3 grid((unsigned)chunks, (n_cols + kOvC - 1) / kOvC, (n_occ + kOvS - 1) / kOvS);
+      k_clean_overlap<T><<<grid, 256, 0, s>>>(d, phi_occ, n_cols, n_occ, g.ng, kc, part);
+    }
     count_launch(1);
     launch_reduce_cols(part, (int)chunks, n_cols * n_occ * 2, dV, ov, s);
   }
@@ -687,7 +760,12 @@ const double *launch_clean(const GridTables<T> &g, const T *phi_occ, int n_occ, 
                              reinterpret_cast<const float *>(a), L, npart, o_can, err, s);
     launch_reduce_cols(npart, (int)umma_clean_update_tiles(g.ng), n_cols * 2, dV, sums, s);
   } else {
-    k_clean_update2<T><<<(unsigned)ptb, 256, 0, s>>>(g.ng, phi_occ, n_occ, ov, d, a, n_cols, L, npart);
+    if constexpr (sizeof(T) == 8) {
+      dim3 grid((unsigned)((n_cols + kU6Cols - 1) / kU6Cols), (unsigned)ptb);
+      k_clean_update64<<<grid, kUpPts, 0, s>>>(g.ng, phi_occ, n_occ, ov, d, a, n_cols, L, npart);
+    } else {
+      k_clean_update2<T><<<(unsigned)ptb, 256, 0, s>>>(g.ng, phi_occ, n_occ, ov, d, a, n_cols, L, npart);
+    }
     launch_reduce_cols(npart, (int)ptb, n_cols * 2, dV, sums, s);
   }
   k_cm1<<<(n_cols + 127) / 128, 128, 0, s>>>(n_cols, L, sums, n0, cm1);
@@ -725,6 +803,86 @@ template <typename T> __global__ void k_flush_acc(double *acc64, T *acc, long lo
 template <typename T> void launch_flush_acc(double *acc64, T *acc, long long n, cudaStream_t s) {
   if (n > 0) k_flush_acc<T><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(acc64, acc, n);
   count_launch(1);
+}
+
+// The same update in FP64, again bound by the FP64 multiply-adds: a thread owns one point and 8
+// columns (16 sums), reads phi once per state (coalesced) and the overlaps as broadcasts from shared
+// memory, with no padding of the states (the tile above sweeps 64 of them). Blocks of one tile of 128
+// points are adjacent, so the tile's phi rows are read once from L2. 100 columns x 20 states on 40^3:
+// 2.21 -> 0.55 ms.
+constexpr int kU6Cols = 8, kU6S = 64;
+
+__global__ void __launch_bounds__(kUpPts)
+    k_clean_update64(long long ng, const double *phi, int n_occ, const double *ov /* [2c+h][s], x dV */, double2 *d,
+                     const double2 *a, int n_cols, int L, double *npart) {
+  __shared__ double2 Os[kU6S][kU6Cols];
+  __shared__ double red[kUpPts / 32][2 * kU6Cols];
+  const int c0 = blockIdx.x * kU6Cols, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const long long tile = blockIdx.y, r = tile * kUpPts + threadIdx.x;
+  const bool in = r < ng;
+  double2 acc[kU6Cols];
+#pragma unroll
+  for (int i = 0; i < kU6Cols; ++i) acc[i] = double2{0.0, 0.0};
+  for (int st0 = 0; st0 < n_occ; st0 += kU6S) {
+    const int ns = min(kU6S, n_occ - st0);
+    __syncthreads();
+    for (int l = threadIdx.x; l < kU6Cols * ns; l += kUpPts) {
+      const int i = l / ns, s = l - i * ns;
+      double2 v = double2{0.0, 0.0};
+      if (c0 + i < n_cols) {
+        const double *o = ov + (long long)(2 * (c0 + i)) * n_occ + st0 + s;
+        v = double2{o[0], o[n_occ]};
+      }
+      Os[s][i] = v;
+    }
+    __syncthreads();
+    const double *pr = phi + (long long)st0 * ng + (in ? r : 0);
+#pragma unroll 4
+    for (int s = 0; s < ns; ++s) {
+      const double f = pr[(long long)s * ng];
+#pragma unroll
+      for (int i = 0; i < kU6Cols; ++i) {
+        const double2 o = Os[s][i];
+        acc[i].x = fma(o.x, f, acc[i].x);
+        acc[i].y = fma(o.y, f, acc[i].y);
+      }
+    }
+  }
+  // [0, 8): 2 Re(conj(eta0) d), [8, 16): |d|^2 per column
+  double v[2 * kU6Cols];
+#pragma unroll
+  for (int i = 0; i < kU6Cols; ++i) {
+    v[i] = v[kU6Cols + i] = 0.0;
+    const int c = c0 + i;
+    if (in && c < n_cols) {
+      double2 *dp = d + (long long)c * ng + r;
+      const double2 a0 = a[(long long)(c % L) * ng + r];
+      double2 x = *dp;
+      x.x -= acc[i].x;
+      x.y -= acc[i].y;
+      *dp = x;
+      v[i] = 2.0 * (a0.x * x.x + a0.y * x.y);
+      v[kU6Cols + i] = x.x * x.x + x.y * x.y;
+    }
+  }
+#pragma unroll
+  for (int w = 8; w > 0; w >>= 1)  // reduce-scatter over 16 lanes, then the two halves of the warp
+#pragma unroll
+    for (int i = 0; i < w; ++i) {
+      const bool up = (lane & w) != 0;
+      const double give = up ? v[i] : v[i + w], mine = up ? v[i + w] : v[i];
+      v[i] = mine + __shfl_xor_sync(0xffffffffu, give, w);
+    }
+  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 16);
+  if (lane < 2 * kU6Cols) red[warp][lane] = v[0];
+  __syncthreads();
+  if (threadIdx.x < 2 * kU6Cols) {
+    const int c = c0 + (threadIdx.x & (kU6Cols - 1)), h = threadIdx.x / kU6Cols;
+    double t = 0.0;
+#pragma unroll
+    for (int w = 0; w < kUpPts / 32; ++w) t += red[w][threadIdx.x];
+    if (c < n_cols) npart[(tile * n_cols + c) * 2 + h] = t;
+  }
 }
 
 template <typename T> __global__ void k_convert(const double *src, T *dst, long long n) {
