@@ -57,6 +57,9 @@ void launch_plane_kin2(const GridTables<float> &g, const XfwdArgs<float> &a, cud
 // copies while the one before is transformed (bounded waits; *err set if one runs out)
 void launch_zkin2(const GridTables<float> &g, float2 *d, int n_items, const float2 *a_next, int L, float *dens,
                   cudaStream_t s, int *err = nullptr);
+// induced density of each pair from its L stored orbitals (Eq. 11), where the inverse pass does not sum it
+template <typename T> void launch_density(const GridTables<T> &g, const C2<T> *d, const C2<T> *a, int P, int L, T *dens,
+                                          cudaStream_t s);
 // out = exp(-i V_loc tau), computed in FP64 from the FP64 potential v64
 template <typename T> void launch_phase_table(const double *v64, long long ng, double tau, C2<T> *out,
                                               cudaStream_t s);

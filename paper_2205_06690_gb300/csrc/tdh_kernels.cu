@@ -381,9 +381,8 @@ __global__ void k_kick(long long ng, const double *q, int P, const C2<T> *a, int
   const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int pair = blockIdx.y;
   if (r >= ng) return;
-  double s, c;
-  sincos(0.5 * alpha * q[(long long)pair * ng + r], &s, &c);
-  const C2<T> f = C2<T>{(T)(-2.0 * s * s), (T)(-2.0 * s * c)};
+  const double2 e = phase_em1<double>(q[(long long)pair * ng + r], alpha);
+  const C2<T> f = C2<T>{(T)e.x, (T)e.y};
   for (int ell = 0; ell < L; ++ell)
     d[((long long)pair * L + ell) * ng + r] = cmul(f, a[(long long)ell * ng + r]);
 }
@@ -419,9 +418,50 @@ __global__ void k_half_phase(long long ng, C2<T> *a, C2<T> *d, const C2<T> *pv, 
   a[(long long)ell * ng + r] = cmul(p, av);
 }
 
+// The same in FP32 with two points per thread (16-byte accesses; even point counts keep every row
+// aligned) and the loads of four pairs in flight: HBM-bound. 68 pairs x 10 orbitals of 96^3:
+// 2125 -> 2056 us; 36 pairs of 48^3: 128 -> 112 us.
+__global__ void __launch_bounds__(256)
+    k_half_phase2(long long n2, float4 *a, float4 *d, const float4 *pv, const float4 *em1, int P, int L) {
+  const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const int ell = blockIdx.y;
+  if (r >= n2) return;
+  const float4 av = a[(long long)ell * n2 + r], p = pv[r];
+  constexpr int UB = 4;
+  for (int p0 = 0; p0 < P; p0 += UB) {
+    float4 dv[UB], em[UB];
+#pragma unroll
+    for (int u = 0; u < UB; ++u) {
+      const int pair = min(p0 + u, P - 1);
+      dv[u] = d[((long long)pair * L + ell) * n2 + r];
+      em[u] = em1 ? em1[(long long)pair * n2 + r] : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll
+    for (int u = 0; u < UB; ++u)
+      if (p0 + u < P) {
+        const float2 lo = pair_phase<float>(float2{p.x, p.y}, float2{em[u].x, em[u].y}, float2{av.x, av.y},
+                                            float2{dv[u].x, dv[u].y});
+        const float2 hi = pair_phase<float>(float2{p.z, p.w}, float2{em[u].z, em[u].w}, float2{av.z, av.w},
+                                            float2{dv[u].z, dv[u].w});
+        d[((long long)(p0 + u) * L + ell) * n2 + r] = make_float4(lo.x, lo.y, hi.x, hi.y);
+      }
+  }
+  const float2 lo = cmul(float2{p.x, p.y}, float2{av.x, av.y}), hi = cmul(float2{p.z, p.w}, float2{av.z, av.w});
+  a[(long long)ell * n2 + r] = make_float4(lo.x, lo.y, hi.x, hi.y);
+}
+
 template <typename T>
 void launch_half_phase(const GridTables<T> &g, C2<T> *a, C2<T> *d, const C2<T> *em1, int P, int L,
                        cudaStream_t s) {
+  if (sizeof(T) == 4 && g.ng % 2 == 0) {
+    const long long n2 = g.ng / 2;
+    dim3 grid((unsigned)((n2 + 255) / 256), L);
+    k_half_phase2<<<grid, 256, 0, s>>>(n2, reinterpret_cast<float4 *>(a), reinterpret_cast<float4 *>(d),
+                                       reinterpret_cast<const float4 *>(g.pv_half), reinterpret_cast<const float4 *>(em1),
+                                       P, L);
+    count_launch(1);
+    return;
+  }
   dim3 grid((unsigned)((g.ng + 255) / 256), L);
   k_half_phase<T><<<grid, 256, 0, s>>>(g.ng, a, d, g.pv_half, em1, P, L);
   count_launch(1);
@@ -464,6 +504,63 @@ __global__ void k_density_renormed(long long ng, const C2<T> *d, const C2<T> *a,
     acc += T(2) * (T(2) * (a0.x * dv.x + a0.y * dv.y) + dv.x * dv.x + dv.y * dv.y);
   }
   dens[(long long)pair * ng + r] = acc;
+}
+
+// The same in FP32 with two points per thread (16-byte loads, even point counts) and the loads of five
+// orbitals in flight. 68 pairs x 10 orbitals of 96^3: 1458 -> 1341 us; 36 pairs of 48^3: 75 -> 60 us.
+__global__ void __launch_bounds__(256)
+    k_density_renormed2(long long n2, const float4 *d, const float4 *a, int L, const double *cm1v, float2 *dens) {
+  extern __shared__ float cm1f[];
+  const int pair = blockIdx.y;
+  for (int l = threadIdx.x; l < L; l += blockDim.x) cm1f[l] = (float)cm1v[(long long)pair * L + l];
+  __syncthreads();
+  const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (r >= n2) return;
+  float s0 = 0.f, s1 = 0.f;
+  constexpr int UB = 5;
+  for (int l0 = 0; l0 < L; l0 += UB) {
+    float4 dv[UB], av[UB];
+#pragma unroll
+    for (int u = 0; u < UB; ++u) {
+      const int l = min(l0 + u, L - 1);
+      dv[u] = d[((long long)pair * L + l) * n2 + r];
+      av[u] = a[(long long)l * n2 + r];
+    }
+#pragma unroll
+    for (int u = 0; u < UB; ++u)
+      if (l0 + u < L) {
+        const float c = cm1f[l0 + u];
+        const float2 a0{av[u].x, av[u].y}, a1{av[u].z, av[u].w};
+        const float2 x0 = renorm_value<float>(float2{dv[u].x, dv[u].y}, a0, c);
+        const float2 x1 = renorm_value<float>(float2{dv[u].z, dv[u].w}, a1, c);
+        s0 += 2.f * (2.f * (a0.x * x0.x + a0.y * x0.y) + x0.x * x0.x + x0.y * x0.y);
+        s1 += 2.f * (2.f * (a1.x * x1.x + a1.y * x1.y) + x1.x * x1.x + x1.y * x1.y);
+      }
+  }
+  dens[(long long)pair * n2 + r] = float2{s0, s1};
+}
+
+// the induced densities of the stored orbitals (see launch_plane_inv_orb)
+template <typename T>
+__global__ void k_density(long long ng, const C2<T> *d, const C2<T> *a, int L, T *dens) {
+  const int pair = blockIdx.y;
+  const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (r >= ng) return;
+  T acc = T(0);
+#pragma unroll 2
+  for (int ell = 0; ell < L; ++ell) {
+    const C2<T> dv = d[((long long)pair * L + ell) * ng + r], a0 = a[(long long)ell * ng + r];
+    acc += T(2) * (T(2) * (a0.x * dv.x + a0.y * dv.y) + dv.x * dv.x + dv.y * dv.y);
+  }
+  dens[(long long)pair * ng + r] = acc;
+}
+
+template <typename T>
+void launch_density(const GridTables<T> &g, const C2<T> *d, const C2<T> *a, int P, int L, T *dens, cudaStream_t s) {
+  const int nt = g.ng * P < 256ll * 304 ? 64 : 256;
+  dim3 grid((unsigned)((g.ng + nt - 1) / nt), P);
+  k_density<T><<<grid, nt, 0, s>>>(g.ng, d, a, L, dens);
+  count_launch(1);
 }
 
 // Overlaps of the complex columns d_c with the occupied orbitals, split over chunks of grid
@@ -533,6 +630,73 @@ __global__ void __launch_bounds__(256)
       o[n_occ] = (double)aim[i][j];
     }
   }
+}
+
+// The same overlaps in FP64. FP64 arithmetic is the bound (about 1.6 multiply-adds per clock and SM), so
+// what counts is that no multiply-add is spent on padding and that every SM has work: a warp owns 4
+// columns x 4 states over one chunk of points, its lanes take consecutive points straight from global
+// memory (3 KB per 32 multiply-adds, a few bytes per clock and SM), and the 32 sums are combined by a
+// reduce-scatter over the lanes (31 additions). The 64 x 64 tile above pads a system of 4 occupied
+// states 16-fold and left it one block: one cleaning of 30 columns on 16^3 (these overlaps and the
+// update below) took 9.2 ms and takes 17 us; 100 columns x 20 states on 40^3, overlaps 8.36 -> 0.52 ms.
+constexpr int kOdC = 4, kOdS = 4, kOdWarps = 4;
+
+// points per chunk: enough chunks for about 16 warps per SM, at least 128 points (4 per lane), whole
+// warps of points
+static long long ov64_chunk(long long ng, int n_cols, int n_occ) {
+  const long long tiles = (long long)((n_cols + kOdC - 1) / kOdC) * ((n_occ + kOdS - 1) / kOdS);
+  const long long want = (152 * 16 + tiles - 1) / tiles;
+  long long c = ((ng + want - 1) / want + 31) / 32 * 32;
+  if (c > 4096) c = 4096;  // a chunk's rows of d and phi stay in L2 while every tile reads them
+  while ((ng + c - 1) / c > 4096) c *= 2;
+  return c < 128 ? 128 : c;
+}
+
+__global__ void __launch_bounds__(32 * kOdWarps)
+    k_clean_overlap64(const double2 *d, const double *phi, int n_cols, int n_occ, long long ng, long long kchunk,
+                      int tiles_c, int tiles, double *part) {
+  const int lane = threadIdx.x & 31;
+  const int tile = blockIdx.x * kOdWarps + (threadIdx.x >> 5);
+  if (tile >= tiles) return;
+  const int c0 = (tile % tiles_c) * kOdC, s0 = (tile / tiles_c) * kOdS;
+  const long long kbeg = (long long)blockIdx.y * kchunk;
+  const long long kend = (kbeg + kchunk < ng) ? kbeg + kchunk : ng;
+  const double2 *dp[kOdC];
+  const double *pp[kOdS];
+  // rows past the last column or state repeat the last one; their sums are not written
+#pragma unroll
+  for (int i = 0; i < kOdC; ++i) dp[i] = d + (long long)min(c0 + i, n_cols - 1) * ng;
+#pragma unroll
+  for (int j = 0; j < kOdS; ++j) pp[j] = phi + (long long)min(s0 + j, n_occ - 1) * ng;
+  double acc[2 * kOdC * kOdS];  // [column][re, im][state]
+#pragma unroll
+  for (int i = 0; i < 2 * kOdC * kOdS; ++i) acc[i] = 0.0;
+  for (long long k = kbeg + lane; k < kend; k += 32) {
+    double2 x[kOdC];
+    double f[kOdS];
+#pragma unroll
+    for (int i = 0; i < kOdC; ++i) x[i] = dp[i][k];
+#pragma unroll
+    for (int j = 0; j < kOdS; ++j) f[j] = pp[j][k];
+#pragma unroll
+    for (int i = 0; i < kOdC; ++i)
+#pragma unroll
+      for (int j = 0; j < kOdS; ++j) {
+        acc[(2 * i) * kOdS + j] = fma(x[i].x, f[j], acc[(2 * i) * kOdS + j]);
+        acc[(2 * i + 1) * kOdS + j] = fma(x[i].y, f[j], acc[(2 * i + 1) * kOdS + j]);
+      }
+  }
+  // reduce-scatter: after the exchange over lane bit w the lane keeps the sums whose index has that bit
+#pragma unroll
+  for (int w = 16; w > 0; w >>= 1)
+#pragma unroll
+    for (int i = 0; i < w; ++i) {
+      const bool up = (lane & w) != 0;
+      const double give = up ? acc[i] : acc[i + w], mine = up ? acc[i + w] : acc[i];
+      acc[i] = mine + __shfl_xor_sync(0xffffffffu, give, w);
+    }
+  const int c = c0 + (lane >> 3), h = (lane >> 2) & 1, s = s0 + (lane & 3);
+  if (c < n_cols && s < n_occ) part[((long long)blockIdx.y * 2 * n_cols + 2 * c + h) * n_occ + s] = acc[0];
 }
 
 // d_c(r) -= sum_s O[c][s] phi_s(r) on 128 points per block, all columns in groups of 32 (4 points
@@ -630,181 +794,6 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-template <typename T> size_t clean_work_bytes(long long ng, int n_occ, int P, int L) {
-  const long long n_cols = (long long)P * L;
-// The same overlaps in FP64. FP64 arithmetic is the bound (about 1.6 multiply-adds per clock and SM), so
-// what counts is that no multiply-add is spent on padding and that every SM has work: a warp owns 4
-// columns x 4 states over one chunk of points, its lanes take consecutive points straight from global
-// memory (3 KB per 32 multiply-adds, a few bytes per clock and SM), and the 32 sums are combined by a
-// reduce-scatter over the lanes (31 additions). The 64 x 64 tile above pads a system of 4 occupied
-// states 16-fold and left it one block: one cleaning of 30 columns on 16^3 (these overlaps and the
-// update below) took 9.2 ms and takes 17 us; 100 columns x 20 states on 40^3, overlaps 8.36 -> 0.52 ms.
-constexpr int kOdC = 4, kOdS = 4, kOdWarps = 4;
-
-// points per chunk: enough chunks for about 16 warps per SM, at least 128 points (4 per lane), whole
-// warps of points
-static long long ov64_chunk(long long ng, int n_cols, int n_occ) {
-  const long long tiles = (long long)((n_cols + kOdC - 1) / kOdC) * ((n_occ + kOdS - 1) / kOdS);
-  const long long want = (152 * 16 + tiles - 1) / tiles;
-  long long c = ((ng + want - 1) / want + 31) / 32 * 32;
-  if (c > 4096) c = 4096;  // a chunk's rows of d and phi stay in L2 while every tile reads them
-  while ((ng + c - 1) / c > 4096) c *= 2;
-  return c < 128 ? 128 : c;
-}
-
-__global__ void __launch_bounds__(32 * kOdWarps)
-    k_clean_overlap64(const double2 *d, const double *phi, int n_cols, int n_occ, long long ng, long long kchunk,
-                      int tiles_c, int tiles, double *part) {
-  const int lane = threadIdx.x & 31;
-  const int tile = blockIdx.x * kOdWarps + (threadIdx.x >> 5);
-  if (tile >= tiles) return;
-  const int c0 = (tile % tiles_c) * kOdC, s0 = (tile / tiles_c) * kOdS;
-  const long long kbeg = (long long)blockIdx.y * kchunk;
-  const long long kend = (kbeg + kchunk < ng) ? kbeg + kchunk : ng;
-  const double2 *dp[kOdC];
-  const double *pp[kOdS];
-  // rows past the last column or state repeat the last one; their sums are not written
-#pragma unroll
-  for (int i = 0; i < kOdC; ++i) dp[i] = d + (long long)min(c0 + i, n_cols - 1) * ng;
-#pragma unroll
-  for (int j = 0; j < kOdS; ++j) pp[j] = phi + (long long)min(s0 + j, n_occ - 1) * ng;
-  double acc[2 * kOdC * kOdS];  // [column][re, im][state]
-#pragma unroll
-  for (int i = 0; i < 2 * kOdC * kOdS; ++i) acc[i] = 0.0;
-  for (long long k = kbeg + lane; k < kend; k += 32) {
-    double2 x[kOdC];
-    double f[kOdS];
-#pragma unroll
-    for (int i = 0; i < kOdC; ++i) x[i] = dp[i][k];
-#pragma unroll
-    for (int j = 0; j < kOdS; ++j) f[j] = pp[j][k];
-#pragma unroll
-    for (int i = 0; i < kOdC; ++i)
-#pragma unroll
-      for (int j = 0; j < kOdS; ++j) {
-        acc[(2 * i) * kOdS + j] = fma(x[i].x, f[j], acc[(2 * i) * kOdS + j]);
-        acc[(2 * i + 1) * kOdS + j] = fma(x[i].y, f[j], acc[(2 * i + 1) * kOdS + j]);
-      }
-  }
-  // reduce-scatter: after the exchange over lane bit w the lane keeps the sums whose index has that bit
-#pragma unroll
-  for (int w = 16; w > 0; w >>= 1)
-#pragma unroll
-    for (int i = 0; i < w; ++i) {
-      const bool up = (lane & w) != 0;
-      const double give = up ? acc[i] : acc[i + w], mine = up ? acc[i + w] : acc[i];
-      acc[i] = mine + __shfl_xor_sync(0xffffffffu, give, w);
-    }
-  const int c = c0 + (lane >> 3), h = (lane >> 2) & 1, s = s0 + (lane & 3);
-  if (c < n_cols && s < n_occ) part[((long long)blockIdx.y * 2 * n_cols + 2 * c + h) * n_occ + s] = acc[0];
-}
-
-  const long long kc = sizeof(T) == 8 ? ov64_chunk(ng, (int)n_cols, n_occ) : gemm_kchunk(ng);
-  const long long chunks = (ng + kc - 1) / kc;
-  const long long ptb = (ng + kUpPts - 1) / kUpPts;
-  size_t b = 0;
-  const size_t tc_part = std::max(umma_prod_gemm_work_bytes((int)(2 * n_cols), n_occ, ng),
-                                  umma_clean_ov_work_bytes((int)n_cols, n_occ, ng));
-  const size_t simt_part = (size_t)(chunks * n_cols * n_occ * 2) * sizeof(double);
-  b += simt_part > tc_part ? simt_part : tc_part;                 // overlap partials
-  b += (size_t)(n_cols * n_occ * 2) * sizeof(double);           // overlaps
-  b += (size_t)(ptb * n_cols * 2) * sizeof(double);             // norm partials
-  b += (size_t)(n_cols * 2) * sizeof(double);                   // norm sums
-  b += (size_t)n_cols * sizeof(double);                         // c - 1 per column
-  b = (b + 127) / 128 * 128;
-  if (sizeof(T) == 4) b += umma_update_o_bytes((int)n_cols, n_occ);  // overlaps as operand tiles
-  return b;
-}
-
-template <typename T>
-const double *launch_clean(const GridTables<T> &g, const T *phi_occ, int n_occ, const C2<T> *a, C2<T> *d,
-                           int P, int L, const double *n0, double dV, double *work, size_t work_bytes,
-                           bool use_tc, const uint8_t *phi_can, int *err, cudaStream_t s, T *dens,
-                           const uint8_t *phi_ov) {
-  (void)work_bytes;
-  const int n_cols = P * L;
-  const long long kc = sizeof(T) == 8 ? ov64_chunk(g.ng, n_cols, n_occ) : gemm_kchunk(g.ng);
-  const long long chunks = (g.ng + kc - 1) / kc;
-  const long long ptb = (g.ng + kUpPts - 1) / kUpPts;
-  double *part = work;
-  const size_t tc_part = std::max(umma_prod_gemm_work_bytes(2 * n_cols, n_occ, g.ng),
-                                  umma_clean_ov_work_bytes(n_cols, n_occ, g.ng)) / sizeof(double);
-  const size_t simt_part = (size_t)(chunks * n_cols * n_occ * 2);
-  double *ov = part + (simt_part > tc_part ? simt_part : tc_part);
-  double *npart = ov + (long long)n_cols * n_occ * 2;
-  double *sums = npart + ptb * n_cols * 2;
-  double *cm1 = sums + (long long)n_cols * 2;
-  if (phi_ov && sizeof(T) == sizeof(float) &&
-      launch_umma_clean_ov(reinterpret_cast<const float *>(d), n_cols, phi_ov, n_occ, g.ng, dV, ov, part, err,
-                           s) == 0) {
-  } else if (use_tc && sizeof(T) == sizeof(float)) {
-    launch_umma_clean_overlap(reinterpret_cast<const float *>(d), n_cols,
-                              reinterpret_cast<const float *>(phi_occ), n_occ, g.ng, dV, ov, part, err, s);
-  } else {
-    if constexpr (sizeof(T) == 8) {
-      const int tc = (n_cols + kOdC - 1) / kOdC, tiles = tc * ((n_occ + kOdS - 1) / kOdS);
-      dim3 grid((unsigned)((tiles + kOdWarps - 1) / kOdWarps), (unsigned)chunks);
-      k_clean_overlap64<<<grid, 32 * kOdWarps, 0, s>>>(d, phi_occ, n_cols, n_occ, g.ng, kc, tc, tiles, part);
-    } else {
-      dim3 grid((unsigned)chunks, (n_cols + kOvC - 1) / kOvC, (n_occ + kOvS - 1) / kOvS);
-      k_clean_overlap<T><<<grid, 256, 0, s>>>(d, phi_occ, n_cols, n_occ, g.ng, kc, part);
-    }
-    count_launch(1);
-    launch_reduce_cols(part, (int)chunks, n_cols * n_occ * 2, dV, ov, s);
-  }
-  if (phi_can && sizeof(T) == sizeof(float)) {
-    size_t o_off = (size_t)((cm1 + n_cols) - work) * sizeof(double);
-    o_off = (o_off + 127) / 128 * 128;
-    uint8_t *o_can = reinterpret_cast<uint8_t *>(work) + o_off;
-    launch_umma_clean_update(ov, n_cols, phi_can, n_occ, g.ng, reinterpret_cast<float *>(d),
-                             reinterpret_cast<const float *>(a), L, npart, o_can, err, s);
-    launch_reduce_cols(npart, (int)umma_clean_update_tiles(g.ng), n_cols * 2, dV, sums, s);
-  } else {
-    if constexpr (sizeof(T) == 8) {
-      dim3 grid((unsigned)((n_cols + kU6Cols - 1) / kU6Cols), (unsigned)ptb);
-      k_clean_update64<<<grid, kUpPts, 0, s>>>(g.ng, phi_occ, n_occ, ov, d, a, n_cols, L, npart);
-    } else {
-      k_clean_update2<T><<<(unsigned)ptb, 256, 0, s>>>(g.ng, phi_occ, n_occ, ov, d, a, n_cols, L, npart);
-    }
-    launch_reduce_cols(npart, (int)ptb, n_cols * 2, dV, sums, s);
-  }
-  k_cm1<<<(n_cols + 127) / 128, 128, 0, s>>>(n_cols, L, sums, n0, cm1);
-  dim3 g3((unsigned)((g.ng + 255) / 256), P);
-  k_density_renormed<T><<<g3, 256, (size_t)L * sizeof(T), s>>>(g.ng, d, a, L, cm1, dens);
-  count_launch(3);
-  return cm1;
-}
-
-// ------------------------------------------------------------------------------------------
-
-// out = exp(-i V_loc tau) per grid point
-// (computed in FP64 from the FP64 potential, then rounded to T)
-template <typename T> __global__ void k_phase_table(const double *v, long long ng, double tau, C2<T> *out) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < ng) {
-    const double2 e = expmi<double>(v[i] * tau);
-    out[i] = C2<T>{(T)e.x, (T)e.y};
-  }
-}
-template <typename T>
-void launch_phase_table(const double *v64, long long ng, double tau, C2<T> *out, cudaStream_t s) {
-  k_phase_table<T><<<(unsigned)((ng + 255) / 256), 256, 0, s>>>(v64, ng, tau, out);
-  count_launch(1);
-}
-
-// acc64 += acc; acc = 0  (FP32 partial sums of the time integral folded into the FP64 W)
-template <typename T> __global__ void k_flush_acc(double *acc64, T *acc, long long n) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) {
-    acc64[i] += (double)acc[i];
-    acc[i] = T(0);
-  }
-}
-template <typename T> void launch_flush_acc(double *acc64, T *acc, long long n, cudaStream_t s) {
-  if (n > 0) k_flush_acc<T><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(acc64, acc, n);
-  count_launch(1);
-}
-
 // The same update in FP64, again bound by the FP64 multiply-adds: a thread owns one point and 8
 // columns (16 sums), reads phi once per state (coalesced) and the overlaps as broadcasts from shared
 // memory, with no padding of the states (the tile above sweeps 64 of them). Blocks of one tile of 128
@@ -885,6 +874,122 @@ __global__ void __launch_bounds__(kUpPts)
   }
 }
 
+template <typename T> size_t clean_work_bytes(long long ng, int n_occ, int P, int L) {
+  const long long n_cols = (long long)P * L;
+  const long long kc = sizeof(T) == 8 ? ov64_chunk(ng, (int)n_cols, n_occ) : gemm_kchunk(ng);
+  const long long chunks = (ng + kc - 1) / kc;
+  const long long ptb = (ng + kUpPts - 1) / kUpPts;
+  size_t b = 0;
+  const size_t tc_part = std::max(umma_prod_gemm_work_bytes((int)(2 * n_cols), n_occ, ng),
+                                  umma_clean_ov_work_bytes((int)n_cols, n_occ, ng));
+  const size_t simt_part = (size_t)(chunks * n_cols * n_occ * 2) * sizeof(double);
+  b += simt_part > tc_part ? simt_part : tc_part;                 // overlap partials
+  b += (size_t)(n_cols * n_occ * 2) * sizeof(double);           // overlaps
+  b += (size_t)(ptb * n_cols * 2) * sizeof(double);             // norm partials
+  b += (size_t)(n_cols * 2) * sizeof(double);                   // norm sums
+  b += (size_t)n_cols * sizeof(double);                         // c - 1 per column
+  b = (b + 127) / 128 * 128;
+  if (sizeof(T) == 4) b += umma_update_o_bytes((int)n_cols, n_occ);  // overlaps as operand tiles
+  return b;
+}
+
+template <typename T>
+const double *launch_clean(const GridTables<T> &g, const T *phi_occ, int n_occ, const C2<T> *a, C2<T> *d,
+                           int P, int L, const double *n0, double dV, double *work, size_t work_bytes,
+                           bool use_tc, const uint8_t *phi_can, int *err, cudaStream_t s, T *dens,
+                           const uint8_t *phi_ov) {
+  (void)work_bytes;
+  const int n_cols = P * L;
+  const long long kc = sizeof(T) == 8 ? ov64_chunk(g.ng, n_cols, n_occ) : gemm_kchunk(g.ng);
+  const long long chunks = (g.ng + kc - 1) / kc;
+  const long long ptb = (g.ng + kUpPts - 1) / kUpPts;
+  double *part = work;
+  const size_t tc_part = std::max(umma_prod_gemm_work_bytes(2 * n_cols, n_occ, g.ng),
+                                  umma_clean_ov_work_bytes(n_cols, n_occ, g.ng)) / sizeof(double);
+  const size_t simt_part = (size_t)(chunks * n_cols * n_occ * 2);
+  double *ov = part + (simt_part > tc_part ? simt_part : tc_part);
+  double *npart = ov + (long long)n_cols * n_occ * 2;
+  double *sums = npart + ptb * n_cols * 2;
+  double *cm1 = sums + (long long)n_cols * 2;
+  if (phi_ov && sizeof(T) == sizeof(float) &&
+      launch_umma_clean_ov(reinterpret_cast<const float *>(d), n_cols, phi_ov, n_occ, g.ng, dV, ov, part, err,
+                           s) == 0) {
+  } else if (use_tc && sizeof(T) == sizeof(float)) {
+    launch_umma_clean_overlap(reinterpret_cast<const float *>(d), n_cols,
+                              reinterpret_cast<const float *>(phi_occ), n_occ, g.ng, dV, ov, part, err, s);
+  } else {
+    if constexpr (sizeof(T) == 8) {
+      const int tc = (n_cols + kOdC - 1) / kOdC, tiles = tc * ((n_occ + kOdS - 1) / kOdS);
+      dim3 grid((unsigned)((tiles + kOdWarps - 1) / kOdWarps), (unsigned)chunks);
+      k_clean_overlap64<<<grid, 32 * kOdWarps, 0, s>>>(d, phi_occ, n_cols, n_occ, g.ng, kc, tc, tiles, part);
+    } else {
+      dim3 grid((unsigned)chunks, (n_cols + kOvC - 1) / kOvC, (n_occ + kOvS - 1) / kOvS);
+      k_clean_overlap<T><<<grid, 256, 0, s>>>(d, phi_occ, n_cols, n_occ, g.ng, kc, part);
+    }
+    count_launch(1);
+    launch_reduce_cols(part, (int)chunks, n_cols * n_occ * 2, dV, ov, s);
+  }
+  if (phi_can && sizeof(T) == sizeof(float)) {
+    size_t o_off = (size_t)((cm1 + n_cols) - work) * sizeof(double);
+    o_off = (o_off + 127) / 128 * 128;
+    uint8_t *o_can = reinterpret_cast<uint8_t *>(work) + o_off;
+    launch_umma_clean_update(ov, n_cols, phi_can, n_occ, g.ng, reinterpret_cast<float *>(d),
+                             reinterpret_cast<const float *>(a), L, npart, o_can, err, s);
+    launch_reduce_cols(npart, (int)umma_clean_update_tiles(g.ng), n_cols * 2, dV, sums, s);
+  } else {
+    if constexpr (sizeof(T) == 8) {
+      dim3 grid((unsigned)((n_cols + kU6Cols - 1) / kU6Cols), (unsigned)ptb);
+      k_clean_update64<<<grid, kUpPts, 0, s>>>(g.ng, phi_occ, n_occ, ov, d, a, n_cols, L, npart);
+    } else {
+      k_clean_update2<T><<<(unsigned)ptb, 256, 0, s>>>(g.ng, phi_occ, n_occ, ov, d, a, n_cols, L, npart);
+    }
+    launch_reduce_cols(npart, (int)ptb, n_cols * 2, dV, sums, s);
+  }
+  k_cm1<<<(n_cols + 127) / 128, 128, 0, s>>>(n_cols, L, sums, n0, cm1);
+  if (sizeof(T) == 4 && g.ng % 2 == 0) {
+    const long long n2 = g.ng / 2;
+    dim3 g2((unsigned)((n2 + 255) / 256), P);
+    k_density_renormed2<<<g2, 256, (size_t)L * sizeof(float), s>>>(n2, reinterpret_cast<const float4 *>(d),
+                                                                   reinterpret_cast<const float4 *>(a), L, cm1,
+                                                                   reinterpret_cast<float2 *>(dens));
+  } else {
+    dim3 g3((unsigned)((g.ng + 255) / 256), P);
+    k_density_renormed<T><<<g3, 256, (size_t)L * sizeof(T), s>>>(g.ng, d, a, L, cm1, dens);
+  }
+  count_launch(3);
+  return cm1;
+}
+
+// ------------------------------------------------------------------------------------------
+
+// out = exp(-i V_loc tau) per grid point
+// (computed in FP64 from the FP64 potential, then rounded to T)
+template <typename T> __global__ void k_phase_table(const double *v, long long ng, double tau, C2<T> *out) {
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < ng) {
+    const double2 e = expmi<double>(v[i] * tau);
+    out[i] = C2<T>{(T)e.x, (T)e.y};
+  }
+}
+template <typename T>
+void launch_phase_table(const double *v64, long long ng, double tau, C2<T> *out, cudaStream_t s) {
+  k_phase_table<T><<<(unsigned)((ng + 255) / 256), 256, 0, s>>>(v64, ng, tau, out);
+  count_launch(1);
+}
+
+// acc64 += acc; acc = 0  (FP32 partial sums of the time integral folded into the FP64 W)
+template <typename T> __global__ void k_flush_acc(double *acc64, T *acc, long long n) {
+  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < n) {
+    acc64[i] += (double)acc[i];
+    acc[i] = T(0);
+  }
+}
+template <typename T> void launch_flush_acc(double *acc64, T *acc, long long n, cudaStream_t s) {
+  if (n > 0) k_flush_acc<T><<<(unsigned)((n + 255) / 256), 256, 0, s>>>(acc64, acc, n);
+  count_launch(1);
+}
+
 template <typename T> __global__ void k_convert(const double *src, T *dst, long long n) {
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) dst[i] = (T)src[i];
@@ -942,6 +1047,7 @@ void init_fft_kernels() {
   template const double *launch_clean<T>(const GridTables<T> &, const T *, int, const C2<T> *,      \
                                          C2<T> *, int, int, const double *, double, double *, size_t, \
                                          bool, const uint8_t *, int *, cudaStream_t, T *, const uint8_t *); \
+  template void launch_density<T>(const GridTables<T> &, const C2<T> *, const C2<T> *, int, int, T *, cudaStream_t); \
   template size_t clean_work_bytes<T>(long long, int, int, int);                                   \
   template void launch_convert<T>(const double *, T *, long long, cudaStream_t);
 
