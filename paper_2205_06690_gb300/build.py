@@ -18,7 +18,7 @@ LIB = os.path.join(PKG, "libsbse.so")
 # record instead of faulting, read by sbse_debug_bounds), linked as libsbse_dbg.so
 OBJ_DBG = os.path.join(PKG, "_build_dbg")
 LIB_DBG = os.path.join(PKG, "libsbse_dbg.so")
-SOURCES = ["sbse_api.cu", "tdh_kernels.cu", "fft_fast.cu", "fft_split.cu", "contract.cu", "eig.cu", "noalloc.cu", "umma_gemm.cu", "fno.cu", "spectrum.cu", "finite_box.cu", "localized.cu", "mixed.cu"]
+SOURCES = ["sbse_api.cu", "tdh_kernels.cu", "fft_fast.cu", "fft_fast64.cu", "fft_more.cu", "fft_split.cu", "fft_few.cu", "contract.cu", "eig.cu", "noalloc.cu", "umma_gemm.cu", "fno.cu", "spectrum.cu", "finite_box.cu", "localized.cu", "mixed.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr",
          "-I", INCLUDE, "-I", CSRC]

@@ -11,7 +11,7 @@
 namespace sbse {
 
 // Sizes with a register FFT, and the offset of each size's twiddle table.
-constexpr int kRegSizes[] = {8, 10, 12, 16, 20, 24, 32, 40, 48, 64, 80, 96};
+constexpr int kRegSizes[] = {8, 10, 12, 16, 18, 20, 24, 25, 27, 30, 32, 36, 40, 45, 48, 50, 54, 60, 64, 80, 96};
 constexpr int kRegCount = sizeof(kRegSizes) / sizeof(int);
 constexpr int reg_offset(int N) {
   int o = 0;

@@ -22,13 +22,32 @@ bool make_tensor_map_f32(CUtensorMap *map, const void *base, int rank, const uin
 
 // ---- register-pencil three-pass round trip (fft_fast.cu), for the sizes fast_supported<T>(N)
 int upload_reg_twiddles();
+int upload_reg_twiddles64();
 // ---- lane-pair split-pencil passes for the grid edges 80 and 96, FP32 (fft_split.cu); the
 // launchers of fft_fast.cu route those sizes here
 bool split_size(int N);
 int upload_split_twiddles();
 void init_split_kernels();
 template <typename T> bool fast_supported(int N);
+template <typename T> bool step_supported(int N);
 template <typename T> void init_fast_kernels();
+// further edges of the same passes (fft_more.cu); mode: PlaneInvMode of fft_pencil.cuh
+bool more_size(int N);
+int upload_more_twiddles();
+template <typename T> void init_more_kernels();
+template <typename T> int more_tiles(int N);
+template <typename T> void launch_more_fwd(const GridTables<T> &g, const XfwdArgs<T> &a, cudaStream_t s);
+template <typename T> void launch_more_z(const GridTables<T> &g, C2<T> *d, int n_items, int mult, cudaStream_t s);
+template <typename T>
+void launch_more_inv(const GridTables<T> &g, C2<T> *d, int n_items, const C2<T> *a_next, int L, T *dens, T *u_out, T *acc,
+                     C2<T> *em1_out, const PoissonOut &po, int mode, cudaStream_t s);
+// ---- Poisson passes with four lanes per pencil, for few packed slots (fft_few.cu)
+int upload_few_twiddles();
+template <typename T> bool few_items(int N, long long n_items);
+template <typename T> void launch_few_fwd(const GridTables<T> &g, const XfwdArgs<T> &a, cudaStream_t s);
+template <typename T> void launch_few_z(const GridTables<T> &g, C2<T> *d, int n_items, int mult, cudaStream_t s);
+template <typename T> void launch_few_inv(const GridTables<T> &g, C2<T> *d, int n_items, const PoissonOut &po, T *u_out,
+                                          T *acc, C2<T> *em1_out, cudaStream_t s);
 
 // ---- FFT passes (tdh_kernels.cu). Items are contiguous arrays of ng complex values.
 template <typename T> void launch_xfwd(const GridTables<T> &g, const XfwdArgs<T> &a, cudaStream_t s);

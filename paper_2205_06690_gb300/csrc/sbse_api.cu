@@ -458,7 +458,11 @@ void round_trip_poisson(sbse_ctx *ctx, const GridTables<T> &g, const XfwdArgs<T>
   cudaStream_t st = ctx->stream;
   C2<T> *pw = fa.out;
   const int S = fa.n_items;
-  if (fast_supported<T>(g.N)) {
+  if (few_items<T>(g.N, S)) {
+    launch_few_fwd<T>(g, fa, st);
+    launch_few_z<T>(g, pw, S, zmult, st);
+    launch_few_inv<T>(g, pw, S, po, u_out, acc, em1_out, st);
+  } else if (fast_supported<T>(g.N)) {
     launch_plane_fwd<T>(g, fa, st);
     launch_zcol<T>(g, pw, S, zmult, st);  // few items: the plain column kernel has more blocks
     launch_plane_inv_poisson<T>(g, pw, S, po, u_out, acc, em1_out, st);
@@ -624,7 +628,7 @@ int run_apply_W(sbse_ctx *ctx, const sbse_tdh_params *p, const std::vector<int> 
   C *acur = a0, *anext = a1;
   // persistent step kernel: dependency-ordered tile queue and completion counters
   // (the persistent step kernel exists for the thread-per-pencil sizes only, not for 80 and 96)
-  const bool persistent = ctx->persistent && fast_supported<T>(ctx->N) && !split_size(ctx->N);
+  const bool persistent = ctx->persistent && step_supported<T>(ctx->N);
   StepQueue sq{};
   int step_grid = 0;
   long long epoch = 0;
@@ -1211,7 +1215,7 @@ int sbse_create(sbse_ctx **out, int device, int precision) {
   sbse::init_fast_kernels<float>();
   sbse::init_fast_kernels<double>();
   sbse::init_split_kernels();
-  if (sbse::upload_reg_twiddles() != 0 || sbse::upload_split_twiddles() != 0) {
+  if (sbse::upload_reg_twiddles() != 0 || sbse::upload_split_twiddles() != 0 || sbse::upload_few_twiddles() != 0) {
     g_create_error = "upload of the FFT twiddle tables failed";
     sbse_destroy(c);
     return SBSE_ERR_CUDA;
@@ -2036,18 +2040,18 @@ int sbse_absorption(sbse_ctx *ctx, int axis, int n_terms, double broadening, int
   const bool launched = launch_absorption(b, phi_o, phi_c, ctx->n_o, ctx->n_c, ctx->N, ctx->h, ctx->box, ctx->dV, ctx->A,
                                           axis, n_terms, broadening, n_omega, ctx->flag, st);
   CHECK_LAUNCH("absorption");
+  if (!launched) return fail(ctx, SBSE_ERR_CUDA, "the Chebyshev recursion could not be launched");
+  int waited = 0;
+  CK(cudaMemcpyAsync(&waited, ctx->flag, sizeof(int), cudaMemcpyDeviceToHost, st));
   CK(cudaMemcpyAsync(sigma, b.sigma, (size_t)n_omega * sizeof(double), cudaMemcpyDeviceToHost, st));
   if (residues)
     CK(cudaMemcpyAsync(residues, b.R, (size_t)n_terms * sizeof(double), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
-  if (!launched) return fail(ctx, SBSE_ERR_CUDA, "the Chebyshev recursion could not be launched");
-  int waited = 0;
-  CK(cudaMemcpyAsync(&waited, ctx->flag, sizeof(int), cudaMemcpyDeviceToHost, st));
+  if (waited) return fail(ctx, SBSE_ERR_DEVICE_TIMEOUT, "a bounded wait of the Chebyshev recursion timed out");
   for (int j = 0; j < n_omega; ++j)
     if (!isfinite(sigma[j])) return fail(ctx, SBSE_ERR_NUMERIC, "spectrum is not finite");
   return SBSE_OK;
 }
-  if (waited) return fail(ctx, SBSE_ERR_DEVICE_TIMEOUT, "a bounded wait of the Chebyshev recursion timed out");
 
 int sbse_set_option(sbse_ctx *ctx, int option, int value) {
   if (!ctx) return SBSE_ERR_INVALID_ARG;

@@ -1,0 +1,255 @@
+"""Kernels at the sizes where they can go wrong: edges of tiles, remainders, the ends of the ranges that
+choose between variants. Against the FP64 oracles, numpy's eigenvalues, or the library's general path.
+
+Tolerances: FP64 results 1e-10 relative (max norm) as everywhere in these tests; the mixed mode's W
+2e-3; eigenvalues 10 n eps |A| (backward stability of the Householder reduction and of the Sturm
+counts); FNO outputs 1e-4 and gradients 2e-3 (FP32 sums of O(B N^3) terms)."""
+import numpy as np
+import pytest
+
+from conftest import rel_err
+from oracle import fno as ofno
+from oracle import mixed, spectrum, tdh
+from test_gpu_fno import _bf16, _pack, _unpack  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    from paper_2205_06690_gb300 import binding
+    binding.load()
+    return binding
+
+
+def _orbitals(N, box, count, seed):
+    """A potential and `count` orthonormal smooth fields (no eigenstates: the kernels need none)."""
+    rng = np.random.default_rng(seed)
+    k = np.fft.fftfreq(N) * N
+    soft = np.exp(-(k[:, None, None] ** 2 + k[None, :, None] ** 2 + k[None, None, :] ** 2) / 9.0)
+    f = np.fft.ifftn(soft * np.fft.fftn(rng.standard_normal((count + 1, N, N, N)), axes=(1, 2, 3)), axes=(1, 2, 3)).real
+    q, _ = np.linalg.qr(f[:count].reshape(count, -1).T)
+    v = -2.0 * np.abs(f[count]) / np.max(np.abs(f[count]))
+    return v, (q.T / (box / N) ** 1.5).reshape(count, N, N, N), np.sort(rng.standard_normal(count))
+
+
+def _apply(B, precision, N, box, v, phi, eps, n_occ, n_o, n_c, prm, pairs, **options):
+    with B.Context(0, precision) as c:
+        for name, value in options.items():
+            B.sbse_set_option(c.h, getattr(B, name), value)
+        c.set_grid(N, box, v)
+        c.set_orbitals(n_occ, n_o, n_c, phi, eps, 0.5)
+        return c.apply_W(prm, pairs, copy_out=True)
+
+
+def _check_w(B, N, n_occ, n_o, pairs, n_s, clean, steps=4):
+    box = 0.4 * N
+    v, phi, eps = _orbitals(N, box, n_occ + 1, N + n_occ)
+    prm = B.TDHParams(n_s=n_s, n_steps=steps, clean_every=clean, dt=0.05, gamma=0.1, alpha=1e-4, seed=5)
+    coeff = tdh.stochastic_coefficients(prm.seed, n_s, n_occ, "gaussian")
+    op = tdh.TDHParams(n_steps=steps, dt=0.05, gamma=0.1, alpha=1e-4, clean_every=clean)
+    ref = tdh.screened_potentials(tdh.Grid(N, box), v, phi, n_occ, n_o, coeff, op, pairs=pairs)
+    ref = np.stack([ref[p].ravel() for p in pairs])
+    assert rel_err(_apply(B, B.SBSE_FP64, N, box, v, phi, eps, n_occ, n_o, 1, prm, pairs), ref) < 1e-10
+    assert rel_err(_apply(B, B.SBSE_MIXED, N, box, v, phi, eps, n_occ, n_o, 1, prm, pairs), ref) < 2e-3
+
+
+@pytest.mark.parametrize("N", [18, 25, 27, 30, 36, 45, 50, 54, 60])
+def test_further_grid_edges_match_oracle(B, N):
+    """Odd pair count (the last Poisson slot packs one density), cleaning inside the run."""
+    _check_w(B, N, 3, 2, [(0, 0), (0, 1), (1, 1)], 3, 2)
+
+
+@pytest.mark.parametrize("n_occ,n_pairs,n_s", [(1, 1, 1), (4, 1, 3), (5, 3, 3), (64, 3, 5), (67, 6, 3)])
+def test_fp64_cleaning_edges_match_oracle(B, n_occ, n_pairs, n_s):
+    """Occupied counts and columns around the 4 x 4 overlap tiles, the 8 columns and 64 states of the
+    update; 10^3 points leave the last chunk and the last tile of 128 points partly filled."""
+    n_o = 1 if n_pairs == 1 else 3
+    _check_w(B, 10, n_occ, n_o, tdh.pair_list(n_o)[:n_pairs], n_s, 1)
+
+
+@pytest.mark.parametrize("N,n_o,count", [(16, 1, 1), (16, 4, 10), (32, 2, 3), (32, 5, 15), (40, 2, 3), (48, 1, 1),
+                                         (48, 4, 9), (64, 2, 3)])
+def test_bare_potentials_of_few_and_many_slots(B, N, n_o, count):
+    """Both sides of the rule that gives a pencil four lanes (FP64, in the init; the slots of FP32 in
+    one propagation step)."""
+    box = 0.3 * N
+    v, phi, eps = _orbitals(N, box, n_o + 1, N)
+    pairs = tdh.pair_list(n_o)[:count]
+    ref = np.stack([tdh.coulomb_periodic(phi[i] * phi[j], tdh.Grid(N, box)).ravel() for i, j in pairs])
+    with B.Context(0, B.SBSE_FP64) as c:
+        c.set_grid(N, box, v)
+        c.set_orbitals(n_o, n_o, 1, phi, eps, 0.5)
+        B.sbse_bare_W(c.h, pairs)
+        assert rel_err(B.sbse_get_W(c.h, pairs, N ** 3), ref) < 1e-10
+    prm = B.TDHParams(n_s=2, n_steps=1, clean_every=0, dt=0.05, gamma=0.1, alpha=1e-4, seed=1)
+    coeff = tdh.stochastic_coefficients(1, 2, n_o, "gaussian")
+    op = tdh.TDHParams(n_steps=1, dt=0.05, gamma=0.1, alpha=1e-4, clean_every=0)
+    w = tdh.screened_potentials(tdh.Grid(N, box), v, phi, n_o, n_o, coeff, op, pairs=pairs[:1])
+    for prec, tol in ((B.SBSE_FP64, 1e-10), (B.SBSE_MIXED, 2e-3)):
+        assert rel_err(_apply(B, prec, N, box, v, phi, eps, n_o, n_o, 1, prm, pairs)[0], w[pairs[0]].ravel()) < tol
+
+
+def _eig_noalloc(B, a, k):
+    torch = pytest.importorskip("torch")
+    d, ev = torch.from_numpy(np.ascontiguousarray(a)).cuda(), torch.empty(k, dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    B.sbse_spectrum_noalloc(d.data_ptr(), a.shape[0], k, ev.data_ptr(), 0)
+    return ev.cpu().numpy()
+
+
+def _sym(n, kind):
+    rng = np.random.default_rng(n)
+    a = rng.standard_normal((n, n))
+    a = 0.5 * (a + a.T)
+    if kind == "diagonal":
+        a = np.diag(np.diag(a))
+    elif kind == "blocks":  # decoupled halves, one of them a multiple of the identity
+        h = n // 2
+        a[:h, h:] = a[h:, :h] = 0.0
+        a[h:, h:] = 0.25 * np.eye(n - h)
+    elif kind == "zero":
+        a[:] = 0.0
+    elif kind == "large":
+        a *= 1e150
+    elif kind == "small":
+        a *= 1e-150
+    return a
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 4, 7, 15, 16, 17, 31, 33, 64, 100, 127, 128, 129, 255, 257, 512])
+@pytest.mark.parametrize("kind", ["dense", "blocks"])
+def test_eigenvalues_at_cluster_edges(B, n, kind):
+    a = _sym(n, kind)
+    k = min(n, 12)
+    ref = np.linalg.eigvalsh(a)
+    assert np.max(np.abs(_eig_noalloc(B, a, k) - ref[:k])) <= 10 * n * 2.2e-16 * max(1e-300, np.max(np.abs(ref)))
+
+
+@pytest.mark.parametrize("kind", ["diagonal", "zero", "large", "small"])
+def test_eigenvalues_of_special_matrices(B, kind):
+    a = _sym(40, kind)
+    ref = np.linalg.eigvalsh(a)
+    assert np.max(np.abs(_eig_noalloc(B, a, 40) - ref)) <= 10 * 40 * 2.2e-16 * max(1e-11, np.max(np.abs(ref)))
+
+
+@pytest.fixture(scope="module")
+def wide(B):
+    """An exchange-only A of 24 x 28 = 672 rows on 16^3: beyond the shared memory of the eigensolver's
+    cluster, and more rows than four per SM for the spectrum."""
+    N, box, n_o, n_c = 16, 8.0, 24, 28
+    v, phi, eps = _orbitals(N, box, n_o + n_c, 2)
+    c = B.Context(0, B.SBSE_FP64)
+    c.set_grid(N, box, v)
+    c.set_orbitals(n_o, n_o, n_c, phi, eps, 0.5)
+    A = c.build_A(B.SBSE_EXCHANGE)
+    yield c, A, phi, N, box, n_o, n_c
+    c.close()
+
+
+def test_eigenvalues_and_vectors_beyond_shared_memory(B, wide):
+    c, A, n = wide[0], wide[1], wide[1].shape[0]
+    ref = np.linalg.eigvalsh(0.5 * (A + A.T))
+    tol = 10 * n * 2.2e-16 * np.max(np.abs(ref))
+    assert np.max(np.abs(c.spectrum(6) - ref[:6])) <= tol
+    ev, X = c.spectrum(6, vectors=True)
+    assert np.max(np.abs(ev - ref[:6])) <= tol
+    assert np.max(np.abs(A @ X - X * ev)) <= 1e-9 * np.max(np.abs(ref)) and np.max(np.abs(X.T @ X - np.eye(6))) <= 1e-9
+
+
+def _chebyshev(A, f0, K, s, omega):
+    c, w = spectrum.scaling(A)
+    R = spectrum.residues(A, f0, K)
+    return spectrum.sigma_chebyshev(R, c, w, omega, s), R
+
+
+def test_absorption_of_wide_matrix(B, wide):
+    c, A, phi, N, box, n_o, n_c = wide
+    f0 = spectrum.dipoles(tdh.Grid(N, box), phi[:n_o], phi[n_o:], 1)
+    omega = np.linspace(0.1, 4.0, 37)
+    ref, R = _chebyshev(A, f0, 65, 0.1, omega)
+    sig, res = c.absorption(1, 65, 0.1, omega)
+    assert rel_err(res, R) < 1e-8 and rel_err(sig, ref) < 1e-8
+
+
+@pytest.mark.parametrize("n_o,n_c,terms", [(1, 1, 2), (1, 3, 3), (3, 11, 64), (5, 13, 257)])
+def test_absorption_of_small_matrices(B, n_o, n_c, terms):
+    """One block, a row count that is no multiple of a warp's or block's rows, few terms."""
+    N, box = 10, 6.0
+    v, phi, eps = _orbitals(N, box, n_o + n_c, n_o)
+    omega = np.linspace(0.1, 4.0, 5)
+    with B.Context(0, B.SBSE_FP64) as c:
+        c.set_grid(N, box, v)
+        c.set_orbitals(n_o, n_o, n_c, phi, eps, 0.5)
+        A = c.build_A(B.SBSE_EXCHANGE)
+        if n_o * n_c == 1:  # Gershgorin discs of one row leave no interval to scale
+            return
+        sig, res = c.absorption(0, terms, 0.2, omega)
+    f0 = spectrum.dipoles(tdh.Grid(N, box), phi[:n_o], phi[n_o:], 0)
+    ref, R = _chebyshev(A, f0, terms, 0.2, omega)
+    assert rel_err(res, R) < 1e-8 and rel_err(sig, ref) < 1e-8
+
+
+@pytest.mark.parametrize("n_occ,n_o,n_c", [(1, 1, 1), (7, 4, 9), (9, 5, 8), (33, 3, 2)])
+def test_hole_grid_projections(B, n_occ, n_o, n_c):
+    """Window and basis counts around the 4 x 8 tiles; a basis of fewer rows takes more chunks."""
+    N, box = 10, 5.0
+    v, phi, eps = _orbitals(N, box, n_occ + n_c, n_occ)
+    g = tdh.Grid(N, box)
+    po = phi[n_occ - n_o:n_occ]
+    W = {(i, j): tdh.coulomb_periodic(po[i] * po[j], g) for i, j in tdh.pair_list(n_o)}
+    f = np.random.default_rng(1).standard_normal((n_o, N, N, N))
+    with B.Context(0, B.SBSE_FP64) as c:
+        c.set_grid(N, box, v)
+        c.set_orbitals(n_occ, n_o, n_c, phi, eps, 0.5)
+        B.sbse_bare_W(c.h, tdh.pair_list(n_o))
+        for proj, cond in ((B.SBSE_Q_OCCUPIED, False), (B.SBSE_Q_CONDUCTION, True)):
+            op = mixed.MixedA(g, v, phi, eps, n_occ, n_o, n_c, W, 0.5, conduction_only=cond)
+            fq = op.Q(f)
+            got = B.sbse_apply_A_mixed(c.h, proj, fq.reshape(n_o, -1)).reshape(fq.shape)
+            assert rel_err(got, op(fq)) < 1e-10
+
+
+@pytest.mark.parametrize("N,C,m,L,batch", [(9, 5, 4, 2, 2), (10, 33, 5, 2, 1), (13, 3, 6, 1, 9), (8, 64, 2, 2, 11),
+                                           (70, 2, 3, 1, 1)])
+def test_fno_edges_match_oracle(B, N, C, m, L, batch):
+    """Odd grids, every mode kept, channel counts off the compiled ones, batches beyond the mix's
+    registers and shared memory, planes of more rows than one tile."""
+    torch = pytest.importorskip("torch")
+    net = B.FNO(N, width=C, modes=m, layers=L, max_batch=batch)
+    vec = _pack(ofno.init_params(C, m, L, seed=N))
+    net.set_params(vec)
+    pr = _unpack(vec, C, m, L, round_bf16=True)
+    rng = np.random.default_rng(1)
+    x = rng.standard_normal((batch, 2, N, N, N)).astype(np.float32)
+    dy = rng.standard_normal((batch, N, N, N)).astype(np.float32)
+    xd, dyd = torch.from_numpy(x).cuda(), torch.from_numpy(dy).cuda()
+    yd = torch.empty((batch, N, N, N), dtype=torch.float32, device="cuda")
+    torch.cuda.synchronize()
+    net.forward(batch, xd.data_ptr(), yd.data_ptr())
+    y, cache = ofno.forward(pr, x.astype(np.float64), m, keep=True)
+    assert rel_err(yd.cpu().numpy(), y) < 1e-4
+    net.gradients(batch, xd.data_ptr(), dyd.data_ptr())
+    gp, ref = _unpack(net.get_params()[1], C, m, L), ofno.backward(pr, cache, dy.astype(np.float64), m)
+    for name in ("lift_w", "lift_b", "proj_w"):
+        assert rel_err(getattr(gp, name), ref[name]) < 2e-3
+    assert abs(gp.proj_b - ref["proj_b"]) < 2e-3 * max(1.0, abs(ref["proj_b"]))
+    for name in ("pw_w", "pw_b", "spec"):
+        for a, b in zip(getattr(gp, name), ref[name]):
+            assert rel_err(a, b) < 2e-3
+    net.close()
+
+
+def test_fno_planes_beyond_shared_memory(B):
+    """Planes whose folded transforms do not fit take the direct sums: forward only, one channel."""
+    torch = pytest.importorskip("torch")
+    N, C, m, L = 168, 1, 84, 1
+    net = B.FNO(N, width=C, modes=m, layers=L, max_batch=1)
+    vec = _pack(ofno.init_params(C, m, L, seed=1))
+    net.set_params(vec)
+    x = np.random.default_rng(1).standard_normal((1, 2, N, N, N)).astype(np.float32)
+    xd, yd = torch.from_numpy(x).cuda(), torch.empty((1, N, N, N), dtype=torch.float32, device="cuda")
+    torch.cuda.synchronize()
+    net.forward(1, xd.data_ptr(), yd.data_ptr())
+    assert rel_err(yd.cpu().numpy(), ofno.forward(_unpack(vec, C, m, L, round_bf16=True), x.astype(np.float64), m)) < 1e-4
+    net.close()
