@@ -212,8 +212,9 @@ class ClockSampler:
 # the sources the pass kernels of each workload are compiled from (their definitions and the data
 # structures they read; declarations of other launchers do not enter)
 KERNEL_SOURCES = {
-    "large96": ["fft_split.cu", "fft_reg.cuh", "passes.cuh", "common.cuh", "tables.cuh"],
-    "default": ["fft_fast.cu", "fft_reg.cuh", "passes.cuh", "tma.cuh", "common.cuh", "tables.cuh"],
+    "large96": ["fft_split.cu", "fft_pair.cuh", "fft_reg.cuh", "passes.cuh", "common.cuh", "tables.cuh"],
+    "default": ["fft_split.cu", "fft_pair.cuh", "fft_fast.cu", "fft_fast.cuh", "fft_pencil.cuh", "fft_few.cu",
+                "fft_reg.cuh", "passes.cuh", "tma.cuh", "common.cuh", "tables.cuh"],
 }
 
 
@@ -786,22 +787,24 @@ def main():
 
     # Roofline. Algorithmic unit: one read and one write of every complex value of the propagated
     # block (blk L n_g points, 16 B/point in FP32). Each pass of a TDH step (phases 5, 6, 7, timed by
-    # events on the library's stream; two passes on the 80/96 grids, three elsewhere) is one such
+    # events on the library's stream; two passes in the mixed mode, three in FP64) is one such
     # sweep; the dominant kernel is the pass with the largest share. The whole propagation step
     # (phase 0) is reported against the same per-step figure, so its fraction shows the cost of
     # several sweeps per step.
     peak, src = measured_peaks()
     csize = 8 if prec == B.SBSE_MIXED else 16
     sweep_bytes = blk * pre.n_s * pre.N ** 3 * 2 * csize
-    split = pre.N in (80, 96)
-    if split:  # two sweeps per step: the kinetic propagator as three one-dimensional operators
-        pass_names = {5: "plane kinetic pass k_plane_kin2 (potential phase + x, y kinetic operators)",
-                      7: "z kinetic pass k_zkin2_tma (z kinetic operator + induced density; columns "
-                         "staged by tensor copies)"}
+    pair = pre.N in (32, 48, 64, 80, 96)
+    if prec == B.SBSE_MIXED:  # two sweeps per step: the kinetic propagator as three one-dimensional operators
+        pass_names = {5: f"plane kinetic pass {'k_plane_kin2' if pair else 'k_plane_kin'} (potential phase + x, y "
+                         "kinetic operators)",
+                      7: "z kinetic pass " + ("k_zkin2_tma (z kinetic operator + induced density; columns staged by "
+                                              "tensor copies)" if pair else
+                                              "k_zkin (z kinetic operator + induced density)")}
     else:
         pass_names = {5: "forward plane pass k_plane_fwd (potential phase + x, y FFTs)",
-                      6: "z-column pass k_zcol_tma (z FFT, kinetic phase, inverse z FFT)",
-                      7: "inverse plane pass k_plane_inv_density_tma (y, x inverse FFTs + density)"}
+                      6: "z-column pass k_zcol (z FFT, kinetic phase, inverse z FFT)",
+                      7: "inverse plane pass k_plane_inv (y, x inverse FFTs) and k_density"}
     passes = {}
     for ph, name in pass_names.items():
         t, nl = phase[ph]

@@ -298,10 +298,9 @@ int sbse_get_stream(const sbse_ctx *ctx, void **stream);
  * register-pencil FFT); 0 uses three separate pass kernels, which are faster on GB300 (the merged
  * kernel is register-limited to fewer resident warps). Results do not depend on it. */
 #define SBSE_OPT_PERSISTENT 3
-/* SBSE_OPT_TMA_PLANES (default 1): in SBSE_MIXED on grids of 32, 40, 48 or 64 points per axis, the
- * inverse plane pass of the pair batch (with the induced density of Eq. 11) and the z-column passes
- * run as persistent kernels fed by bulk asynchronous copies (TMA) of their next planes or column
- * slabs; 0 uses the plain pass kernels. Results do not depend on it. */
+/* SBSE_OPT_TMA_PLANES (default 1): in SBSE_MIXED on grids of 32, 48, 64, 80 or 96 points per axis, the
+ * z sweep of a large pair batch (with the induced density of Eq. 11) is fed by bulk asynchronous
+ * copies (TMA) of its next column slab; 0 uses plain loads. Results do not depend on it. */
 #define SBSE_OPT_TMA_PLANES 4
 /* SBSE_OPT_GRAPH (default 1): sbse_apply_W captures its time loop (all launches of all steps, on
  * the context's two streams) into a CUDA graph and replays it on later calls whose buffers, sizes,

@@ -49,7 +49,7 @@ def _variants(n: int, precision: int, pair_bytes: float):
     chunks = [c for c in _CHUNKS_MB if c == 0 or pair_bytes > c * 2 ** 20]
     if n in (80, 96) and precision == B.SBSE_MIXED:
         return [(0, 1, c) for c in chunks]  # the two-sweep passes
-    tma = [0, 1] if (precision == B.SBSE_MIXED and n in (32, 40, 48, 64)) else [1]
+    tma = [0, 1] if (precision == B.SBSE_MIXED and n in (32, 48, 64)) else [1]
     out = []
     for p in (0, 1):
         for t in tma:

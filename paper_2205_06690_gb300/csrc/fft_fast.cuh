@@ -67,108 +67,74 @@ template <typename T> void init_fast_kernels() {
 }
 
 template <typename T> void launch_plane_fwd(const GridTables<T> &g, const XfwdArgs<T> &a, cudaStream_t s) {
+  count_launch(1);
   if constexpr (sizeof(T) == 4) {
     if (split_size(g.N)) {
       launch_plane_fwd2(g, a, s);
-      count_launch(1);
       return;
     }
   }
   if (more_size(g.N)) {
     launch_more_fwd<T>(g, a, s);
-    count_launch(1);
     return;
   }
 #define SBSE_CALL(n) FastOps<T>::template fwd<n>(g, a, s)
   SBSE_FAST_SWITCH(g.N, SBSE_CALL)
 #undef SBSE_CALL
-  count_launch(1);
 }
 
-template <typename T>
-void launch_zcol(const GridTables<T> &g, C2<T> *d, int n_items, int mult, cudaStream_t s, int *tma_err) {
+template <typename T> void launch_zcol(const GridTables<T> &g, C2<T> *d, int n_items, int mult, cudaStream_t s) {
+  count_launch(1);
   if constexpr (sizeof(T) == 4) {
     if (split_size(g.N)) {
       launch_zcol2(g, d, n_items, mult, s);
-      count_launch(1);
       return;
-    }
-    if (tma_err) {
-      bool done = false;
-#define SBSE_CALL(n) done = zcol_tma<n>(g, d, n_items, mult, tma_err, s)
-      SBSE_FAST_SWITCH(g.N, SBSE_CALL)
-#undef SBSE_CALL
-      if (done) {
-        count_launch(1);
-        return;
-      }
     }
   }
   if (more_size(g.N)) {
     launch_more_z<T>(g, d, n_items, mult, s);
-    count_launch(1);
     return;
   }
 #define SBSE_CALL(n) FastOps<T>::template z<n>(g, d, n_items, mult, s)
   SBSE_FAST_SWITCH(g.N, SBSE_CALL)
 #undef SBSE_CALL
-  count_launch(1);
 }
 
 template <typename T>
 void launch_plane_inv_orb(const GridTables<T> &g, C2<T> *d, int n_items, const C2<T> *a_next, int L,
-                          T *dens, cudaStream_t s, int *tma_err) {
-  if constexpr (sizeof(T) == 4) {
-    if (dens && tma_err) {
-      bool done = false;
-#define SBSE_CALL(n) done = inv_density_tma<n>(g, d, n_items, a_next, L, dens, tma_err, s)
-      SBSE_FAST_SWITCH(g.N, SBSE_CALL)
-#undef SBSE_CALL
-      if (done) {
-        count_launch(1);
-        return;
-      }
-    }
-  }
-  // The density summed in the inverse pass needs one block per pair and plane group, working through the
-  // pair's L orbitals in turn, and N more registers. In FP64 (its registers spill, and the narrow FP64
-  // pipe of every SM must be kept fed) and where those blocks are few, the pass stores the orbitals and
-  // a second kernel sums the density in the same order: 3 pairs on 16^3 in FP64, 318 -> 16 + 5 us;
-  // 10 pairs on 40^3, 918 -> 560 + 73 us.
-  const int tiles = more_size(g.N) ? more_tiles<T>(g.N) : step_tiles_per_orbital<T>(g.N);
-  const bool split = dens && (sizeof(T) == 8 || (long long)(n_items / L) * tiles < 4 * kFewBlocks);
-  const int mode = dens && !split ? PI_DENSITY : PI_PLAIN;
+                          T *dens, cudaStream_t s) {
+  // A second kernel sums the density from the stored orbitals: in the inverse pass it needs one block per
+  // pair and plane group working through the pair's L orbitals in turn, and N more registers, which spill
+  // in FP64. 3 pairs on 16^3: 318 -> 16 + 5 us; 10 pairs on 40^3, 918 -> 560 + 73 us.
   const PoissonOut po{0, 0.0, 0.0, 0.0};
+  count_launch(1);
   if (more_size(g.N)) {
-    launch_more_inv<T>(g, d, n_items, a_next, L, dens, nullptr, nullptr, nullptr, po, mode, s);
+    launch_more_inv<T>(g, d, n_items, nullptr, nullptr, nullptr, po, PI_PLAIN, s);
   } else {
-#define SBSE_CALL(n) FastOps<T>::template inv<n>(g, d, n_items, a_next, L, dens, nullptr, nullptr, nullptr, po, mode, s)
+#define SBSE_CALL(n) FastOps<T>::template inv<n>(g, d, n_items, nullptr, nullptr, nullptr, po, PI_PLAIN, s)
     SBSE_FAST_SWITCH(g.N, SBSE_CALL)
 #undef SBSE_CALL
   }
-  count_launch(1);
-  if (split) launch_density<T>(g, d, a_next, n_items / L, L, dens, s);
+  if (dens) launch_density<T>(g, d, a_next, n_items / L, L, dens, s);
 }
 
 template <typename T>
 void launch_plane_inv_poisson(const GridTables<T> &g, C2<T> *d, int n_slots, const PoissonOut &po,
                               T *u_out, T *acc, C2<T> *em1_out, cudaStream_t s) {
+  count_launch(1);
   if constexpr (sizeof(T) == 4) {
     if (split_size(g.N)) {
       launch_plane_inv2_poisson(g, d, n_slots, po, u_out, acc, em1_out, s);
-      count_launch(1);
       return;
     }
   }
   if (more_size(g.N)) {
-    launch_more_inv<T>(g, d, n_slots, nullptr, 1, nullptr, u_out, acc, em1_out, po, PI_POISSON, s);
-    count_launch(1);
+    launch_more_inv<T>(g, d, n_slots, u_out, acc, em1_out, po, PI_POISSON, s);
     return;
   }
-#define SBSE_CALL(n) FastOps<T>::template inv<n>(g, d, n_slots, nullptr, 1, nullptr, u_out, acc, em1_out, po, PI_POISSON, s)
+#define SBSE_CALL(n) FastOps<T>::template inv<n>(g, d, n_slots, u_out, acc, em1_out, po, PI_POISSON, s)
   SBSE_FAST_SWITCH(g.N, SBSE_CALL)
 #undef SBSE_CALL
-  count_launch(1);
 }
 
 // grids of the persistent step kernel
@@ -184,9 +150,7 @@ template <typename T> bool step_supported(int N) { return fast_supported<T>(N) &
   template bool fast_supported<T>(int);                                                            \
   template void init_fast_kernels<T>();                                                            \
   template void launch_plane_fwd<T>(const GridTables<T> &, const XfwdArgs<T> &, cudaStream_t);     \
-  template void launch_zcol<T>(const GridTables<T> &, C2<T> *, int, int, cudaStream_t, int *);     \
-  template void launch_plane_inv_orb<T>(const GridTables<T> &, C2<T> *, int, const C2<T> *, int,   \
-                                        T *, cudaStream_t, int *);                                 \
+  template void launch_zcol<T>(const GridTables<T> &, C2<T> *, int, int, cudaStream_t);            \
   template void launch_plane_inv_poisson<T>(const GridTables<T> &, C2<T> *, int, const PoissonOut &, \
                                             T *, T *, C2<T> *, cudaStream_t);
 

@@ -39,14 +39,6 @@ template <typename T> void init_more_kernels() {
 #undef SBSE_ATTR
 }
 
-template <typename T> int more_tiles(int N) {
-  int r = 0;
-#define SBSE_CALL(n) r = FastOps<T>::template tiles_per_orbital<n>()
-  SBSE_MORE_SWITCH(N, SBSE_CALL)
-#undef SBSE_CALL
-  return r;
-}
-
 template <typename T> void launch_more_fwd(const GridTables<T> &g, const XfwdArgs<T> &a, cudaStream_t s) {
 #define SBSE_CALL(n) FastOps<T>::template fwd<n>(g, a, s)
   SBSE_MORE_SWITCH(g.N, SBSE_CALL)
@@ -60,20 +52,32 @@ template <typename T> void launch_more_z(const GridTables<T> &g, C2<T> *d, int n
 }
 
 template <typename T>
-void launch_more_inv(const GridTables<T> &g, C2<T> *d, int n_items, const C2<T> *a_next, int L, T *dens, T *u_out, T *acc,
-                     C2<T> *em1_out, const PoissonOut &po, int mode, cudaStream_t s) {
-#define SBSE_CALL(n) FastOps<T>::template inv<n>(g, d, n_items, a_next, L, dens, u_out, acc, em1_out, po, mode, s)
+void launch_more_inv(const GridTables<T> &g, C2<T> *d, int n_items, T *u_out, T *acc, C2<T> *em1_out, const PoissonOut &po,
+                     int mode, cudaStream_t s) {
+#define SBSE_CALL(n) FastOps<T>::template inv<n>(g, d, n_items, u_out, acc, em1_out, po, mode, s)
+  SBSE_MORE_SWITCH(g.N, SBSE_CALL)
+#undef SBSE_CALL
+}
+
+void launch_more_kin(const GridTables<float> &g, const XfwdArgs<float> &a, cudaStream_t s) {
+#define SBSE_CALL(n) FastOps<float>::kin<n>(g, a, s)
+  SBSE_MORE_SWITCH(g.N, SBSE_CALL)
+#undef SBSE_CALL
+}
+
+void launch_more_zkin(const GridTables<float> &g, float2 *d, int n_items, const float2 *a_next, int L, float *dens,
+                      cudaStream_t s) {
+#define SBSE_CALL(n) FastOps<float>::zkin<n>(g, d, n_items, a_next, L, dens, s)
   SBSE_MORE_SWITCH(g.N, SBSE_CALL)
 #undef SBSE_CALL
 }
 
 #define SBSE_MORE_INST(T)                                                                                        \
   template void init_more_kernels<T>();                                                                          \
-  template int more_tiles<T>(int);                                                                               \
   template void launch_more_fwd<T>(const GridTables<T> &, const XfwdArgs<T> &, cudaStream_t);                    \
   template void launch_more_z<T>(const GridTables<T> &, C2<T> *, int, int, cudaStream_t);                        \
-  template void launch_more_inv<T>(const GridTables<T> &, C2<T> *, int, const C2<T> *, int, T *, T *, T *, C2<T> *, \
-                                   const PoissonOut &, int, cudaStream_t);
+  template void launch_more_inv<T>(const GridTables<T> &, C2<T> *, int, T *, T *, C2<T> *, const PoissonOut &, int, \
+                                   cudaStream_t);
 SBSE_MORE_INST(float)
 SBSE_MORE_INST(double)
 

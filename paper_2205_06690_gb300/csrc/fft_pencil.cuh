@@ -18,11 +18,7 @@
 
 #include <type_traits>
 
-#include "fft_reg.cuh"
-#include "bounds.cuh"
-#include "kernels.h"
-#include "passes.cuh"
-#include "tma.cuh"
+#include "fft_pair.cuh"
 
 namespace sbse {
 
@@ -78,11 +74,25 @@ template <typename T, int N> constexpr size_t plane_smem() {
 
 // ------------------------------------------------------------------------------------------
 
-// forward x and y FFTs of the PPB planes starting at plane offset `off` (= z0 N^2) of `item`, with
-// the fused pre-operation; S is the block's shared tile
-template <typename T, int N, bool PAIR, int PPB = kPPB<T, N>>
+// One-dimensional kinetic operator F^-1 diag(kt) F of a pencil in registers (kt = kin / N)
+template <int N> __device__ __forceinline__ void kin_pencil(float2 (&v)[N], const float2 *kt) {
+  fft_reg<float, N, -1, TwP<float>>(v);
+#pragma unroll
+  for (int k = 0; k < N; ++k) v[k] = cmul(v[k], kt[k]);
+  fft_reg<float, N, +1, TwP<float>>(v);
+}
+// kt of the block, K / N rounded once (a rounded 1 / N would scale every transform of every step by the same
+// error); the caller synchronises
+template <int N> __device__ __forceinline__ void load_kin(float2 *kt, const GView<float> &g) {
+  for (int i = threadIdx.x; i < N; i += blockDim.x) kt[i] = g.kin[N + 3 * (N / 2) + i];
+}
+
+// The PPB planes starting at plane offset `off` (= z0 N^2) of `item`: the fused pre-operation, then the
+// forward x and y FFTs, or with KIN (FP32 orbitals) the x and y kinetic operators; S is the block's
+// shared tile
+template <typename T, int N, bool PAIR, int PPB = kPPB<T, N>, bool KIN = false>
 __device__ __forceinline__ void fwd_planes(const GView<T> &g, const XfwdArgs<T> &a, long long item,
-                                           long long off, C2<T> *S) {
+                                           long long off, C2<T> *S, const C2<T> *kt = nullptr) {
   using C = C2<T>;
   constexpr int LD = N + 1, NN = N * N, NT = PPB * N;
   const PreopItem<T> it = preop_item<T>(g, a, item);
@@ -166,7 +176,10 @@ __device__ __forceinline__ void fwd_planes(const GView<T> &g, const XfwdArgs<T> 
     C *row = S + (pl * N + q) * LD;
 #pragma unroll
     for (int x = 0; x < N; ++x) v[x] = row[x];
-    fft_reg<T, N, -1, TwP<T>>(v);
+    if constexpr (KIN)
+      kin_pencil<N>(v, kt);
+    else
+      fft_reg<T, N, -1, TwP<T>>(v);
 #pragma unroll
     for (int x = 0; x < N; ++x) row[x] = v[x];
   }
@@ -176,7 +189,10 @@ __device__ __forceinline__ void fwd_planes(const GView<T> &g, const XfwdArgs<T> 
     const C *col = S + pl * N * LD + q;
 #pragma unroll
     for (int y = 0; y < N; ++y) v[y] = col[y * LD];
-    fft_reg<T, N, -1, TwP<T>>(v);
+    if constexpr (KIN)
+      kin_pencil<N>(v, kt);
+    else
+      fft_reg<T, N, -1, TwP<T>>(v);
     C *out = a.out + item * g.ng + off + pl * NN + q;
 #pragma unroll
     for (int y = 0; y < N; ++y) out[y * N] = v[y];
@@ -224,6 +240,80 @@ __global__ void __launch_bounds__(PPB * N) k_plane_fwd(GView<T> g, XfwdArgs<T> a
   fwd_planes<T, N, PAIR, PPB>(g, a, item, (p0 - item * N) * NN, reinterpret_cast<C2<T> *>(smem_raw));
 }
 
+// First sweep of the two-sweep split-operator step of the FP32 orbitals: the kinetic propagator is the
+// product of one operator per axis, so the planes take the potential phase and the x and y operators, and
+// the second sweep (k_zkin) the z operator. Two sweeps over the orbitals instead of the three of a 3D
+// round trip. 15 pairs of 45^3: planes 82 us, z 14.5 us and density 13.6 us; the whole W 12.0 ms (three
+// sweeps: 12.4 ms). Grids with lane-pair pencils (fft_split.cu) take theirs.
+template <int N, bool PAIR, int PPB>
+__global__ void __launch_bounds__(PPB * N) k_plane_kin(GView<float> g, XfwdArgs<float> a, long long planes_total) {
+  constexpr int NN = N * N;
+  extern __shared__ unsigned char smem_raw[];
+  __shared__ float2 kt[N];
+  load_kin<N>(kt, g);  // (read after the pre-operation's barrier)
+  const long long p0 = (long long)blockIdx.x * PPB;
+  const long long item = p0 / N;
+  (void)SBSE_IDX(p0 + PPB - 1, planes_total);
+  (void)SBSE_IDX(item, a.n_items);
+  fwd_planes<float, N, PAIR, PPB, true>(g, a, item, (p0 - item * N) * NN, reinterpret_cast<float2 *>(smem_raw), kt);
+}
+
+// the density of a column of one orbital added to acc[z * stride] (first: assigned), eta0 loaded in batches
+template <int N, bool COH>
+__device__ __forceinline__ void add_density(const float2 (&v)[N], const float2 *ab, float *acc, int stride, bool first) {
+  constexpr int UB = 16, NN = N * N;
+#pragma unroll
+  for (int z0 = 0; z0 < N; z0 += UB) {
+    float2 a0[UB];
+#pragma unroll
+    for (int k = 0; k < UB; ++k)
+      if (z0 + k < N) a0[k] = ldv<COH>(ab + (long long)(z0 + k) * NN);
+#pragma unroll
+    for (int k = 0; k < UB; ++k)
+      if (z0 + k < N) {
+        const float t = density_term<float>(a0[k], v[z0 + k]);
+        float &d = acc[(z0 + k) * stride];
+        d = first ? t : d + t;
+      }
+    asm volatile("" ::: "memory");  // keep the next batch's loads below this one (registers)
+  }
+}
+
+// Second sweep: the z kinetic operator, a thread per (x, y) column. DENS: of each of the L orbitals of a pair
+// (unit), summing the pair's induced density in shared memory.
+constexpr int kZkT = 128;
+template <int N, bool DENS>
+__global__ void __launch_bounds__(kZkT)
+    k_zkin(GView<float> g, float2 *data, const float2 *a_next, float *dens, int n_units, int L) {
+  using C = float2;
+  constexpr int NN = N * N;
+  __shared__ C kt[N];
+  __shared__ float D[DENS ? N * kZkT : 1];
+  load_kin<N>(kt, g);
+  __syncthreads();
+  const long long cols = (NN + blockDim.x - 1) / blockDim.x;  // blocks per unit
+  const long long unit = blockIdx.x / cols;
+  const int rem = (int)(blockIdx.x - unit * cols) * blockDim.x + threadIdx.x;
+  if (rem >= NN) return;
+  (void)SBSE_IDX(unit, n_units);
+  const int n_orb = DENS ? L : 1;
+  for (int ell = 0; ell < n_orb; ++ell) {
+    C *base = data + (unit * n_orb + ell) * g.ng + rem;
+    C v[N];
+#pragma unroll
+    for (int z = 0; z < N; ++z) v[z] = base[(long long)z * NN];
+    kin_pencil<N>(v, kt);
+#pragma unroll
+    for (int z = 0; z < N; ++z) base[(long long)z * NN] = v[z];
+    if constexpr (DENS) add_density<N, false>(v, a_next + (long long)ell * g.ng + rem, D + threadIdx.x, kZkT, ell == 0);
+  }
+  if constexpr (DENS) {
+    float *db = dens + unit * g.ng + rem;
+#pragma unroll 8
+    for (int z = 0; z < N; ++z) db[(long long)z * NN] = D[z * kZkT + threadIdx.x];
+  }
+}
+
 // one (x, y) column of one item: forward z FFT, multiplier, inverse z FFT (thread per column)
 template <typename T, int N, bool COH>
 __device__ __forceinline__ void zcol_column(const GView<T> &g, C2<T> *data, long long item, int rem,
@@ -267,11 +357,10 @@ __global__ void __launch_bounds__(128) k_zcol(GView<T> g, C2<T> *data, long long
   zcol_column<T, N, false>(g, data, item, (int)(c - item * NN), mult);
 }
 
-enum PlaneInvMode { PI_PLAIN = 0, PI_DENSITY = 1, PI_POISSON = 2 };
+enum PlaneInvMode { PI_PLAIN = 0, PI_POISSON = 1 };
 
 struct PlaneInvArgs {
-  long long planes_total;  // PLAIN, POISSON: planes of all items
-  int L;                   // DENSITY: orbitals per pair
+  long long planes_total;  // planes of all items
   PoissonOut po;           // POISSON
 };
 
@@ -326,7 +415,7 @@ __device__ __forceinline__ void inv_density_planes(const GView<T> &g, C2<T> *dat
       const C dv = S[(threadIdx.x / N) * LD + threadIdx.x % N + k * PPB * LD];
       base[l] = dv;
       const C a0 = ldv<COH>(ab + l);
-      accd[k] += T(2) * (T(2) * (a0.x * dv.x + a0.y * dv.y) + dv.x * dv.x + dv.y * dv.y);
+      accd[k] += density_term<T>(a0, dv);
     }
     __syncthreads();
   }
@@ -340,7 +429,7 @@ template <typename T, int N, bool COH, int PPB = kPPB<T, N>>
 __device__ __forceinline__ void inv_plain_planes(const GView<T> &g, C2<T> *data, long long item,
                                                  long long off, C2<T> *S) {
   using C = C2<T>;
-  constexpr int LD = N + 1, NN = N * N, NT = PPB * N;
+  constexpr int LD = N + 1, NT = PPB * N;
   const int pl = threadIdx.x / N, q = threadIdx.x - pl * N;
   C *base = data + item * g.ng + off;
   plane_inverse<T, N, COH>(S, base, pl, q);
@@ -353,18 +442,12 @@ __device__ __forceinline__ void inv_plain_planes(const GView<T> &g, C2<T> *data,
 
 template <typename T, int N, int MODE, int PPB = kPPB<T, N>>
 __global__ void __launch_bounds__(PPB * N)
-    k_plane_inv(GView<T> g, C2<T> *data, const C2<T> *a_next, T *dens, T *u_out, T *acc,
-                C2<T> *em1_out, PlaneInvArgs pa) {
+    k_plane_inv(GView<T> g, C2<T> *data, T *u_out, T *acc, C2<T> *em1_out, PlaneInvArgs pa) {
   using C = C2<T>;
   constexpr int LD = N + 1, NN = N * N, NT = PPB * N;
   extern __shared__ unsigned char smem_raw[];
   C *S = reinterpret_cast<C *>(smem_raw);
   const int pl = threadIdx.x / N, q = threadIdx.x - pl * N;
-  if constexpr (MODE == PI_DENSITY) {
-    // blockIdx.y = pair, blockIdx.x = group of PPB planes of each of its L orbitals
-    inv_density_planes<T, N, false>(g, data, a_next, dens, blockIdx.y, pa.L, blockIdx.x * PPB, S);
-    return;
-  }
   const long long p0 = (long long)blockIdx.x * PPB;  // PPB divides N: all planes of one item
   const long long item = p0 / N;
   const long long off = (p0 - item * N) * NN;
@@ -410,276 +493,8 @@ __global__ void __launch_bounds__(PPB * N)
   }
 }
 
-// ------------------------------------------------------------------------------------------
-// Inverse plane pass of the pair batch with the induced density, streamed by bulk copies (TMA):
-// a persistent block walks its (pair, plane group) units and, inside each, the L orbitals; the PPB
-// contiguous planes of the next orbital (and of eta0 at the same planes) are copied into shared
-// memory while the current ones are transformed, so no thread waits on a global load. Per chunk:
-// y inverse FFTs read the staged planes (thread per column, conflict-free) into the padded work
-// tile, which frees the staging buffer for the next chunk's copy; x inverse FFTs in the work tile;
-// the epilogue stores the orbital and accumulates the density from the staged eta0.
-
-// planes per chunk: largest divisor of N with <= 128 threads and <= 112 KB of shared memory
-// (two blocks per SM)
-constexpr int tma_inv_ppb(int N) {
-  int best = 0;
-  for (int d = 1; d <= N; ++d)
-    if (N % d == 0 && d * N <= 128 && (long long)d * N * N * 16 + (long long)d * N * (N + 1) * 8 <= 112 * 1024)
-      best = d;
-  return best;
-}
-template <int N> constexpr size_t tma_inv_smem() {
-  return (size_t)tma_inv_ppb(N) * N * N * 16 + (size_t)tma_inv_ppb(N) * N * (N + 1) * 8;
-}
-// grids streamed this way (even N: every chunk offset is a multiple of 16 bytes)
-constexpr bool tma_inv_size(int N) { return N == 32 || N == 40 || N == 48 || N == 64; }
-
-template <int N>
-__global__ void __launch_bounds__(tma_inv_ppb(N) * N)
-    k_plane_inv_density_tma(GView<float> g, float2 *data, const float2 *a_next, float *dens, int L,
-                            int n_pairs, int *err) {
-  using C = float2;
-  constexpr int PPB = tma_inv_ppb(N), NN = N * N, LD = N + 1, NT = PPB * N, G = N / PPB;
-  constexpr unsigned kChunk = PPB * NN * sizeof(C);
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  C *Sd = reinterpret_cast<C *>(smem_raw);  // staged orbital planes (dense)
-  C *Sa = Sd + PPB * NN;                     // staged eta0 planes (dense)
-  C *W = Sa + PPB * NN;                      // work tile, rows padded to N + 1
-  __shared__ __align__(8) uint64_t bar_d, bar_a;
-  const long long units = (long long)n_pairs * G;
-  long long u = blockIdx.x;
-  if (u >= units) return;
-  const int pl = threadIdx.x / N, q = threadIdx.x - pl * N;
-  auto src_d = [&](long long uu, int e) {
-    return data + ((uu / G) * L + e) * g.ng + (uu % G) * (long long)(PPB * NN);
-  };
-  auto src_a = [&](long long uu, int e) { return a_next + (long long)e * g.ng + (uu % G) * (long long)(PPB * NN); };
-  if (threadIdx.x == 0) {
-    tma_bar_init(&bar_d, 1);
-    tma_bar_init(&bar_a, 1);
-    tma_bar_expect(&bar_d, kChunk);
-    tma_load_1d(Sd, src_d(u, 0), kChunk, &bar_d);
-    tma_bar_expect(&bar_a, kChunk);
-    tma_load_1d(Sa, src_a(u, 0), kChunk, &bar_a);
-  }
-  __syncthreads();
-  unsigned ph_d = 0, ph_a = 0;
-  bool pend_d = true, pend_a = true, ok = true;
-  int ell = 0;
-  float accd[N];
-#pragma unroll
-  for (int k = 0; k < N; ++k) accd[k] = 0.f;
-  while (true) {
-    long long un = u;
-    int en = ell + 1;
-    if (en == L) {
-      en = 0;
-      un += gridDim.x;
-    }
-    const bool has_next = un < units;
-    // y inverse FFTs from the staged planes into the work tile
-    if (!__syncthreads_and(tma_bar_wait(&bar_d, ph_d))) {
-      ok = false;
-      break;
-    }
-    ph_d ^= 1u;
-    pend_d = false;
-    {
-      C v[N];
-#pragma unroll
-      for (int y = 0; y < N; ++y) v[y] = Sd[pl * NN + y * N + q];
-      fft_reg<float, N, +1, TwP<float>>(v);
-#pragma unroll
-      for (int y = 0; y < N; ++y) W[(pl * N + y) * LD + q] = v[y];
-    }
-    __syncthreads();
-    if (threadIdx.x == 0 && has_next) {
-      tma_fence_proxy();
-      tma_bar_expect(&bar_d, kChunk);
-      tma_load_1d(Sd, src_d(un, en), kChunk, &bar_d);
-    }
-    pend_d = has_next;
-    {
-      C v[N];
-      C *row = W + (pl * N + q) * LD;
-#pragma unroll
-      for (int x = 0; x < N; ++x) v[x] = row[x];
-      fft_reg<float, N, +1, TwP<float>>(v);
-#pragma unroll
-      for (int x = 0; x < N; ++x) row[x] = v[x];
-    }
-    if (!__syncthreads_and(tma_bar_wait(&bar_a, ph_a))) {
-      ok = false;
-      break;
-    }
-    ph_a ^= 1u;
-    pend_a = false;
-    const long long pair = u / G, off = (u % G) * (long long)(PPB * NN);
-    C *base = data + (pair * L + ell) * g.ng + off;
-#pragma unroll
-    for (int k = 0; k < N; ++k) {
-      const int l = threadIdx.x + k * NT;
-      const C dv = W[(threadIdx.x / N) * LD + threadIdx.x % N + k * PPB * LD];
-      base[l] = dv;
-      const C a0 = Sa[l];
-      accd[k] += 2.f * (2.f * (a0.x * dv.x + a0.y * dv.y) + dv.x * dv.x + dv.y * dv.y);
-    }
-    __syncthreads();
-    if (threadIdx.x == 0 && has_next) {
-      tma_fence_proxy();
-      tma_bar_expect(&bar_a, kChunk);
-      tma_load_1d(Sa, src_a(un, en), kChunk, &bar_a);
-    }
-    pend_a = has_next;
-    if (ell == L - 1) {
-      float *db = dens + pair * g.ng + off;
-#pragma unroll
-      for (int k = 0; k < N; ++k) {
-        db[threadIdx.x + k * NT] = accd[k];
-        accd[k] = 0.f;
-      }
-    }
-    if (!has_next) break;
-    u = un;
-    ell = en;
-  }
-  if (!ok) {
-    if (threadIdx.x == 0) atomicExch(err, 1);
-    // copies still in flight must land before the block's shared memory is released
-    if (pend_d) tma_bar_wait(&bar_d, ph_d);
-    if (pend_a) tma_bar_wait(&bar_a, ph_a);
-  }
-}
-
-// z-column pass streamed by bulk copies: a persistent block walks (item, slab of Y rows) units;
-// the slab's N z-rows (Y N contiguous points each) are copied into shared memory, every thread takes
-// its column (conflict-free across x) into registers, the buffer is refilled with the next unit,
-// and the forward z FFT, the multiplier and the inverse z FFT run while the copies are in flight.
-constexpr int tma_z_rows(int N) {
-  int best = 0;
-  for (int y = 1; y <= N; ++y)
-    if (N % y == 0 && y * N <= 256 && (long long)y * N * N * 8 <= 80 * 1024) best = y;
-  return best;
-}
-
-template <int N>
-__global__ void __launch_bounds__(tma_z_rows(N) * N)
-    k_zcol_tma(GView<float> g, float2 *data, long long n_items, int mult, int *err) {
-  using C = float2;
-  constexpr int Y = tma_z_rows(N), NN = N * N, G = N / Y;
-  constexpr unsigned kRow = Y * N * sizeof(C);
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  C *S = reinterpret_cast<C *>(smem_raw);  // [z][y][x] of the slab
-  __shared__ __align__(8) uint64_t bar;
-  const long long units = n_items * G;
-  long long u = blockIdx.x;
-  if (u >= units) return;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int yy = threadIdx.x / N, x = threadIdx.x - yy * N;
-  auto issue = [&](long long uu) {  // warp 0: one arrival with the byte count, then N row copies
-    const C *src = data + (uu / G) * g.ng + (uu % G) * (long long)(Y * N);
-    if (lane == 0) tma_bar_expect(&bar, kRow * N);
-    __syncwarp();
-    for (int z = lane; z < N; z += 32) tma_load_1d(S + z * Y * N, src + (long long)z * NN, kRow, &bar);
-  };
-  if (threadIdx.x == 0) tma_bar_init(&bar, 1);
-  __syncthreads();
-  if (warp == 0) issue(u);
-  unsigned ph = 0;
-  bool pend = true, ok = true;
-  const float inv_ng = 1.f / (float)(N * N * N);
-  while (true) {
-    const long long un = u + gridDim.x;
-    const bool has_next = un < units;
-    if (!__syncthreads_and(tma_bar_wait(&bar, ph))) {
-      ok = false;
-      break;
-    }
-    ph ^= 1u;
-    pend = false;
-    C v[N];
-#pragma unroll
-    for (int z = 0; z < N; ++z) v[z] = S[(z * Y + yy) * N + x];
-    __syncthreads();
-    if (warp == 0 && has_next) {
-      tma_fence_proxy();
-      issue(un);
-    }
-    pend = has_next;
-    const int y = (int)(u % G) * Y + yy;
-    fft_reg<float, N, -1, TwP<float>>(v);
-    if (mult == Z_KINETIC) {
-      const C mxy = cscale(cmul(g.kin[x], g.kin[y]), inv_ng);
-#pragma unroll
-      for (int z = 0; z < N; ++z) v[z] = cmul(v[z], cmul(mxy, g.kin[z]));
-    } else {
-      const float gxy = g.k2[x] + g.k2[y];
-#pragma unroll
-      for (int z = 0; z < N; ++z) {
-        const float G2 = gxy + g.k2[z];
-        v[z] = cscale(v[z], G2 > 0.f ? float(4.0 * M_PI) * inv_ng / G2 : 0.f);
-      }
-    }
-    fft_reg<float, N, +1, TwP<float>>(v);
-    C *base = data + (u / G) * g.ng + (long long)y * N + x;
-#pragma unroll
-    for (int z = 0; z < N; ++z) base[(long long)z * NN] = v[z];
-    if (!has_next) break;
-    u = un;
-  }
-  if (!ok) {
-    if (threadIdx.x == 0) atomicExch(err, 1);
-    if (pend) tma_bar_wait(&bar, ph);
-  }
-}
-
-// resident blocks per SM times SMs of the current device for a kernel and launch shape (0 if the
-// query fails)
-template <typename K> static long long resident_slots(K kernel, int threads, size_t smem) {
-  int dev = 0, sms = 0, per_sm = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem) != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
-  return (long long)per_sm * sms;
-}
-
-template <int N>
-static bool zcol_tma(const GridTables<float> &g, float2 *d, int n_items, int mult, int *err, cudaStream_t s) {
-  if constexpr (tma_inv_size(N)) {
-    constexpr int Y = tma_z_rows(N);
-    constexpr size_t sm = (size_t)Y * N * N * sizeof(float2);
-    const long long units = (long long)n_items * (N / Y);
-    // resident blocks of the whole GPU; function-local static: initialised once, thread-safe
-    static const long long slots = resident_slots(k_zcol_tma<N>, Y * N, sm);
-    if (slots < 1 || units < 1) return false;
-    const long long grid = units < slots ? units : slots;
-    k_zcol_tma<N><<<(unsigned)grid, Y * N, sm, s>>>(view(g), d, n_items, mult, err);
-    return true;
-  }
-  return false;
-}
-
-template <int N>
-static bool inv_density_tma(const GridTables<float> &g, float2 *d, int n_items, const float2 *a_next, int L,
-                            float *dens, int *err, cudaStream_t s) {
-  if constexpr (tma_inv_size(N)) {
-    constexpr int PPB = tma_inv_ppb(N);
-    const long long units = (long long)(n_items / L) * (N / PPB);
-    // a unit works through its pair's L orbitals in turn: with fewer units than SMs the stored-orbitals form
-    // is faster (10 pairs of 32^3, 80 units: 20.0 -> 8.9 + 5.3 us)
-    if (units < 152) return false;
-    static const long long slots = resident_slots(k_plane_inv_density_tma<N>, PPB * N, tma_inv_smem<N>());
-    if (slots < 1) return false;
-    const long long grid = units < slots ? units : slots;
-    k_plane_inv_density_tma<N><<<(unsigned)grid, PPB * N, tma_inv_smem<N>(), s>>>(view(g), d, a_next, dens, L,
-                                                                                  n_items / L, err);
-    return true;
-  }
-  return false;
-}
+// grids whose FP32 orbitals take the lane-pair sweeps (fft_split.cu): the persistent step does too
+constexpr bool lane_pairs(int N) { return N == 32 || N == 48 || N == 64; }
 
 // ------------------------------------------------------------------------------------------
 // Persistent split-operator step: one launch advances the eta0 set and every pair's L orbitals by
@@ -705,6 +520,60 @@ __device__ __forceinline__ bool wait_geq(const unsigned *p, unsigned target, uns
   return false;
 }
 
+// One tile with lane-pair pencils: its PPB planes, or its PPB N columns, in two halves
+template <int N>
+__device__ __forceinline__ void step_tile_pairs(const GView<float> &g, const XfwdArgs<float> &fa, const XfwdArgs<float> &fp,
+                                                float2 *a_next, float2 *d, float *dens, int L, int4 it, float2 *S,
+                                                const float2 *tab) {
+  using C = float2;
+  constexpr int PPB = kPPB<float, N>, NN = N * N, NT = PPB * N, H = N / 2;
+  static_assert(PPB % 2 == 0, "two halves of PPB / 2 planes");
+  const int grp = threadIdx.x / (2 * N), tid = threadIdx.x - grp * 2 * N;
+  if (it.x == SI_A_FWD || it.x == SI_P_FWD) {
+#pragma unroll 1
+    for (int half = 0; half < 2; ++half) {
+      if (half) __syncthreads();
+      const long long off = ((long long)it.z * PPB + half * (PPB / 2) + grp) * NN;
+      C *tile = S + grp * N * (N + 1);
+      if (it.x == SI_P_FWD)
+        kin2_plane<N, true>(g, fp, it.y, off, tile, tab, tid);
+      else
+        kin2_plane<N, false>(g, fa, it.y, off, tile, tab, tid);
+    }
+    return;
+  }
+  const bool pair = it.x == SI_P_INV;
+  if (!pair && it.x != SI_A_Z) return;
+  const int lane = threadIdx.x & 31, s = lane >> 4, cw = (threadIdx.x >> 5) * 16 + (lane & 15);
+  float *D = reinterpret_cast<float *>(S) + cw;
+#pragma unroll 1
+  for (int half = 0; half < 2; ++half) {
+    const int rem = it.z * NT + half * (NT / 2) + cw;
+    for (int l = 0; l < (pair ? L : 1); ++l) {
+      C *base = (pair ? d + ((long long)it.y * L + l) * g.ng : a_next + (long long)it.y * g.ng) + rem;
+      C v[H];
+#pragma unroll
+      for (int m = 0; m < H; ++m) v[m] = __ldcg(base + (long long)(2 * m + s) * NN);
+      kin_roundtrip<N>(v, s, tab);
+#pragma unroll
+      for (int m = 0; m < H; ++m) base[(long long)(2 * m + s) * NN] = v[m];
+      if (pair) {
+        const C *ab = a_next + (long long)l * g.ng + rem;
+#pragma unroll
+        for (int m = 0; m < H; ++m) {
+          const float t = density_term<float>(__ldcg(ab + (long long)(2 * m + s) * NN), v[m]);
+          float &acc = D[(2 * m + s) * (NT / 2)];
+          acc = l ? acc + t : t;
+        }
+      }
+    }
+    if (pair)
+#pragma unroll 8
+      for (int m = 0; m < H; ++m)
+        dens[(long long)it.y * g.ng + (long long)(2 * m + s) * NN + rem] = D[(2 * m + s) * (NT / 2)];
+  }
+}
+
 template <typename T, int N>
 __global__ void __launch_bounds__(kPPB<T, N> * N)
     k_step_persistent(GView<T> g, XfwdArgs<T> fa, XfwdArgs<T> fp, C2<T> *a_next, C2<T> *d, T *dens,
@@ -715,6 +584,16 @@ __global__ void __launch_bounds__(kPPB<T, N> * N)
   C *S = reinterpret_cast<C *>(smem_raw);
   __shared__ int4 cur;
   __shared__ int go;
+  // FP32 takes the two sweeps of k_plane_kin and k_zkin (SI_A_Z, SI_P_INV: z operator on NT columns),
+  // with lane pairs where the sweeps take them
+  constexpr bool KIN = sizeof(T) == 4;
+  constexpr bool LP = KIN && lane_pairs(N);
+  __shared__ C kt[LP ? 3 * N / 2 : KIN ? N : 1];
+  if constexpr (LP) {  // (read after the first tile's barrier)
+    for (int i = threadIdx.x; i < 3 * N / 2; i += blockDim.x) kt[i] = g.kin[N + i];
+  } else if constexpr (KIN) {
+    load_kin<N>(kt, g);
+  }
   const unsigned tgt = (q.epoch + 1) * (unsigned)G;
   for (;;) {
     if (threadIdx.x == 0) {
@@ -729,7 +608,8 @@ __global__ void __launch_bounds__(kPPB<T, N> * N)
         ok = wait_geq(q.p_fwd + it.y, tgt, q.wait_limit);
       } else if (it.x == SI_P_INV) {
         ok = wait_geq(q.a_inv, (q.epoch + 1) * (unsigned)(L * G), q.wait_limit);
-        for (int l = 0; l < L && ok; ++l) ok = wait_geq(q.p_z + it.y * L + l, tgt, q.wait_limit);
+        const unsigned *before = KIN ? q.p_fwd : q.p_z;
+        for (int l = 0; l < L && ok; ++l) ok = wait_geq(before + it.y * L + l, tgt, q.wait_limit);
       }
       if (!ok) atomicExch(q.err, 1);
       __threadfence();
@@ -740,14 +620,43 @@ __global__ void __launch_bounds__(kPPB<T, N> * N)
     const int4 it = cur;
     if (it.x < 0) break;
     if (go) {
-      switch (it.x) {
-        case SI_A_FWD: fwd_planes<T, N, false>(g, fa, it.y, (long long)it.z * PPB * NN, S); break;
-        case SI_P_FWD: fwd_planes<T, N, true>(g, fp, it.y, (long long)it.z * PPB * NN, S); break;
-        case SI_A_Z: zcol_column<T, N, true>(g, a_next, it.y, it.z * NT + threadIdx.x, Z_KINETIC); break;
-        case SI_P_Z: zcol_column<T, N, true>(g, d, it.y, it.z * NT + threadIdx.x, Z_KINETIC); break;
-        case SI_A_INV: inv_plain_planes<T, N, true>(g, a_next, it.y, (long long)it.z * PPB * NN, S); break;
-        case SI_P_INV: inv_density_planes<T, N, true>(g, d, a_next, dens, it.y, L, it.z * PPB, S); break;
-        default: break;
+      if constexpr (LP) {
+        step_tile_pairs<N>(g, fa, fp, a_next, d, dens, L, it, S, kt);
+      } else if constexpr (KIN) {
+        const int rem = it.z * NT + threadIdx.x;
+        switch (it.x) {
+          case SI_A_FWD: fwd_planes<T, N, false, PPB, true>(g, fa, it.y, (long long)it.z * PPB * NN, S, kt); break;
+          case SI_P_FWD: fwd_planes<T, N, true, PPB, true>(g, fp, it.y, (long long)it.z * PPB * NN, S, kt); break;
+          case SI_A_Z:
+          case SI_P_INV: {
+            const bool pair = it.x == SI_P_INV;
+            float *D = reinterpret_cast<float *>(S);
+            for (int l = 0; l < (pair ? L : 1); ++l) {
+              C *base = (pair ? d + ((long long)it.y * L + l) * g.ng : a_next + (long long)it.y * g.ng) + rem;
+              C v[N];
+#pragma unroll
+              for (int z = 0; z < N; ++z) v[z] = __ldcg(base + (long long)z * NN);
+              kin_pencil<N>(v, kt);
+#pragma unroll
+              for (int z = 0; z < N; ++z) base[(long long)z * NN] = v[z];
+              if (pair) add_density<N, true>(v, a_next + (long long)l * g.ng + rem, D + threadIdx.x, NT, l == 0);
+            }
+            if (pair)
+              for (int z = 0; z < N; ++z) dens[(long long)it.y * g.ng + (long long)z * NN + rem] = D[z * NT + threadIdx.x];
+            break;
+          }
+          default: break;
+        }
+      } else {
+        switch (it.x) {
+          case SI_A_FWD: fwd_planes<T, N, false>(g, fa, it.y, (long long)it.z * PPB * NN, S); break;
+          case SI_P_FWD: fwd_planes<T, N, true>(g, fp, it.y, (long long)it.z * PPB * NN, S); break;
+          case SI_A_Z: zcol_column<T, N, true>(g, a_next, it.y, it.z * NT + threadIdx.x, Z_KINETIC); break;
+          case SI_P_Z: zcol_column<T, N, true>(g, d, it.y, it.z * NT + threadIdx.x, Z_KINETIC); break;
+          case SI_A_INV: inv_plain_planes<T, N, true>(g, a_next, it.y, (long long)it.z * PPB * NN, S); break;
+          case SI_P_INV: inv_density_planes<T, N, true>(g, d, a_next, dens, it.y, L, it.z * PPB, S); break;
+          default: break;
+        }
       }
     }
     __syncthreads();
@@ -755,7 +664,7 @@ __global__ void __launch_bounds__(kPPB<T, N> * N)
       __threadfence();
       unsigned *c = nullptr;
       if (it.x == SI_A_FWD) c = q.a_fwd + it.y;
-      else if (it.x == SI_A_Z) c = q.a_z + it.y;
+      else if (it.x == SI_A_Z) c = KIN ? q.a_inv : q.a_z + it.y;
       else if (it.x == SI_A_INV) c = q.a_inv;
       else if (it.x == SI_P_FWD) c = q.p_fwd + it.y;
       else if (it.x == SI_P_Z) c = q.p_z + it.y;
@@ -770,24 +679,27 @@ __global__ void __launch_bounds__(kPPB<T, N> * N)
 template <typename T, int N, bool STEP = false> void set_attrs() {
   const int sm = (int)plane_smem<T, N>();
   if constexpr (STEP) cudaFuncSetAttribute(k_step_persistent<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  cudaFuncSetAttribute(k_plane_fwd<T, N, true, fwd_ppb<T, N, true>()>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)fwd_smem<T, N, true>());
-  cudaFuncSetAttribute(k_plane_fwd<T, N, false, kPPB<T, N>>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  if constexpr (kFew<T, N> < kPPB<T, N> && few_plane_smem<T, N>() > 48 * 1024) {
-    const int sf = (int)few_plane_smem<T, N>();
-    cudaFuncSetAttribute(k_plane_fwd<T, N, true, kFew<T, N>>, cudaFuncAttributeMaxDynamicSharedMemorySize, sf);
-    cudaFuncSetAttribute(k_plane_fwd<T, N, false, kFew<T, N>>, cudaFuncAttributeMaxDynamicSharedMemorySize, sf);
-    cudaFuncSetAttribute(k_plane_inv<T, N, PI_PLAIN, kFew<T, N>>, cudaFuncAttributeMaxDynamicSharedMemorySize, sf);
+  const int sf = (int)few_plane_smem<T, N>();
+  constexpr bool few = kFew<T, N> < kPPB<T, N> && few_plane_smem<T, N>() > 48 * 1024;
+  auto limit = [](auto *k, int bytes) { cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); };
+  limit(k_plane_fwd<T, N, false, kPPB<T, N>>, sm);
+  limit(k_plane_inv<T, N, PI_POISSON>, sm);
+  if constexpr (few) limit(k_plane_fwd<T, N, false, kFew<T, N>>, sf);
+  if constexpr (sizeof(T) == 4 && !lane_pairs(N)) {
+    limit(k_plane_kin<N, false, kPPB<T, N>>, sm);
+    limit(k_plane_kin<N, true, fwd_ppb<T, N, true>()>, (int)fwd_smem<T, N, true>());
+    if constexpr (few) {
+      limit(k_plane_kin<N, false, kFew<T, N>>, sf);
+      limit(k_plane_kin<N, true, kFew<T, N>>, sf);
+    }
   }
-  cudaFuncSetAttribute(k_plane_inv<T, N, PI_PLAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  if constexpr (sizeof(T) == 4)
-    cudaFuncSetAttribute(k_plane_inv<T, N, PI_DENSITY>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  cudaFuncSetAttribute(k_plane_inv<T, N, PI_POISSON>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  if constexpr (sizeof(T) == 4 && tma_inv_size(N)) {
-    cudaFuncSetAttribute(k_plane_inv_density_tma<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)tma_inv_smem<N>());
-    cudaFuncSetAttribute(k_zcol_tma<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)(tma_z_rows(N) * N * N * sizeof(float2)));
+  if constexpr (sizeof(T) == 8) {
+    limit(k_plane_fwd<T, N, true, kPPB<T, N>>, sm);
+    limit(k_plane_inv<T, N, PI_PLAIN>, sm);
+    if constexpr (few) {
+      limit(k_plane_fwd<T, N, true, kFew<T, N>>, sf);
+      limit(k_plane_inv<T, N, PI_PLAIN, kFew<T, N>>, sf);
+    }
   }
 }
 
@@ -812,21 +724,59 @@ template <typename T> struct FastOps {
     return 0;
   }
   template <int N> static int tiles_per_orbital() { return N / kPPB<T, N>; }
+  // packing modes, and the FP64 orbitals
   template <int N> static void fwd(const GridTables<T> &g, const XfwdArgs<T> &a, cudaStream_t s) {
     if constexpr (!(sizeof(T) == 8 && N > 48)) {
       const long long planes = (long long)a.n_items * N;
-      constexpr int P2 = fwd_ppb<T, N, true>(), PF = kFew<T, N>;
-      if (few_planes<T, N>(planes)) {
-        if (a.mode == XF_PHASE_PAIR)
-          k_plane_fwd<T, N, true, PF><<<(unsigned)(planes / PF), PF * N, few_plane_smem<T, N>(), s>>>(view(g), a, planes);
-        else
-          k_plane_fwd<T, N, false, PF><<<(unsigned)(planes / PF), PF * N, few_plane_smem<T, N>(), s>>>(view(g), a, planes);
-      } else if (a.mode == XF_PHASE_PAIR) {
-        k_plane_fwd<T, N, true, P2><<<(unsigned)(planes / P2), P2 * N, fwd_smem<T, N, true>(), s>>>(view(g), a, planes);
-      } else {
-        k_plane_fwd<T, N, false, kPPB<T, N>><<<(unsigned)(planes / kPPB<T, N>), kPPB<T, N> * N, plane_smem<T, N>(),
-                                               s>>>(view(g), a, planes);
+      constexpr int PP = kPPB<T, N>, PF = kFew<T, N>;
+      const bool few = few_planes<T, N>(planes);
+      const unsigned blocks = (unsigned)(planes / (few ? PF : PP));
+      if constexpr (sizeof(T) == 8) {
+        if (a.mode == XF_PHASE_PAIR) {
+          if (few)
+            k_plane_fwd<T, N, true, PF><<<blocks, PF * N, few_plane_smem<T, N>(), s>>>(view(g), a, planes);
+          else
+            k_plane_fwd<T, N, true, PP><<<blocks, PP * N, plane_smem<T, N>(), s>>>(view(g), a, planes);
+          return;
+        }
       }
+      if (few)
+        k_plane_fwd<T, N, false, PF><<<blocks, PF * N, few_plane_smem<T, N>(), s>>>(view(g), a, planes);
+      else
+        k_plane_fwd<T, N, false, PP><<<blocks, PP * N, plane_smem<T, N>(), s>>>(view(g), a, planes);
+    }
+  }
+  // the two sweeps of the FP32 orbitals
+  template <int N> static void kin(const GridTables<T> &g, const XfwdArgs<T> &a, cudaStream_t s) {
+    if constexpr (sizeof(T) == 4 && !lane_pairs(N)) {
+      const long long planes = (long long)a.n_items * N;
+      constexpr int P2 = fwd_ppb<T, N, true>(), PP = kPPB<T, N>, PF = kFew<T, N>;
+      const bool pair = a.mode == XF_PHASE_PAIR;
+      if (few_planes<T, N>(planes)) {
+        const unsigned blocks = (unsigned)(planes / PF);
+        if (pair) k_plane_kin<N, true, PF><<<blocks, PF * N, few_plane_smem<T, N>(), s>>>(view(g), a, planes);
+        else k_plane_kin<N, false, PF><<<blocks, PF * N, few_plane_smem<T, N>(), s>>>(view(g), a, planes);
+      } else if (pair) {
+        k_plane_kin<N, true, P2><<<(unsigned)(planes / P2), P2 * N, fwd_smem<T, N, true>(), s>>>(view(g), a, planes);
+      } else {
+        k_plane_kin<N, false, PP><<<(unsigned)(planes / PP), PP * N, plane_smem<T, N>(), s>>>(view(g), a, planes);
+      }
+    }
+  }
+  template <int N>
+  static void zkin(const GridTables<T> &g, C2<T> *d, int n_items, const C2<T> *a_next, int L, T *dens, cudaStream_t s) {
+    if constexpr (sizeof(T) == 4 && !lane_pairs(N)) {
+      constexpr long long per_unit = (N * N + kZkT - 1) / kZkT;
+      // the density summed in the sweep needs one block per pair and 128 columns, working through L orbitals
+      // in turn: below two blocks per SM a second kernel sums it from the stored orbitals
+      if (dens && n_items / L * per_unit >= 304) {
+        k_zkin<N, true><<<(unsigned)(n_items / L * per_unit), kZkT, 0, s>>>(view(g), d, a_next, dens, n_items / L, L);
+        return;
+      }
+      const int nt = n_items * per_unit < 152 ? 32 : kZkT;
+      k_zkin<N, false><<<(unsigned)((long long)n_items * ((N * N + nt - 1) / nt)), nt, 0, s>>>(view(g), d, nullptr, nullptr,
+                                                                                          n_items, 1);
+      if (dens) launch_density<float>(g, d, a_next, n_items / L, L, dens, s);
     }
   }
   template <int N> static void z(const GridTables<T> &g, C2<T> *d, int n_items, int mult, cudaStream_t s) {
@@ -837,31 +787,26 @@ template <typename T> struct FastOps {
       k_zcol<T, N><<<(unsigned)((cols + nt - 1) / nt), nt, 0, s>>>(view(g), d, cols, mult);
     }
   }
+  // mode: PI_PLAIN (FP64 orbitals) or PI_POISSON
   template <int N>
-  static void inv(const GridTables<T> &g, C2<T> *d, int n_items, const C2<T> *a_next, int L, T *dens,
-                  T *u_out, T *acc, C2<T> *em1_out, const PoissonOut &po, int mode, cudaStream_t s) {
+  static void inv(const GridTables<T> &g, C2<T> *d, int n_items, T *u_out, T *acc, C2<T> *em1_out, const PoissonOut &po,
+                  int mode, cudaStream_t s) {
     if constexpr (!(sizeof(T) == 8 && N > 48)) {
-      PlaneInvArgs pa{(long long)n_items * N, L, po};
-      const size_t sm = plane_smem<T, N>();
-      constexpr int NT = kPPB<T, N> * N;
-      if (sizeof(T) == 4 && mode == PI_DENSITY) {
-        if constexpr (sizeof(T) == 4) {
-          dim3 grid(N / kPPB<T, N>, n_items / L);
-          k_plane_inv<T, N, PI_DENSITY><<<grid, NT, sm, s>>>(view(g), d, a_next, dens, nullptr, nullptr,
-                                                              nullptr, pa);
+      const PlaneInvArgs pa{(long long)n_items * N, po};
+      constexpr int PP = kPPB<T, N>, PF = kFew<T, N>;
+      const unsigned blocks = (unsigned)(pa.planes_total / PP);
+      if constexpr (sizeof(T) == 8) {
+        if (mode == PI_PLAIN) {
+          if (few_planes<T, N>(pa.planes_total))
+            k_plane_inv<T, N, PI_PLAIN, PF><<<(unsigned)(pa.planes_total / PF), PF * N, few_plane_smem<T, N>(), s>>>(
+                view(g), d, nullptr, nullptr, nullptr, pa);
+          else
+            k_plane_inv<T, N, PI_PLAIN><<<blocks, PP * N, plane_smem<T, N>(), s>>>(view(g), d, nullptr, nullptr, nullptr, pa);
+          return;
         }
-      } else if (mode == PI_PLAIN && few_planes<T, N>(pa.planes_total)) {
-        constexpr int PF = kFew<T, N>;
-        k_plane_inv<T, N, PI_PLAIN, PF><<<(unsigned)(pa.planes_total / PF), PF * N, few_plane_smem<T, N>(), s>>>(
-            view(g), d, nullptr, nullptr, nullptr, nullptr, nullptr, pa);
-      } else if (mode == PI_PLAIN) {
-        k_plane_inv<T, N, PI_PLAIN><<<(unsigned)(pa.planes_total / kPPB<T, N>), NT, sm, s>>>(
-            view(g), d, nullptr, nullptr, nullptr, nullptr, nullptr, pa);
-      } else {
-        k_plane_inv<T, N, PI_POISSON><<<(unsigned)(pa.planes_total / kPPB<T, N>), NT, sm, s>>>(
-            view(g), d, nullptr, nullptr, u_out, acc, em1_out, pa);
       }
-  }
+      k_plane_inv<T, N, PI_POISSON><<<blocks, PP * N, plane_smem<T, N>(), s>>>(view(g), d, u_out, acc, em1_out, pa);
+    }
   }
 };
 

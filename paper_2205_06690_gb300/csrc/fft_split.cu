@@ -1,9 +1,9 @@
-// Three-pass 3D FFT round trip for the grid edges N = 80 and 96 (FP32): the split-operator step
-// of Eq. (10), the Poisson solves of Eq. (11) / q_ij and the exchange potentials of Eq. (1) on the
-// paper-scale grids (the 520-electron system of Sec. III sits on ~0.85M points, 96^3 here).
+// Lane-pair passes (FP32). N = 80 and 96: the split-operator step of Eq. (10), the Poisson solves of
+// Eq. (11) / q_ij and the exchange potentials of Eq. (1) on the paper-scale grids (the 520-electron
+// system of Sec. III sits on ~0.85M points, 96^3 here). N = 32, 48 and 64: the split-operator step.
 //
-// A pencil of N points is too long for one thread's registers next to the epilogue's state, so it
-// is split over a lane pair (l, l ^ 16) of one warp: N = 2H, each lane holds H points, transforms
+// A pencil of N points is too long for one thread's registers next to the epilogue's state (80, 96), or
+// leaves room for too few warps to hide the loads (48: 12 warps per SM), so it is split over a lane pair (l, l ^ 16) of one warp: N = 2H, each lane holds H points, transforms
 // them with the register FFT of length H, and one radix-2 butterfly across the pair (operands
 // swapped by warp shuffles) completes the transform. Forward transforms take the pencil
 // interleaved (lane s holds x[2m + s]) and return it in two quarter blocks (decimation in time);
@@ -26,176 +26,14 @@
 // Blocks are ordered plane-major (plane outer, item inner), so the tables read beside the orbitals
 // (eta0 of each stochastic orbital, the potential phases, E - 1 of each pair) are the same z-slice
 // for consecutive blocks and stay in L2 even when the whole table set does not fit there.
-#include <math.h>
-
-#include <type_traits>
-
-#include "fft_reg.cuh"
-#include "kernels.h"
-#include "bounds.cuh"
-#include "passes.cuh"
-#include "tma.cuh"
+#include "fft_pair.cuh"
 
 namespace sbse {
 
 namespace {
 
-__constant__ float2 c_tws[kRegTotal];
-
-struct TwS {
-  __device__ __forceinline__ static float2 get(int i) { return c_tws[i]; }
-};
-
-constexpr unsigned kFull = 0xffffffffu;
-
-// exp(SIGN 2 pi i k / N)
-template <int N, int SIGN> __device__ __forceinline__ float2 tw_full(int k) {
-  float2 w = TwS::get(reg_offset(N) + k);
-  if (SIGN > 0) w.y = -w.y;
-  return w;
-}
-
-__device__ __forceinline__ float2 shfl_pair(float2 v) {
-  return make_float2(__shfl_xor_sync(kFull, v.x, 16), __shfl_xor_sync(kFull, v.y, 16));
-}
-
-// Decimation in time across the lane pair. On entry lane s of the pair holds x[2m + s], m < H;
-// on return it holds X[s Q + j] in v[j] and X[H + s Q + j] in v[Q + j] (j < Q = H / 2), where
-// X[k] = sum_n x[n] exp(SIGN 2 pi i n k / N): X[k] = E[k] + W^k O[k], X[k + H] = E[k] - W^k O[k]
-// with E, O the H-point transforms of the even and odd samples.
-template <int N, int SIGN> __device__ __forceinline__ void fft2_dit(float2 (&v)[N / 2], int s) {
-  constexpr int H = N / 2, Q = H / 2;
-  fft_reg<float, H, SIGN, TwS>(v);
-#pragma unroll
-  for (int j = 0; j < Q; ++j) {
-    // lane 0 keeps E[j] and needs O[j]; lane 1 keeps O[Q + j] and needs E[Q + j]
-    const float2 rcv = shfl_pair(s ? v[j] : v[Q + j]);
-    const float2 e = s ? rcv : v[j];
-    const float2 o = s ? v[Q + j] : rcv;
-    float2 t = cmul(o, tw_full<N, SIGN>(j));
-    if (s) t = cmul_si(t, SIGN);  // W^Q = exp(SIGN i pi / 2) = SIGN i
-    v[j] = cadd(e, t);
-    v[Q + j] = csub(e, t);
-  }
-}
-
-// Decimation in frequency across the lane pair: the inverse of the layout change above. On entry
-// lane s holds X[s Q + j] in v[j] and X[H + s Q + j] in v[Q + j]; on return it holds x[2m + s] in
-// v[m], x[n] = sum_k X[k] exp(SIGN 2 pi i n k / N). The even outputs are the H-point transform of
-// a_k = X[k] + X[k + H], the odd ones that of b_k = (X[k] - X[k + H]) W^k; lane 0 gathers every
-// a_k and lane 1 every b_k.
-template <int N, int SIGN> __device__ __forceinline__ void fft2_dif(float2 (&v)[N / 2], int s) {
-  constexpr int H = N / 2, Q = H / 2;
-#pragma unroll
-  for (int j = 0; j < Q; ++j) {
-    const float2 a = cadd(v[j], v[Q + j]);
-    float2 b = cmul(csub(v[j], v[Q + j]), tw_full<N, SIGN>(j));
-    if (s) b = cmul_si(b, SIGN);
-    const float2 rcv = shfl_pair(s ? a : b);
-    v[j] = s ? rcv : a;
-    v[Q + j] = s ? b : rcv;
-  }
-  fft_reg<float, H, SIGN, TwS>(v);
-}
-
-// the padded plane tile; the density pass adds the pair's density accumulator (N^2 floats)
-// One-dimensional kinetic operator F^-1 diag(K / N) F on the pencil held by a lane pair, without
-// leaving registers: on entry lane s holds x[2m + s], on return y[2m + s] (y = F^-1 K F x / N). Each
-// lane takes the half-length transform of its samples (E for the even ones, O for the odd ones),
-// receives the other lane's, forms E Kp + O M1 (lane 0: even outputs) or O Kp + E M2 (lane 1: odd
-// outputs), and transforms back. tab = [Kp | M1 | M2], N/2 entries each (see set_kinetic).
-template <int N>
-__device__ __forceinline__ void kin_roundtrip(float2 (&v)[N / 2], int s, const float2 *tab) {
-  constexpr int H = N / 2;
-  fft_reg<float, H, -1, TwS>(v);
-  const float2 *mt = tab + (s ? 2 * H : H);
-#pragma unroll
-  for (int k = 0; k < H; ++k) {
-    const float2 o = shfl_pair(v[k]);
-    const float2 kp = tab[k], mk = mt[k];
-    v[k] = cmac2(v[k], kp, o, mk);
-  }
-  fft_reg<float, H, +1, TwS>(v);
-}
-
 template <int N> constexpr size_t split_smem() { return (size_t)N * (N + 1) * sizeof(float2); }
 template <int N> constexpr size_t split_density_smem() { return split_smem<N>() + (size_t)N * N * sizeof(float); }
-
-// ------------------------------------------------------------------------------------------
-// The pre-operation of a forward plane pass into the padded tile. Thread t of the 2N covers the
-// points t + k 2N (k < N / 2) of the plane, i.e. row t / N + 2k, column t % N.
-template <int N, bool PAIR>
-__device__ __forceinline__ void preop_plane(const GView<float> &g, const XfwdArgs<float> &a, long long item,
-                                            long long off, float2 *S) {
-  using C = float2;
-  constexpr int LD = N + 1, NT = 2 * N, KP = N / 2, UB = 8;
-  const PreopItem<float> it = preop_item<float>(g, a, item);
-  (void)SBSE_IDX(item, a.n_items);
-  (void)SBSE_IDX(off + threadIdx.x + (long long)(KP - 1) * NT, g.ng);  // the largest point this thread reads
-  if constexpr (PAIR) (void)SBSE_IDX(item / a.L, a.n_items / a.L);     // the pair of E - 1
-  const int y0 = threadIdx.x / N;
-  C *srow = S + y0 * LD + (threadIdx.x - y0 * N);
-  if constexpr (PAIR) {
-    const C *dp = it.in + off + threadIdx.x, *ap = it.a + off + threadIdx.x, *pp = it.pv + off + threadIdx.x;
-    const C *ep = it.em1 ? it.em1 + off + threadIdx.x : nullptr;
-    // the deferred renormalisation is pending only in the step after a cleaning (cm1 != 0, the same
-    // for the whole block): the other steps skip its arithmetic (d is then unchanged by it)
-    auto sweep = [&](auto renorm) {
-      constexpr bool RN = decltype(renorm)::value;
-#pragma unroll 1
-      for (int k0 = 0; k0 < KP; k0 += UB) {
-        C dv[UB], av[UB], pv[UB], ev[UB];
-#pragma unroll
-        for (int k = 0; k < UB; ++k) {
-          if (k0 + k < KP) {
-            const int l = (k0 + k) * NT;
-            dv[k] = dp[l];
-            av[k] = ap[l];
-            pv[k] = pp[l];
-            ev[k] = ep ? ep[l] : C{0.f, 0.f};
-          }
-        }
-#pragma unroll
-        for (int k = 0; k < UB; ++k)
-          if (k0 + k < KP)
-            srow[2 * (k0 + k) * LD] =
-                pair_phase<float>(pv[k], ev[k], av[k], RN ? renorm_value<float>(dv[k], av[k], it.cm1) : dv[k]);
-      }
-    };
-    if (it.cm1 != 0.f)
-      sweep(std::true_type{});
-    else
-      sweep(std::false_type{});
-  } else {
-    auto run = [&](auto f) {
-#pragma unroll 1
-      for (int k0 = 0; k0 < KP; k0 += UB) {
-        C v[UB];
-#pragma unroll
-        for (int k = 0; k < UB; ++k)
-          if (k0 + k < KP) v[k] = f(off + threadIdx.x + (k0 + k) * NT);
-#pragma unroll
-        for (int k = 0; k < UB; ++k)
-          if (k0 + k < KP) srow[2 * (k0 + k) * LD] = v[k];
-      }
-    };
-    if (it.mode == XF_PHASE_A) {
-      run([&](long long i) { return cmul(it.pv[i], it.in[i]); });
-    } else if (it.mode == XF_PACK_DN) {
-      if (it.r1)
-        run([&](long long i) { return C{it.r0[i], it.r1[i]}; });
-      else
-        run([&](long long i) { return C{it.r0[i], 0.f}; });
-    } else if (it.mode == XF_PACK_PROD) {
-      if (it.r2)
-        run([&](long long i) { return C{it.r0[i] * it.r1[i], it.r2[i] * it.r3[i]}; });
-      else
-        run([&](long long i) { return C{it.r0[i] * it.r1[i], 0.f}; });
-    } else {
-      run([&](long long i) { return preop_at<float>(g, it, i); });
-    }
-  }
-}
 
 // ------------------------------------------------------------------------------------------
 // plane forward pass of the three-pass round trip (Poisson packing of densities and pair
@@ -210,7 +48,7 @@ __global__ void __launch_bounds__(2 * N, N == 96 ? 2 : 3) k_plane_fwd2(GView<flo
   const int z = (int)(blockIdx.x / (unsigned)n_items);
   const long long item = (long long)blockIdx.x - (long long)z * n_items;
   const long long off = (long long)z * NN;
-  preop_plane<N, false>(g, a, item, off, S);
+  preop_plane<N, false>(g, a, item, off, S, threadIdx.x);
   __syncthreads();
   const int lane = threadIdx.x & 31, s = lane >> 4, p = (threadIdx.x >> 5) * 16 + (lane & 15);
   {  // x transforms, pencil p = row p of the tile, in place
@@ -248,44 +86,23 @@ __global__ void __launch_bounds__(2 * N, N == 96 ? 2 : 3) k_plane_fwd2(GView<flo
 // exp(-i dt |G|^2 / 2) = prod_axes exp(-i dt k_a^2 / 2), so in real space it is the product of three
 // one-dimensional operators F_a^-1 K_a F_a, one per axis, which commute. This pass applies the
 // potential phase (the pre-operation) and the x and y operators to one z-plane held in shared
-// memory (kin_roundtrip along each axis); the second sweep applies the z operator. One HBM round trip per sweep: two per step instead of the three of a 3D FFT round trip.
+// memory (kin_roundtrip along each axis); the second sweep applies the z operator. One HBM round trip
+// per sweep: two per step instead of the three of a 3D FFT round trip. 36 pairs of 48^3 x 16 orbitals:
+// 160 + 119 us (three thread-per-pencil sweeps: 147 + 113 + 113; the same two sweeps with a thread per pencil:
+// 208 + 157, held by 12 warps per SM); 10 pairs of 32^3: 14.1 us for the planes.
+
+// blocks per SM that the registers should allow: N points of a lane pair per thread pair
+constexpr int kin2_blocks(int N) { return N == 96 ? 2 : N == 80 ? 3 : N == 64 ? 5 : N == 48 ? 8 : 12; }
 
 template <int N, bool PAIR>
-__global__ void __launch_bounds__(2 * N, N == 96 ? 2 : 3) k_plane_kin2(GView<float> g, XfwdArgs<float> a, int n_items) {
-  using C = float2;
-  constexpr int LD = N + 1, NN = N * N, H = N / 2, Q = H / 2;
+__global__ void __launch_bounds__(2 * N, kin2_blocks(N)) k_plane_kin2(GView<float> g, XfwdArgs<float> a, int n_items) {
+  constexpr int NN = N * N, H = N / 2;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  C *S = reinterpret_cast<C *>(smem_raw);
   const int z = (int)(blockIdx.x / (unsigned)n_items);
   const long long item = (long long)blockIdx.x - (long long)z * n_items;
-  const long long off = (long long)z * NN;
-  __shared__ C tab[3 * H];
+  __shared__ float2 tab[3 * H];
   for (int i = threadIdx.x; i < 3 * H; i += blockDim.x) tab[i] = g.kin[N + i];
-  preop_plane<N, PAIR>(g, a, item, off, S);
-  __syncthreads();
-  const int lane = threadIdx.x & 31, s = lane >> 4, p = (threadIdx.x >> 5) * 16 + (lane & 15);
-  {  // x operator on row p, in place
-    C v[H];
-    C *row = S + p * LD;
-#pragma unroll
-    for (int m = 0; m < H; ++m) v[m] = row[2 * m + s];
-    kin_roundtrip<N>(v, s, tab);
-    __syncwarp();
-#pragma unroll
-    for (int m = 0; m < H; ++m) row[2 * m + s] = v[m];
-  }
-  __syncthreads();
-  {  // y operator on column p, stored to global
-    C v[H];
-    const C *col = S + p;
-#pragma unroll
-    for (int m = 0; m < H; ++m) v[m] = col[(2 * m + s) * LD];
-    kin_roundtrip<N>(v, s, tab);
-    (void)SBSE_IDX(off + p + (long long)(N - 1) * N, g.ng);
-    C *out = a.out + item * g.ng + off + p;
-#pragma unroll
-    for (int m = 0; m < H; ++m) out[(2 * m + s) * N] = v[m];
-  }
+  kin2_plane<N, PAIR>(g, a, item, (long long)z * NN, reinterpret_cast<float2 *>(smem_raw), tab, threadIdx.x);
 }
 
 // Second sweep: the z operator on 64 columns of one item (PLAIN) or of each of the L orbitals of a
@@ -294,7 +111,7 @@ __global__ void __launch_bounds__(2 * N, N == 96 ? 2 : 3) k_plane_kin2(GView<flo
 constexpr int kZDPitch = 80;  // density rows of 64 columns padded so the two half-warps miss each other's banks
 
 template <int N, bool DENS>
-__global__ void __launch_bounds__(128, 3) k_zkin2(GView<float> g, float2 *data, const float2 *a_next, float *dens,
+__global__ void __launch_bounds__(128, N >= 80 ? 3 : DENS || N == 64 ? 4 : 6) k_zkin2(GView<float> g, float2 *data, const float2 *a_next, float *dens,
                                                   int n_units, int L) {
   using C = float2;
   constexpr int NN = N * N, H = N / 2, UB = 16;
@@ -330,7 +147,7 @@ __global__ void __launch_bounds__(128, 3) k_zkin2(GView<float> g, float2 *data, 
         for (int k = 0; k < UB; ++k) {
           if (m0 + k < H) {
             const C dv = v[m0 + k];
-            const float t = 2.f * (2.f * (a0[k].x * dv.x + a0[k].y * dv.y) + dv.x * dv.x + dv.y * dv.y);
+            const float t = density_term<float>(a0[k], dv);
             float &acc = D[(2 * (m0 + k) + s) * kZDPitch + cw];
             acc = ell ? acc + t : t;
           }
@@ -371,11 +188,11 @@ __device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *map, i
 }
 
 template <int N>
-__global__ void __launch_bounds__(2 * kZtCw, 5)
+__global__ void __launch_bounds__(2 * kZtCw, N >= 80 ? 5 : N == 64 ? 7 : 10)
     k_zkin2_tma(const __grid_constant__ CUtensorMap dmap, GView<float> g, float2 *data, const float2 *a_next,
                 float *dens, int n_units, int L, int *err) {
   using C = float2;
-  constexpr int NN = N * N, H = N / 2, UB = 48;
+  constexpr int NN = N * N, H = N / 2, UB = N >= 80 ? 48 : N / 2;
   constexpr unsigned kStage = (unsigned)N * kZtCw * sizeof(C);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned char *smem = smem_raw + ((kZtAlign - (tma_smem_addr(smem_raw) & (kZtAlign - 1))) & (kZtAlign - 1));
@@ -431,7 +248,7 @@ __global__ void __launch_bounds__(2 * kZtCw, 5)
       for (int k = 0; k < UB; ++k) {
         if (m0 + k < H) {
           const C dv = v[m0 + k];
-          const float t = 2.f * (2.f * (a0[k].x * dv.x + a0[k].y * dv.y) + dv.x * dv.x + dv.y * dv.y);
+          const float t = density_term<float>(a0[k], dv);
           float &acc = D[(2 * (m0 + k) + s) * kZtPitch + cw];
           acc = ell ? acc + t : t;
         }
@@ -579,10 +396,12 @@ __global__ void __launch_bounds__(2 * N, N == 96 ? 2 : 3) k_plane_inv2(GView<flo
 
 template <int N> void set_split_attrs() {
   const int sm = (int)split_smem<N>();
-  cudaFuncSetAttribute(k_plane_fwd2<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+  if constexpr (N >= 80) {
+    cudaFuncSetAttribute(k_plane_fwd2<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    cudaFuncSetAttribute(k_plane_inv2<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+  }
   cudaFuncSetAttribute(k_plane_kin2<N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
   cudaFuncSetAttribute(k_plane_kin2<N, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  cudaFuncSetAttribute(k_plane_inv2<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
 }
 
 template <int N> void fwd2(const GridTables<float> &g, const XfwdArgs<float> &a, cudaStream_t s) {
@@ -607,6 +426,14 @@ template <int N>
 void zkin2(const GridTables<float> &g, float2 *d, int n_items, const float2 *a_next, int L, float *dens,
            cudaStream_t s, int *err) {
   const int units = dens ? n_items / L : n_items;
+  if (dens && (long long)units * (N * N / kZtCw) < 608) {
+    // a block works through its pair's L orbitals in turn: where that leaves most of the SMs' schedulers
+    // without a warp, a second kernel sums the density from the stored orbitals (10 pairs x 4 orbitals of 32^3:
+    // 5.5 + 5.7 us; 36 pairs of 48^3 take 119 us in one sweep)
+    k_zkin2<N, false><<<(unsigned)n_items * (N * N / 64), 128, 0, s>>>(view(g), d, nullptr, nullptr, n_items, 1);
+    launch_density<float>(g, d, a_next, units, L, dens, s);
+    return;
+  }
   if (dens && err) {
     // d as n_items orbitals x N z-planes x 2 N^2 floats; boxes of 2 ZT_CW floats x N planes x 1
     CUtensorMap map;
@@ -637,20 +464,14 @@ void inv2(const GridTables<float> &g, float2 *d, int n_units, float *u_out, floa
 }  // namespace
 
 bool split_size(int N) { return N == 80 || N == 96; }
+bool pair_size(int N) { return N == 32 || N == 48 || N == 64; }
 
-int upload_split_twiddles() {
-  float2 hf[kRegTotal];
-  for (int s = 0; s < kRegCount; ++s) {
-    const int N = kRegSizes[s], off = reg_offset(N);
-    for (int k = 0; k < N; ++k) {
-      const double a = -2.0 * M_PI * (double)k / (double)N;
-      hf[off + k] = make_float2((float)cos(a), (float)sin(a));
-    }
-  }
-  return cudaMemcpyToSymbol(c_tws, hf, sizeof(hf)) == cudaSuccess ? 0 : -1;
-}
+int upload_split_twiddles() { return upload_pair_twiddles(); }
 
 void init_split_kernels() {
+  set_split_attrs<32>();
+  set_split_attrs<48>();
+  set_split_attrs<64>();
   set_split_attrs<80>();
   set_split_attrs<96>();
 }
@@ -671,15 +492,27 @@ void launch_plane_inv2_poisson(const GridTables<float> &g, float2 *d, int n_slot
   else if (g.N == 96) inv2<96>(g, d, n_slots, u_out, acc, em1_out, po, s);
 }
 
+#define SBSE_PAIR_SWITCH(N, CALL) \
+  switch (N) {                    \
+    case 32: CALL(32); break;     \
+    case 48: CALL(48); break;     \
+    case 64: CALL(64); break;     \
+    case 80: CALL(80); break;     \
+    case 96: CALL(96); break;     \
+    default: break;               \
+  }
+
 void launch_plane_kin2(const GridTables<float> &g, const XfwdArgs<float> &a, cudaStream_t s) {
-  if (g.N == 80) kin2<80>(g, a, s);
-  else if (g.N == 96) kin2<96>(g, a, s);
+#define SBSE_CALL(n) kin2<n>(g, a, s)
+  SBSE_PAIR_SWITCH(g.N, SBSE_CALL)
+#undef SBSE_CALL
 }
 
 void launch_zkin2(const GridTables<float> &g, float2 *d, int n_items, const float2 *a_next, int L, float *dens,
                   cudaStream_t s, int *err) {
-  if (g.N == 80) zkin2<80>(g, d, n_items, a_next, L, dens, s, err);
-  else if (g.N == 96) zkin2<96>(g, d, n_items, a_next, L, dens, s, err);
+#define SBSE_CALL(n) zkin2<n>(g, d, n_items, a_next, L, dens, s, err)
+  SBSE_PAIR_SWITCH(g.N, SBSE_CALL)
+#undef SBSE_CALL
 }
 
 }  // namespace sbse

@@ -23,9 +23,11 @@ bool make_tensor_map_f32(CUtensorMap *map, const void *base, int rank, const uin
 // ---- register-pencil three-pass round trip (fft_fast.cu), for the sizes fast_supported<T>(N)
 int upload_reg_twiddles();
 int upload_reg_twiddles64();
-// ---- lane-pair split-pencil passes for the grid edges 80 and 96, FP32 (fft_split.cu); the
+// ---- lane-pair split-pencil passes, FP32: every pass of the grid edges 80 and 96 (fft_split.cu); the
 // launchers of fft_fast.cu route those sizes here
 bool split_size(int N);
+// further edges whose FP32 orbitals take the lane-pair sweeps (their Poisson passes are those of fft_fast.cu)
+bool pair_size(int N);
 int upload_split_twiddles();
 void init_split_kernels();
 template <typename T> bool fast_supported(int N);
@@ -35,12 +37,20 @@ template <typename T> void init_fast_kernels();
 bool more_size(int N);
 int upload_more_twiddles();
 template <typename T> void init_more_kernels();
-template <typename T> int more_tiles(int N);
 template <typename T> void launch_more_fwd(const GridTables<T> &g, const XfwdArgs<T> &a, cudaStream_t s);
 template <typename T> void launch_more_z(const GridTables<T> &g, C2<T> *d, int n_items, int mult, cudaStream_t s);
 template <typename T>
-void launch_more_inv(const GridTables<T> &g, C2<T> *d, int n_items, const C2<T> *a_next, int L, T *dens, T *u_out, T *acc,
-                     C2<T> *em1_out, const PoissonOut &po, int mode, cudaStream_t s);
+void launch_more_inv(const GridTables<T> &g, C2<T> *d, int n_items, T *u_out, T *acc, C2<T> *em1_out, const PoissonOut &po,
+                     int mode, cudaStream_t s);
+void launch_more_kin(const GridTables<float> &g, const XfwdArgs<float> &a, cudaStream_t s);
+void launch_more_zkin(const GridTables<float> &g, float2 *d, int n_items, const float2 *a_next, int L, float *dens,
+                      cudaStream_t s);
+// the two sweeps of a split-operator step of the FP32 orbitals on the register-pencil grids (as
+// launch_plane_kin2 / launch_zkin2 on the split sizes). err != null: the pair batch's second sweep may be
+// streamed by bulk copies (bounded waits; *err set if one runs out)
+void launch_kin_planes(const GridTables<float> &g, const XfwdArgs<float> &a, cudaStream_t s);
+void launch_kin_z(const GridTables<float> &g, float2 *d, int n_items, const float2 *a_next, int L, float *dens,
+                  cudaStream_t s, int *err);
 // ---- Poisson passes with four lanes per pencil, for few packed slots (fft_few.cu)
 int upload_few_twiddles();
 template <typename T> bool few_items(int N, long long n_items);
@@ -52,14 +62,10 @@ template <typename T> void launch_few_inv(const GridTables<T> &g, C2<T> *d, int 
 // ---- FFT passes (tdh_kernels.cu). Items are contiguous arrays of ng complex values.
 template <typename T> void launch_xfwd(const GridTables<T> &g, const XfwdArgs<T> &a, cudaStream_t s);
 template <typename T> void launch_plane_fwd(const GridTables<T> &g, const XfwdArgs<T> &a, cudaStream_t s);
-// tma_err != null (FP32, N in 32 / 40 / 48 / 64): the bulk-copy streamed column kernel
-template <typename T> void launch_zcol(const GridTables<T> &g, C2<T> *d, int n_items, int mult, cudaStream_t s,
-                                       int *tma_err = nullptr);
-// tma_err != null (FP32, density epilogue, N in 32 / 40 / 48 / 64): the bulk-copy streamed kernel,
-// which sets *tma_err if one of its bounded waits runs out
+template <typename T> void launch_zcol(const GridTables<T> &g, C2<T> *d, int n_items, int mult, cudaStream_t s);
+// (FP64 orbitals) plane inverse pass, and the pairs' induced density when dens != null
 template <typename T> void launch_plane_inv_orb(const GridTables<T> &g, C2<T> *d, int n_items,
-                                                const C2<T> *a_next, int L, T *dens, cudaStream_t s,
-                                                int *tma_err = nullptr);
+                                                const C2<T> *a_next, int L, T *dens, cudaStream_t s);
 template <typename T> void launch_plane_inv_poisson(const GridTables<T> &g, C2<T> *d, int n_slots,
                                                     const PoissonOut &po, T *u_out, T *acc,
                                                     C2<T> *em1_out, cudaStream_t s);
@@ -223,7 +229,7 @@ void launch_sigma_from_residues(const double *R, int K, const double *cw, const 
 
 // ---- absorption spectrum by a Chebyshev expansion of A (spectrum.cu)
 struct SpectrumBufs {
-  double *f0, *cw, *hist, *R, *D, *omega, *sigma;
+  double *f0, *cw, *hist, *R, *D, *omega, *sigma, *squares;
 };
 size_t spectrum_work_bytes(int n, int n_terms, int n_omega);
 SpectrumBufs spectrum_bufs(double *work, int n, int n_terms, int n_omega);

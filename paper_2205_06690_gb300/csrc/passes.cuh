@@ -103,6 +103,13 @@ __device__ __forceinline__ C2<T> pair_phase(C2<T> pv, C2<T> em1, C2<T> av, C2<T>
   return cmul(pv, cmac2(em1, av, E, dv));
 }
 
+// contribution of one orbital to the induced density of its pair (Eq. 11), 2 (2 Re(conj(eta0) d) + |d|^2), as
+// fixed operations: every kernel that sums it gives the same bits
+template <typename T> __device__ __forceinline__ T density_term(C2<T> a0, C2<T> dv) {
+  const T s = fma(a0.y, dv.y, a0.x * dv.x), q = fma(dv.y, dv.y, dv.x * dv.x);
+  return T(2) * fma(T(2), s, q);
+}
+
 template <typename T>
 __device__ __forceinline__ C2<T> preop_at(const GView<T> &g, const PreopItem<T> &it, long long idx) {
   using C = C2<T>;

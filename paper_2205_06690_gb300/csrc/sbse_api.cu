@@ -107,7 +107,7 @@ struct sbse_ctx {
   int tensor_cores = 1;
   // split-operator step as one persistent kernel (SBSE_OPT_PERSISTENT)
   int persistent = 0;
-  // inverse plane pass of the pair batch streamed by bulk copies (SBSE_OPT_TMA_PLANES)
+  // z sweep of the pair batch streamed by bulk copies (SBSE_OPT_TMA_PLANES)
   int tma_planes = 1;
   // time loop of sbse_apply_W captured once and replayed as a CUDA graph (SBSE_OPT_GRAPH)
   int use_graph = 1;
@@ -300,8 +300,9 @@ template <typename T> int build_tables(sbse_ctx *ctx, GridTables<T> &g, const do
   }
   int rc;
   if ((rc = dalloc(ctx, &g.tw, N * sizeof(C2<T>)))) return rc;
-  // per-axis kinetic factors (N), then for even N the lane-pair round-trip multipliers (3 N / 2)
-  if ((rc = dalloc(ctx, &g.kin, (N + 3 * (N / 2)) * sizeof(C2<T>)))) return rc;
+  // per-axis kinetic factors (N), then for even N the lane-pair round-trip multipliers (3 N / 2), then the
+  // factors over N
+  if ((rc = dalloc(ctx, &g.kin, (2 * N + 3 * (N / 2)) * sizeof(C2<T>)))) return rc;
   if ((rc = dalloc(ctx, &g.k2, N * sizeof(T)))) return rc;
   if ((rc = dalloc(ctx, &g.v_loc, ctx->ng * sizeof(T)))) return rc;
   if ((rc = dalloc(ctx, &g.pv_dt, ctx->ng * sizeof(C2<T>)))) return rc;
@@ -318,7 +319,7 @@ template <typename T> int build_tables(sbse_ctx *ctx, GridTables<T> &g, const do
 // kinetic propagator per axis: exp(-i k_m^2 dt / 2); the 3D factor is the product over axes
 template <typename T> int set_kinetic(sbse_ctx *ctx, GridTables<T> &g, double dt) {
   const int N = ctx->N, H = N / 2;
-  std::vector<C2<T>> kin(N + 3 * H);
+  std::vector<C2<T>> kin(2 * N + 3 * H);
   std::vector<double> kr(N), ki(N);
   for (int m = 0; m < N; ++m) {
     const double kk = kval(m, N, ctx->box);
@@ -326,6 +327,7 @@ template <typename T> int set_kinetic(sbse_ctx *ctx, GridTables<T> &g, double dt
     kr[m] = cos(ph);
     ki[m] = sin(ph);
     kin[m] = C2<T>{(T)kr[m], (T)ki[m]};
+    kin[N + 3 * H + m] = C2<T>{(T)(kr[m] / N), (T)(ki[m] / N)};
   }
   // The one-dimensional kinetic operator F^-1 diag(K) F on the even and odd samples (one per lane
   // of a lane pair): with E, O the half-length transforms, the even outputs are the inverse
@@ -427,18 +429,31 @@ void round_trip_orbitals(sbse_ctx *ctx, const GridTables<T> &g, const XfwdArgs<T
     }
   }
   if (fast_supported<T>(g.N)) {
-    if (parts & RT_FWD_Z) {
-      if (sub) clk_begin(ctx, 5, &ck);
-      launch_plane_fwd<T>(g, fa, st);
-      if (sub) clk_end(ctx, ck);
-      if (sub) clk_begin(ctx, 6, &ck);
-      launch_zcol<T>(g, data, n_items, Z_KINETIC, st, ctx->tma_planes ? ctx->flag : nullptr);
-      if (sub) clk_end(ctx, ck);
-    }
-    if (parts & RT_INV) {
-      if (sub) clk_begin(ctx, 7, &ck);
-      launch_plane_inv_orb<T>(g, data, n_items, a_next, L, dens, st, ctx->tma_planes ? ctx->flag : nullptr);
-      if (sub) clk_end(ctx, ck);
+    if constexpr (sizeof(T) == 4) {
+      if (parts & RT_FWD_Z) {
+        if (sub) clk_begin(ctx, 5, &ck);
+        launch_kin_planes(g, fa, st);
+        if (sub) clk_end(ctx, ck);
+      }
+      if (parts & RT_INV) {
+        if (sub) clk_begin(ctx, 7, &ck);
+        launch_kin_z(g, data, n_items, a_next, L, dens, st, ctx->tma_planes ? ctx->flag : nullptr);
+        if (sub) clk_end(ctx, ck);
+      }
+    } else {
+      if (parts & RT_FWD_Z) {
+        if (sub) clk_begin(ctx, 5, &ck);
+        launch_plane_fwd<T>(g, fa, st);
+        if (sub) clk_end(ctx, ck);
+        if (sub) clk_begin(ctx, 6, &ck);
+        launch_zcol<T>(g, data, n_items, Z_KINETIC, st);
+        if (sub) clk_end(ctx, ck);
+      }
+      if (parts & RT_INV) {
+        if (sub) clk_begin(ctx, 7, &ck);
+        launch_plane_inv_orb<T>(g, data, n_items, a_next, L, dens, st);
+        if (sub) clk_end(ctx, ck);
+      }
     }
   } else {
     if (parts & RT_FWD_Z) {
@@ -641,15 +656,19 @@ int run_apply_W(sbse_ctx *ctx, const sbse_tdh_params *p, const std::vector<int> 
     auto fwd_pair = [&](int j) { for (int l = 0; l < L; ++l) add_orb(SI_P_FWD, j * L + l); };
     auto z_pair = [&](int j) { for (int l = 0; l < L; ++l) add_orb(SI_P_Z, j * L + l); };
     auto inv_pair = [&](int j) { for (int t = 0; t < G; ++t) items.push_back(make_int4(SI_P_INV, j, t, 0)); };
+    // FP32 steps have two sweeps: the z operator of a pair's orbitals and its density are one item
+    constexpr bool two = sizeof(T) == 4;
     for (int l = 0; l < L; ++l) add_orb(SI_A_FWD, l);
     fwd_pair(0);
     for (int l = 0; l < L; ++l) add_orb(SI_A_Z, l);
     if (P > 1) fwd_pair(1);
-    z_pair(0);
-    for (int l = 0; l < L; ++l) add_orb(SI_A_INV, l);
+    if (!two) {
+      z_pair(0);
+      for (int l = 0; l < L; ++l) add_orb(SI_A_INV, l);
+    }
     for (int j = 2; j < P + 2; ++j) {  // pair j forward, pair j-1 z, pair j-2 inverse + density
       if (j < P) fwd_pair(j);
-      if (j - 1 < P) z_pair(j - 1);
+      if (!two && j - 1 < P) z_pair(j - 1);
       inv_pair(j - 2);
     }
     const size_t n_cnt = 2 + 2 * (size_t)L + 2 * (size_t)P * L;

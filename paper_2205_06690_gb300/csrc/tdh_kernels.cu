@@ -550,7 +550,7 @@ __global__ void k_density(long long ng, const C2<T> *d, const C2<T> *a, int L, T
 #pragma unroll 2
   for (int ell = 0; ell < L; ++ell) {
     const C2<T> dv = d[((long long)pair * L + ell) * ng + r], a0 = a[(long long)ell * ng + r];
-    acc += T(2) * (T(2) * (a0.x * dv.x + a0.y * dv.y) + dv.x * dv.x + dv.y * dv.y);
+    acc += density_term<T>(a0, dv);
   }
   dens[(long long)pair * ng + r] = acc;
 }

@@ -90,6 +90,23 @@ def test_bare_potentials_of_few_and_many_slots(B, N, n_o, count):
         assert rel_err(_apply(B, prec, N, box, v, phi, eps, n_o, n_o, 1, prm, pairs)[0], w[pairs[0]].ravel()) < tol
 
 
+@pytest.mark.parametrize("N,n_pairs,n_s", [(18, 15, 2), (24, 3, 3), (32, 3, 3), (32, 21, 1), (40, 6, 1), (48, 3, 2),
+                                           (48, 10, 1), (64, 1, 2), (64, 6, 1)])
+def test_two_sweep_step_of_few_and_many_pairs(B, N, n_pairs, n_s):
+    """Both sides of the rules that sum the density in the z sweep, with and without bulk copies."""
+    n_o, box = 6, 0.4 * N
+    pairs = tdh.pair_list(n_o)[:n_pairs]
+    v, phi, eps = _orbitals(N, box, n_o + 1, N)
+    prm = B.TDHParams(n_s=n_s, n_steps=2, clean_every=0, dt=0.05, gamma=0.1, alpha=1e-4, seed=3)
+    coeff = tdh.stochastic_coefficients(prm.seed, n_s, n_o, "gaussian")
+    op = tdh.TDHParams(n_steps=2, dt=0.05, gamma=0.1, alpha=1e-4, clean_every=0)
+    ref = tdh.screened_potentials(tdh.Grid(N, box), v, phi, n_o, n_o, coeff, op, pairs=pairs)
+    ref = np.stack([ref[p].ravel() for p in pairs])
+    for tma in (0, 1):
+        w = _apply(B, B.SBSE_MIXED, N, box, v, phi, eps, n_o, n_o, 1, prm, pairs, SBSE_OPT_TMA_PLANES=tma)
+        assert rel_err(w, ref) < 2e-3
+
+
 def _eig_noalloc(B, a, k):
     torch = pytest.importorskip("torch")
     d, ev = torch.from_numpy(np.ascontiguousarray(a)).cuda(), torch.empty(k, dtype=torch.float64, device="cuda")
@@ -170,9 +187,13 @@ def test_absorption_of_wide_matrix(B, wide):
     ref, R = _chebyshev(A, f0, 65, 0.1, omega)
     sig, res = c.absorption(1, 65, 0.1, omega)
     assert rel_err(res, R) < 1e-8 and rel_err(sig, ref) < 1e-8
+    ref, R = _chebyshev(A, f0, 2050, 0.1, omega)  # enough terms for rounds of four
+    sig, res = c.absorption(1, 2050, 0.1, omega)
+    assert rel_err(res, R) < 1e-8 and rel_err(sig, ref) < 1e-8
 
 
-@pytest.mark.parametrize("n_o,n_c,terms", [(1, 1, 2), (1, 3, 3), (3, 11, 64), (5, 13, 257)])
+@pytest.mark.parametrize("n_o,n_c,terms", [(1, 1, 2), (1, 3, 3), (3, 11, 64), (5, 13, 257), (1, 3, 63),
+                                          (1, 7, 64), (4, 8, 66), (5, 13, 65), (13, 10, 127)])
 def test_absorption_of_small_matrices(B, n_o, n_c, terms):
     """One block, a row count that is no multiple of a warp's or block's rows, few terms."""
     N, box = 10, 6.0
