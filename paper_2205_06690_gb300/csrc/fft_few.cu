@@ -143,10 +143,11 @@ __global__ void __launch_bounds__(kFewZ) k_few_z(GView<T> g, C2<T> *data, int mu
     for (int k = 0; k < M; ++k) v[k] = cmul(v[k], cmul(mxy, g.kin[fb + k]));
   } else {
     const T gxy = g.k2[x] + g.k2[y];
+    const bool half = mult == Z_HOLE_GRID && item + 1 < n_items;
 #pragma unroll
     for (int k = 0; k < M; ++k) {
       const T G2 = gxy + g.k2[fb + k];
-      v[k] = cscale(v[k], mult == Z_HALF_G2 ? T(0.5) * G2 * inv_ng : (G2 > T(0) ? T(4.0 * M_PI) * inv_ng / G2 : T(0)));
+      v[k] = cscale(v[k], half ? T(0.5) * G2 * inv_ng : (G2 > T(0) ? T(4.0 * M_PI) * inv_ng / G2 : T(0)));
     }
   }
   quad_inv<T, N>(v, q, tw);

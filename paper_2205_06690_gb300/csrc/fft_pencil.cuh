@@ -331,7 +331,7 @@ __device__ __forceinline__ void zcol_column(const GView<T> &g, C2<T> *data, long
     const C mxy = cscale(cmul(g.kin[x], g.kin[y]), inv_ng);
 #pragma unroll
     for (int z = 0; z < N; ++z) v[z] = cmul(v[z], cmul(mxy, g.kin[z]));
-  } else if (mult == Z_HALF_G2) {
+  } else if (mult == Z_HOLE_GRID) {
     const T gxy = g.k2[x] + g.k2[y];
 #pragma unroll
     for (int z = 0; z < N; ++z) v[z] = cscale(v[z], T(0.5) * (gxy + g.k2[z]) * inv_ng);
@@ -354,6 +354,7 @@ __global__ void __launch_bounds__(128) k_zcol(GView<T> g, C2<T> *data, long long
   const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= cols_total) return;
   const long long item = c / NN;
+  if (mult == Z_HOLE_GRID && (item + 1) * NN == cols_total) mult = Z_POISSON;  // the last slot
   zcol_column<T, N, false>(g, data, item, (int)(c - item * NN), mult);
 }
 

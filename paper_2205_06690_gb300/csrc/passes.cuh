@@ -80,8 +80,9 @@ __device__ __forceinline__ PreopItem<T> preop_item(const GView<T> &g, const Xfwd
     it.em1 = a.em1 ? a.em1 + (long long)pair * g.ng : nullptr;
     it.cm1 = a.cm1 ? (T)a.cm1[item] : T(0);
   } else if (a.mode == XF_PACK_DN) {
-    it.r0 = a.dn + 2 * item * g.ng;
-    it.r1 = (2 * item + 1 < a.n_dn) ? a.dn + (2 * item + 1) * g.ng : nullptr;
+    const bool own = a.dn_last && item == a.n_items - 1;
+    it.r0 = own ? a.dn_last : a.dn + 2 * item * g.ng;
+    it.r1 = (!own && 2 * item + 1 < a.n_dn) ? a.dn + (2 * item + 1) * g.ng : nullptr;
   } else {
     const int4 q = a.prod[item];
     it.r0 = a.orb + (long long)q.x * g.ng;

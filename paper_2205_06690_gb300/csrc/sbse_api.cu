@@ -1065,7 +1065,8 @@ template <typename T> int run_direct_block(sbse_ctx *ctx, const std::vector<int>
 
 // ---- mixed hole-grid representation (Sec. II.C): A = Q A-bar on f_j(r), FP64 on the device
 struct MixedBufs {
-  double *tf, *dn, *dv, *pwork, *dwork;
+  double *tf;  // kinetic terms of the rows, padded to full slots, then the potential of the exciton density
+  double *pwork, *dwork;
   C2<double> *pw;
 };
 
@@ -1074,19 +1075,19 @@ int mixed_bufs(sbse_ctx *ctx, int n_extra_fields, MixedBufs *mb, double **extra)
   const int n_o = ctx->n_o;
   // (not monotonic in the number of basis rows: fewer rows are cut into more chunks)
   const size_t pwd = std::max(project_work_doubles(n_o, ctx->n_occ, ng), project_work_doubles(n_o, ctx->n_c, ng));
-  const size_t doubles = (size_t)n_o * ng + 2 * (size_t)ng + pwd + dot_work_doubles() + (size_t)n_extra_fields * n_o * ng;
+  const size_t slots = (size_t)(n_o + 1) / 2 + 1;
+  const size_t doubles = (2 * slots - 1) * ng + dot_work_doubles() + (size_t)n_extra_fields * n_o * ng;
   void *vp;
   int rc;
   if ((rc = ensure(ctx, WS_MIX, doubles * sizeof(double), &vp))) return rc;
   double *p = (double *)vp;
   mb->tf = p;
-  mb->dn = mb->tf + (long long)n_o * ng;
-  mb->dv = mb->dn + ng;
-  mb->pwork = mb->dv + ng;
-  mb->dwork = mb->pwork + pwd;
+  mb->dwork = mb->tf + (2 * slots - 1) * ng;
   *extra = mb->dwork + dot_work_doubles();
-  if ((rc = ensure(ctx, WS_PW, (size_t)((n_o + 1) / 2) * ng * sizeof(C2<double>), &vp))) return rc;
+  // the packed slots, and the projections' partial sums when the slots are done with
+  if ((rc = ensure(ctx, WS_PW, std::max(slots * (size_t)ng * sizeof(C2<double>), pwd * sizeof(double)), &vp))) return rc;
   mb->pw = (C2<double> *)vp;
+  mb->pwork = (double *)vp;
   return SBSE_OK;
 }
 
@@ -1099,15 +1100,19 @@ int mixed_apply(sbse_ctx *ctx, int projector, const double *f, double *out, doub
   cudaStream_t st = ctx->stream;
   XfwdArgs<double> xa{};
   xa.mode = XF_PACK_DN;
-  xa.n_items = (n_o + 1) / 2;
+  // One round trip for the kinetic terms of the rows and the potential of the exciton density (held in `out`
+  // until the operator writes it): the passes of a few slots leave most SMs idle, so the density's slot is
+  // free (4 rows of 32^3: 106 us per term of the expansion, 159 with two trips).
+  launch_exciton_density(phi_o, f, n_o, ng, out, st);
+  const int slots = (n_o + 1) / 2 + 1;
+  xa.n_items = slots;
   xa.out = mb.pw;
   xa.dn = f;
   xa.n_dn = n_o;
-  round_trip_poisson<double>(ctx, ctx->g64, xa, PoissonOut{n_o, 1.0, 0.0, 0.0}, mb.tf, nullptr, nullptr, Z_HALF_G2);
-  launch_exciton_density(phi_o, f, n_o, ng, mb.dn, st);
-  int rc;
-  if ((rc = poisson<double>(ctx, ctx->g64, mb.dn, 1, mb.pw, mb.dv, nullptr, 0.0, nullptr, 0.0))) return rc;
-  launch_abar(mb.tf, f, ctx->v64, ctx->eps_dev, ctx->scissor, shift, mb.dv, phi_o, ctx->W, n_o, ng, out, st);
+  xa.dn_last = out;
+  round_trip_poisson<double>(ctx, ctx->g64, xa, PoissonOut{2 * slots - 1, 1.0, 0.0, 0.0}, mb.tf, nullptr, nullptr, Z_HOLE_GRID);
+  const double *dv = mb.tf + (long long)(2 * slots - 2) * ng;
+  launch_abar(mb.tf, f, ctx->v64, ctx->eps_dev, ctx->scissor, shift, dv, phi_o, ctx->W, n_o, ng, out, st);
   if (projector == 0)
     launch_project(out, n_o, ctx->phi64, ctx->n_occ, ng, ctx->dV, 0, mb.pwork, st);
   else

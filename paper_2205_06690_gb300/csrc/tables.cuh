@@ -39,6 +39,7 @@ template <typename T> struct XfwdArgs {
   int L;                 // PAIR: orbitals per pair
   const T *dn;           // PACK_DN: density per pair; slot s packs 2s (re) and 2s+1 (im)
   int n_dn;              // PACK_DN: number of densities
+  const T *dn_last;      // PACK_DN: the only density of the last slot (null: as the others)
   const T *orb;          // PACK_PROD: orbital rows (ng each)
   const int4 *prod;      // PACK_PROD: per slot (i1, j1, i2, j2); i2 < 0 -> imaginary part 0
 };
@@ -54,7 +55,8 @@ struct PoissonOut {
 
 // multiplier of the z pass: kinetic propagator, Coulomb kernel 4 pi / |G|^2 (G = 0 dropped), or the
 // kinetic energy |G|^2 / 2 (the spectral -1/2 Laplacian); each with the 1/N^3 of the round trip
-enum ZMult { Z_KINETIC = 0, Z_POISSON = 1, Z_HALF_G2 = 2 };
+// Z_HOLE_GRID: G^2 / 2 (kinetic energy) for every slot but the last, 4 pi / G^2 for the last
+enum ZMult { Z_KINETIC = 0, Z_POISSON = 1, Z_HOLE_GRID = 2 };
 
 // tile queue and completion counters of the persistent split-operator step (fft_fast.cu)
 enum StepItemKind { SI_A_FWD = 0, SI_A_Z = 1, SI_A_INV = 2, SI_P_FWD = 3, SI_P_Z = 4, SI_P_INV = 5 };
