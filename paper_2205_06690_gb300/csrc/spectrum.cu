@@ -59,6 +59,10 @@ __global__ void __launch_bounds__(kSpT)
   if (threadIdx.x == 0) f0[blockIdx.x] = s * dV;
 }
 
+// a vector entry as it is stored: every NaN as the one with this payload, so that none equals kUnset
+constexpr unsigned long long kUnset = ~0ull;
+__device__ __forceinline__ double entry(double v) { return v == v ? v : __longlong_as_double(0x7ff8000000000000ll); }
+
 // cw = {c, w} from the Gershgorin discs of the rows of A (a warp per row), and v_0 = f0
 constexpr int kInitT = 1024;
 __global__ void __launch_bounds__(kInitT) k_cheb_init(const double *A, int n, const double *f0, double *cw, double *v0) {
@@ -74,7 +78,7 @@ __global__ void __launch_bounds__(kInitT) k_cheb_init(const double *A, int n, co
     lo = fmin(lo, d - rad);
     hi = fmax(hi, d + rad);
   }
-  for (int r = threadIdx.x; r < n; r += kInitT) v0[r] = f0[r];
+  for (int r = threadIdx.x; r < n; r += kInitT) v0[r] = entry(f0[r]);
   if (lane == 0) {
     slo[warp] = lo;
     shi[warp] = hi;
@@ -93,14 +97,13 @@ __global__ void __launch_bounds__(kInitT) k_cheb_init(const double *A, int n, co
 // The recursion with a stride of S terms, in one cooperative launch: v_{t+S} = 2 T_S(A~) v_t - v_{t-S}
 // advances the S vectors of a round by one matrix (S = 1: A~ itself). Every v_t is kept as row t of `hist`.
 // A warp per row of the matrix (rows stay in the SM's L1), the round's vectors staged in shared memory.
-// The rows of hist are filled with an all-ones bit pattern first (a NaN that no arithmetic produces), and a
+// The rows of hist are filled with an all-ones bit pattern first (a NaN that `entry` never lets through), and a
 // block waits for the entries of the round themselves, so a round costs one store-to-load trip through L2
 // and S dot products (FP64-bound: about 1 us each for 512 rows), and no barrier. 4095 terms of a 512 x 512
 // A took 25.6 ms as separate launches, 23.9 ms with a grid barrier per term, 13.0 ms with S = 1, and take
 // 7.4 ms with S = 4 including the two products that make T_4(A~). Every wait is bounded; one that runs
 // out sets *err and the block leaves.
 constexpr unsigned kPollLimit = 1u << 21;
-constexpr unsigned long long kUnset = ~0ull;
 
 // mat: A with cw = {c, w} (S = 1, mat = A, scaled on the fly), or T_S(A~) with cw = null. STAGED: the round's
 // vectors in shared memory, and (rows) the first row of each warp as well.
@@ -186,7 +189,7 @@ __global__ void k_cheb_run(const double *mat, int n, const double *cw, double *h
           before = mine == 0 ? at : (STAGED ? sv[(S - mine) * n + r] : __ldcg(hist + (long long)(S - mine) * n + r));
         else
           before = r == r0 ? v_old : __ldcg(hist + (long long)(t - S + mine) * n + r);
-        const double v = 2.0 * at - before;
+        const double v = entry(2.0 * at - before);
         asm volatile("st.relaxed.gpu.global.f64 [%0], %1;" ::"l"(hist + (long long)tn * n + r), "d"(v) : "memory");
         if (r == r0) v_old = vr;
       }
@@ -234,7 +237,7 @@ template <class M> __global__ void __launch_bounds__(kSpT) k_cheb_first(M m, int
   double s = 0.0;
   for (int j = lane; j < n; j += 32) s = fma(m.at(r, j), x[j], s);
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (lane == 0) y[r] = third ? 2.0 * s - x[r] : s;
+  if (lane == 0) y[r] = entry(third ? 2.0 * s - x[r] : s);
 }
 
 constexpr int kStride = 4, kSqChunks = 4;
@@ -277,7 +280,7 @@ __global__ void __launch_bounds__(kSpT) k_cheb_density(const double *R, int K, c
 }
 
 // sigma_j = omega_j / K sum_k G_s(c + w x_k - omega_j) D_k: a block per frequency (before: a thread, four
-// blocks for 400 frequencies, 8.9 ms; here 54 us). Gaussians below the smallest FP64 number are skipped.
+// blocks for 400 frequencies, 8.9 ms; here 54 us). Gaussians below the smallest FP64 number are not evaluated.
 __global__ void __launch_bounds__(kSpT)
     k_sigma(const double *D, int K, const double *tab, const double *cw, const double *omega, int n_omega, double s,
             double *sigma) {
@@ -289,7 +292,7 @@ __global__ void __launch_bounds__(kSpT)
     for (int k = threadIdx.x; k < K; k += kSpT) {
       const double e = (c + w * tab[2 * k + 1] - om) / s;
       const double q = e * e;
-      if (!(q > 1500.0)) acc = fma(exp(-0.5 * q), D[k], acc);
+      acc = fma(q > 1500.0 ? 0.0 : exp(-0.5 * q), D[k], acc);  // (a D that is not finite stays one)
     }
     acc = block_sum_fixed(acc, red);
     if (threadIdx.x == 0) sigma[j] = om * norm * acc / (double)K;

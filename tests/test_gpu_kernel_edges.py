@@ -274,3 +274,17 @@ def test_fno_planes_beyond_shared_memory(B):
     net.forward(1, xd.data_ptr(), yd.data_ptr())
     assert rel_err(yd.cpu().numpy(), ofno.forward(_unpack(vec, C, m, L, round_bf16=True), x.astype(np.float64), m)) < 1e-4
     net.close()
+
+
+def test_absorption_without_interval_is_not_finite(B):
+    """One row leaves no interval to scale: the vectors are NaN, and the call says so instead of waiting."""
+    N, box = 10, 6.0
+    v, phi, eps = _orbitals(N, box, 2, 1)
+    with B.Context(0, B.SBSE_FP64) as c:
+        c.set_grid(N, box, v)
+        c.set_orbitals(1, 1, 1, phi, eps, 0.5)
+        c.build_A(B.SBSE_EXCHANGE)
+        for terms, omega in ((2, 1.0), (70, 1.0), (70, 1e3)):  # (far from every Gaussian as well)
+            with pytest.raises(B.SbseError) as e:
+                c.absorption(0, terms, 0.2, np.array([omega]))
+            assert e.value.code == B.SBSE_ERR_NUMERIC
