@@ -303,15 +303,15 @@ __global__ void __launch_bounds__(kSpT)
 
 size_t sigma_work_doubles(int K) { return 5 * (size_t)K; }  // D, then the cosine table
 
-size_t spectrum_work_bytes(int n, int n_terms, int n_omega) {
+size_t spectrum_work_bytes(int n, int n_terms, int n_omega, bool squares) {
   // f0, cw, the vectors (n_terms x n), R, D and its cosine table, omega, sigma; T_2, T_4 and the chunks of
   // their products
-  const size_t nn = cheb_strided(n, n_terms) ? (size_t)n * n : 0;
+  const size_t nn = squares && cheb_strided(n, n_terms) ? (size_t)n * n : 0;
   return sizeof(double) * ((size_t)n + 2 + (size_t)n * n_terms + (size_t)n_terms + sigma_work_doubles(n_terms) +
                            2 * (size_t)n_omega + (2 + kSqChunks) * nn);
 }
 
-SpectrumBufs spectrum_bufs(double *work, int n, int n_terms, int n_omega) {
+SpectrumBufs spectrum_bufs(double *work, int n, int n_terms, int n_omega, bool squares) {
   SpectrumBufs b{};
   b.f0 = work;
   b.cw = b.f0 + n;
@@ -320,7 +320,7 @@ SpectrumBufs spectrum_bufs(double *work, int n, int n_terms, int n_omega) {
   b.D = b.R + n_terms;
   b.omega = b.D + sigma_work_doubles(n_terms);
   b.sigma = b.omega + n_omega;
-  b.squares = b.sigma + n_omega;
+  b.squares = squares && cheb_strided(n, n_terms) ? b.sigma + n_omega : nullptr;
   return b;
 }
 
@@ -341,7 +341,7 @@ bool launch_absorption(const SpectrumBufs &b, const double *phi_o, const double 
   cudaMemsetAsync(b.hist, 0xff, (size_t)n * n_terms * sizeof(double), st);
   k_cheb_init<<<1, kInitT, 0, st>>>(A, n, b.f0, b.cw, b.hist);
   count_launch(2);
-  const bool strided = cheb_strided(n, n_terms);
+  const bool strided = b.squares != nullptr;
   const double *mat = A, *cw = b.cw;
   if (strided) {
     // T_2 = 2 A~ A~ - 1, T_4 = 2 T_2 T_2 - 1; v_1 = A~ v_0, v_2 = T_2 v_0, v_3 = 2 T_2 v_1 - v_1

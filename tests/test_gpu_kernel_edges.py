@@ -288,3 +288,35 @@ def test_absorption_without_interval_is_not_finite(B):
             with pytest.raises(B.SbseError) as e:
                 c.absorption(0, terms, 0.2, np.array([omega]))
             assert e.value.code == B.SBSE_ERR_NUMERIC
+
+
+def test_absorption_at_a_memory_limit(B):
+    """A context without room for the matrix squares (10 MiB at 462 rows) takes single terms: it needs no
+    more than the vectors above what few terms need, and gives the same spectrum."""
+    N, box, n_o, n_c, few, many = 10, 6.0, 21, 22, 63, 1024
+    v, phi, eps = _orbitals(N, box, n_o + n_c, 3)
+    omega = np.linspace(0.1, 4.0, 5)
+    n = n_o * n_c
+
+    def least(terms):
+        with B.Context(0, B.SBSE_FP64) as c:
+            c.set_grid(N, box, v)
+            c.set_orbitals(n_o, n_o, n_c, phi, eps, 0.5)
+            c.build_A(B.SBSE_EXCHANGE)
+            for limit in range(1, 200):
+                B.sbse_set_option(c.h, B.SBSE_OPT_MEM_LIMIT_MB, limit)
+                try:
+                    at_limit = c.absorption(0, terms, 0.2, omega)
+                except B.SbseError as e:
+                    assert e.code == B.SBSE_ERR_OOM
+                    continue
+                break
+        with B.Context(0, B.SBSE_FP64) as c:
+            c.set_grid(N, box, v)
+            c.set_orbitals(n_o, n_o, n_c, phi, eps, 0.5)
+            c.build_A(B.SBSE_EXCHANGE)
+            free = c.absorption(0, terms, 0.2, omega)
+        assert all(rel_err(a, b) < 1e-8 for a, b in zip(at_limit, free))
+        return limit
+
+    assert least(many) <= least(few) + ((n + 6) * (many - few) * 8 >> 20) + 2
