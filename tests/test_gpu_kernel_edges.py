@@ -320,3 +320,21 @@ def test_absorption_at_a_memory_limit(B):
         return limit
 
     assert least(many) <= least(few) + ((n + 6) * (many - few) * 8 >> 20) + 2
+
+
+@pytest.mark.parametrize("N,C,batch", [(9, 5, 2), (24, 33, 1), (32, 64, 1)])
+def test_fno_bias_gradient_of_cancelling_fields(B, N, C, batch):
+    """Sums that cancel to a small part of their terms: rounded to FP32 once (2^-23), after pairs of floats
+    over at most 1024 points (1024 2^-46 of the absolute sum)."""
+    torch = pytest.importorskip("torch")
+    net = B.FNO(N, width=C, modes=2, layers=1, max_batch=batch)
+    net.set_params(_pack(ofno.init_params(C, 2, 1, seed=N)))
+    rng = np.random.default_rng(N)
+    dy = rng.standard_normal((batch, N, N, N))
+    dy = (dy - dy.mean() + 1e-4 / N ** 3).astype(np.float32)
+    xd, dyd = torch.zeros((batch, 2, N, N, N), device="cuda"), torch.from_numpy(dy).cuda()
+    torch.cuda.synchronize()
+    net.gradients(batch, xd.data_ptr(), dyd.data_ptr())
+    got, ref = float(net.get_params()[1][-1]), float(dy.sum(dtype=np.float64))
+    assert abs(got - ref) <= 2.0 ** -23 * abs(ref) + 2.0 ** -36 * float(np.abs(dy).sum(dtype=np.float64))
+    net.close()
