@@ -15,6 +15,7 @@
 #include <utility>
 #include <vector>
 
+#include "gemm_nt.cuh"
 #include "kernels.h"
 #include "sbse.h"
 
@@ -417,11 +418,12 @@ void forward_impl(sbse_fno *f, int B, const float *x, bool keep_u) {
   count_launch(1);
 }
 
-// weight gradient w[M][Nn] = sum_{b,r} A[b][row][r] Bm[b][col][r], and bias[M] = sum_{b,r} A (if not null)
+// weight gradient w[M][Nn] = sum_{b,r} A[b][row][r] Bm[b][col][r], and bias[M] = sum_{b,r} A
 int wgrad(sbse_fno *f, const float *A, int M, const float *Bm, int Nn, int B, float *w, float *bias) {
   const long long chunks_b = (f->ng + kWgChunk - 1) / kWgChunk, chunks = chunks_b * B;
+  const long long K = (long long)B * f->ng, kc = gemm_kchunk(K), kchunks = (K + kc - 1) / kc;
   const int cols = M * (Nn + 1);
-  const size_t need = (size_t)chunks * cols * sizeof(double);
+  const size_t need = ((size_t)chunks * cols + (size_t)kchunks * M) * sizeof(double);
   if (need > f->gpart_cap) {
     if (f->gpart) cudaFree(f->gpart);
     f->gpart = nullptr;
@@ -430,11 +432,14 @@ int wgrad(sbse_fno *f, const float *A, int M, const float *Bm, int Nn, int B, fl
     if (rc) return rc;
     f->gpart_cap = need;
   }
+  double *rpart = f->gpart + chunks * cols, *plain = f->gout + cols;
   k_fo_wgrad<<<(unsigned)chunks, kWgT, wg_smem(M, Nn), f->stream>>>(A, M, Bm, Nn, f->ng, chunks_b, f->gpart);
-  count_launch(1);
   launch_reduce_cols(f->gpart, (int)chunks, cols, 1.0, f->gout, f->stream);
-  k_fo_wgrad_out<<<nblk(cols), kT, 0, f->stream>>>(f->gout, M, Nn, w, bias);
-  count_launch(1);
+  dim3 grid((unsigned)kchunks, (unsigned)((M + kBsRows - 1) / kBsRows));
+  k_fo_row_sums<<<grid, kBsT, 0, f->stream>>>(A, M, f->ng, K, kc, rpart);
+  launch_reduce_cols(rpart, (int)kchunks, M, 1.0, plain, f->stream);
+  k_fo_wgrad_out<<<nblk(cols), kT, 0, f->stream>>>(f->gout, plain, M, Nn, w, bias);
+  count_launch(3);
   return SBSE_OK;
 }
 

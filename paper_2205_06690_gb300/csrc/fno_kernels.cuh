@@ -565,11 +565,12 @@ __global__ void __launch_bounds__(kPwT)
 
 // ---- weight gradients -------------------------------------------------------------------------------
 // part[chunk][i][j] = sum over a chunk of points of A[b][i][r] B[b][j][r], i < M, j < Nn, and for j = Nn
-// the sum of A[b][i][r] (the bias gradient): M, Nn <= 64 channels. 4 x 4 outputs per thread, the
+// the sum of A[b][i][r]: M, Nn <= 64 channels. 4 x 4 outputs per thread, the
 // threads left over split the points of a tile and are summed at the end. Chunks are summed in FP32
-// and stored in FP64 partials; the sums of A, which cancel most, as pairs of floats (Knuth's two-sum). Bound by shared-memory reads (8 per 16 multiply-adds). 32 x 32 over
+// and stored in FP64 partials; the sums of A, which cancel most, as pairs of floats (Knuth's two-sum) for
+// k_fo_wgrad_out. Bound by shared-memory reads (8 per 16 multiply-adds). 32 x 32 over
 // 4 x 64^3 points: about 320 us (829 us, and 510 us for the bias alone, by the 64 x 64 tile GEMM).
-// Three blocks per SM (80 registers): the gradients of the 64^3 network take 6.12 ms, 6.48 ms with two.
+// Three blocks per SM (80 registers): the gradients of the 64^3 network take 0.36 ms less than with two.
 constexpr int kWgT = 256, kWgK = 64, kWgChunk = 1024;
 
 inline size_t wg_smem(int M, int Nn) { return 2 * (size_t)(M + Nn) * (kWgK + 1) * sizeof(float); }
@@ -670,13 +671,62 @@ __global__ void __launch_bounds__(kWgT, 3)
   }
 }
 
-// FP64 sums [M][Nn + 1] -> weight gradient [M][Nn] and bias gradient [M]
-__global__ void k_fo_wgrad_out(const double *g, int M, int Nn, float *w, float *bias) {
+// part[chunk][i] = sum over a chunk of the points k = b ng + r of A[b][i][r], one FP32 addition after the
+// other. The order is part of the result: a bias gradient is a sum that cancels, so its last digits are those of the
+// order of its additions. A lane of the last warp adds the points of a row, from a ring of tiles that the
+// other warps keep three ahead. Bound by the chain of 4096 additions and the latency of the tiles: 43 us for 32
+// rows over 4 x 64^3 points (24 us for one row).
+constexpr int kBsLoad = 256, kBsT = kBsLoad + 32, kBsRows = 32, kBsP = 64, kBsStages = 4;
+__global__ void __launch_bounds__(kBsT)
+    k_fo_row_sums(const float *A, int M, long long ng, long long K, long long kchunk, double *part) {
+  __shared__ float tile[kBsStages][kBsRows * (kBsP + 1)];
+  const int m0 = blockIdx.y * kBsRows, rows = min(kBsRows, M - m0);
+  const long long kbeg = (long long)blockIdx.x * kchunk, kend = min(kbeg + kchunk, K);
+  const int n_tiles = (int)((kend - kbeg + kBsP - 1) / kBsP), m = (int)threadIdx.x - kBsLoad;
+  const int p = threadIdx.x % kBsP;  // the same point of every row of a tile
+  long long k = kbeg + p, b = k / ng, r = k - b * ng;
+  auto load = [&](int it) {  // tiles in order; past the last one an empty group
+    if (it < n_tiles) {
+      const bool in = k < kend;
+      const float *src = in ? A + (b * M + m0) * ng + r : A;
+      for (int c = threadIdx.x / kBsP; c < rows; c += kBsLoad / kBsP)
+        cp_async4(&tile[it % kBsStages][c * (kBsP + 1) + p], src + (in ? c * ng : 0), in);
+      k += kBsP;
+      for (r += kBsP; r >= ng; r -= ng) ++b;
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  float s = 0.f;
+  if (m < 0)
+    for (int it = 0; it < kBsStages - 1; ++it) load(it);
+  for (int it = 0; it < n_tiles; ++it) {
+    if (m < 0) asm volatile("cp.async.wait_group %0;" ::"n"(kBsStages - 2) : "memory");
+    __syncthreads();  // tile `it` is there, and the one before it is summed: its place is free
+    if (m < 0) {
+      load(it + kBsStages - 1);
+    } else if (m < rows) {
+      const float *row = tile[it % kBsStages] + m * (kBsP + 1);
+      float v[kBsP];
+#pragma unroll
+      for (int q = 0; q < kBsP; ++q) v[q] = row[q];
+#pragma unroll
+      for (int q = 0; q < kBsP; ++q) s += v[q];
+    }
+  }
+  if (m >= 0 && m < rows) part[(long long)blockIdx.x * M + m0 + m] = (double)s;
+}
+
+// FP64 sums g[M][Nn + 1] (the last column as pairs of floats) and plain[M] (in order, k_fo_row_sums) -> weight
+// gradient [M][Nn] and bias gradient [M]. The bias gradient is the plain sum, infinities included, unless
+// cancellation leaves it less than ten right bits: then it is the sum of the pairs.
+__global__ void k_fo_wgrad_out(const double *g, const double *plain, int M, int Nn, float *w, float *bias) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= M * (Nn + 1)) return;
   const int i = t / (Nn + 1), j = t - i * (Nn + 1);
-  if (j < Nn) w[i * Nn + j] = (float)g[t];
-  else if (bias) bias[i] = (float)g[t];
+  if (j < Nn)
+    w[i * Nn + j] = (float)g[t];
+  else if (bias)
+    bias[i] = (float)(fabs(plain[i] - g[t]) > 0x1p-10 * fabs(g[t]) ? g[t] : plain[i]);
 }
 
 }  // namespace sbse

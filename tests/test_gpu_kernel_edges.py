@@ -338,3 +338,35 @@ def test_fno_bias_gradient_of_cancelling_fields(B, N, C, batch):
     got, ref = float(net.get_params()[1][-1]), float(dy.sum(dtype=np.float64))
     assert abs(got - ref) <= 2.0 ** -23 * abs(ref) + 2.0 ** -36 * float(np.abs(dy).sum(dtype=np.float64))
     net.close()
+
+
+@pytest.mark.parametrize("N,C,batch", [(9, 5, 2), (16, 32, 1), (24, 33, 3)])
+def test_fno_bias_gradients_add_in_order(B, N, C, batch):
+    """Bias gradients are the FP32 sums of 4096 points in a row, chunks joined in FP64, to the bit (one chunk
+    that is not full, a full one, a full one and a remainder across batch entries; 5, 32 and 33 rows), and keep
+    an infinite entry."""
+    torch = pytest.importorskip("torch")
+    net = B.FNO(N, width=C, modes=2, layers=1, max_batch=batch)
+    vec = _pack(ofno.init_params(C, 2, 1, seed=N))
+    net.set_params(vec)
+    w = vec[-1 - C:-1]  # the projection: dL/dU of the only layer is w[c] dy
+    xd = torch.zeros((batch, 2, N, N, N), device="cuda")
+
+    def bias(dy):
+        d = torch.from_numpy(dy).cuda()
+        torch.cuda.synchronize()
+        net.gradients(batch, xd.data_ptr(), d.data_ptr())
+        g = net.get_params()[1]
+        return np.append(g[-1 - 2 * C:-1 - C], g[-1])
+
+    def in_order(x):
+        return np.float32(sum(float(np.add.accumulate(x[k:k + 4096], dtype=np.float32)[-1]) for k in range(0, x.size, 4096)))
+
+    dy = np.random.default_rng(N).standard_normal((batch, N, N, N)).astype(np.float32)
+    ref = np.array([in_order((c * dy).ravel()) for c in np.append(w, np.float32(1))])
+    exact = float(dy.sum(dtype=np.float64))
+    assert abs(float(ref[-1]) - exact) < 2.0 ** -12 * abs(exact)  # (sums that keep their leading bits)
+    assert np.array_equal(bias(dy), ref)
+    dy[-1, 1, 2, 3] = np.inf
+    assert np.array_equal(bias(dy), np.copysign(np.float32(np.inf), np.append(w, np.float32(1))))
+    net.close()
