@@ -1,6 +1,6 @@
 // Lowest eigenvalues of the real symmetric Tamm-Dancoff matrix A (Eq. 1), in FP64 on the device:
 // Householder reduction to tridiagonal form (one thread-block cluster, the matrix in its distributed
-// shared memory) followed by Sturm-sequence multisection, one warp per requested eigenvalue.
+// shared memory) followed by Sturm-sequence multisection, one block per requested eigenvalue.
 #include <cooperative_groups.h>
 #include <math.h>
 
@@ -315,6 +315,8 @@ __device__ __forceinline__ int sturm_count(const double *ds, const double *es, i
 // on each of the SM's sub-partitions costs no more time than one warp). Eight warps of eight
 // eigenvalues on one SM with the quotient form took 5.9 ms for ten eigenvalues at n = 512, this 0.58 ms;
 // at n = 128, 1.48 ms and 0.15 ms.
+// A tridiagonal with an entry that is not finite has no eigenvalues: NaN (fmin and fmax pass over a NaN, so
+// bounds and norm do not show it).
 constexpr int kBisT = 128;
 __global__ void __launch_bounds__(kBisT) k_bisect(const double *dg, const double *of, int n, int k, double *ev) {
   extern __shared__ double sm[];
@@ -322,8 +324,10 @@ __global__ void __launch_bounds__(kBisT) k_bisect(const double *dg, const double
   double *ds = sm, *es = sm + n;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, j = blockIdx.x;
   double lo = dg[0], hi = dg[0], nrm = 0.0;
+  bool finite = true;
   for (int i = threadIdx.x; i < n; i += kBisT) {
     const double d = dg[i];
+    finite = finite && fabs(d) < INFINITY && (i == n - 1 || fabs(of[i]) < INFINITY);
     const double r = (i > 0 ? fabs(of[i - 1]) : 0.0) + (i < n - 1 ? fabs(of[i]) : 0.0);
     lo = fmin(lo, d - r);
     hi = fmax(hi, d + r);
@@ -339,7 +343,10 @@ __global__ void __launch_bounds__(kBisT) k_bisect(const double *dg, const double
     bound[1][warp] = hi;
     bound[2][warp] = nrm;
   }
-  __syncthreads();
+  if (!__syncthreads_and(finite)) {
+    if (threadIdx.x == 0) ev[j] = NAN;
+    return;
+  }
   for (int w = 0; w < kBisT / 32; ++w) {
     lo = fmin(lo, bound[0][w]);
     hi = fmax(hi, bound[1][w]);

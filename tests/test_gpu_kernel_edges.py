@@ -370,3 +370,39 @@ def test_fno_bias_gradients_add_in_order(B, N, C, batch):
     dy[-1, 1, 2, 3] = np.inf
     assert np.array_equal(bias(dy), np.copysign(np.float32(np.inf), np.append(w, np.float32(1))))
     net.close()
+
+
+@pytest.mark.parametrize("n", [1, 2, 3, 40, 257])
+@pytest.mark.parametrize("where", ["all", "corner", "last", "inf"])
+def test_eigenvalues_of_matrices_that_are_not_finite(B, n, where):
+    """No eigenvalue comes out as a number, the zero of a vanishing matrix least of all."""
+    a = _sym(n, "dense")
+    if where == "all":
+        a[:] = np.nan
+    elif where == "corner":  # the first row and column stay finite
+        a[n // 2:, n // 2:] = np.nan
+    elif where == "last":
+        a[n - 1, n - 1] = np.nan
+    else:
+        a[0, n - 1] = a[n - 1, 0] = np.inf
+    assert np.all(np.isnan(_eig_noalloc(B, a, min(n, 12))))
+
+
+def test_spectrum_of_a_diverged_surrogate_is_refused(B):
+    """W fields that are NaN reach A unchecked; eigenvalues and vectors of it are a numeric error."""
+    torch = pytest.importorskip("torch")
+    N, box, n_o, n_c = 10, 6.0, 3, 4
+    v, phi, eps = _orbitals(N, box, n_o + n_c, 4)
+    pairs = tdh.pair_list(n_o)
+    y = torch.full((len(pairs), N, N, N), float("nan"), device="cuda")
+    torch.cuda.synchronize()
+    with B.Context(0, B.SBSE_FP64) as c:
+        c.set_grid(N, box, v)
+        c.set_orbitals(n_o, n_o, n_c, phi, eps, 0.5)
+        B.sbse_bare_W(c.h, pairs)
+        B.sbse_add_W(c.h, pairs, y.data_ptr(), 1.0)
+        c.build_A()
+        for vectors in (False, True):
+            with pytest.raises(B.SbseError) as e:
+                c.spectrum(5, vectors=vectors)
+            assert e.value.code == B.SBSE_ERR_NUMERIC
