@@ -16,6 +16,7 @@
 
 #include "kernels.h"
 #include "sbse.h"
+#include "smem_limit.h"
 
 namespace {
 thread_local std::string g_create_error;
@@ -32,16 +33,13 @@ static std::vector<int (*)(unsigned long long *)> &bounds_readers() {
   return r;
 }
 void register_bounds_reader(int (*reader)(unsigned long long *)) { bounds_readers().push_back(reader); }
-// The dynamic shared memory limit is an attribute of the kernel, shared by every context and host
-// thread: lowering it for one launch could make another thread's larger launch of the same kernel
-// fail in between. So it is only ever raised, under a lock.
 void raise_smem_limit(const void *fn, size_t bytes) {
-  static std::mutex mx;
-  static std::unordered_map<const void *, size_t> cur;
-  std::lock_guard<std::mutex> lk(mx);
-  size_t &c = cur[fn];
-  if (bytes > c && cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) == cudaSuccess)
-    c = bytes;
+  static SmemLimits limits;
+  int device = 0;
+  if (cudaGetDevice(&device) != cudaSuccess) return;
+  limits.raise(device, fn, bytes, [fn](size_t n) {
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)n) == cudaSuccess;
+  });
 }
 }
 
