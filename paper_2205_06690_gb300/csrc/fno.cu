@@ -371,15 +371,26 @@ void mix_backward(sbse_fno *f, float2 *F, const float2 *dG, const __nv_bfloat16 
   }
 }
 
+// kernels with the batch in gridDim.y: launch(first batch entry, entries), at most kMaxGridY at a time
+constexpr int kMaxGridY = 65535;
+template <class F> void over_batch(int B, F launch) {
+  for (int b0 = 0; b0 < B; b0 += kMaxGridY) {
+    launch(b0, B - b0 < kMaxGridY ? B - b0 : kMaxGridY);
+    count_launch(1);
+  }
+}
+
 template <int CP>
 void pointwise_launch(sbse_fno *f, bool back, const float *S, const float *V, const __nv_bfloat16 *W, const float *bias,
                       const float *Uprev, float *U, float *out, int B, int act) {
-  dim3 g((unsigned)((f->ng + kPwT * kPw - 1) / (kPwT * kPw)), (unsigned)B);
-  if (back)
-    k_fo_pointwise_back<CP><<<g, kPwT, 0, f->stream>>>(V, W, S, Uprev, out, f->C, f->ng);
-  else
-    k_fo_pointwise<CP><<<g, kPwT, 0, f->stream>>>(S, V, W, bias, U, out, f->C, f->ng, act);
-  count_launch(1);
+  over_batch(B, [&](int b0, int nb) {
+    dim3 g((unsigned)((f->ng + kPwT * kPw - 1) / (kPwT * kPw)), (unsigned)nb);
+    const long long o = (long long)b0 * f->C * f->ng;
+    if (back)
+      k_fo_pointwise_back<CP><<<g, kPwT, 0, f->stream>>>(V + o, W, S + o, Uprev ? Uprev + o : nullptr, out + o, f->C, f->ng);
+    else
+      k_fo_pointwise<CP><<<g, kPwT, 0, f->stream>>>(S + o, V + o, W, bias, U ? U + o : nullptr, out + o, f->C, f->ng, act);
+  });
 }
 
 // the compiled channel count at or above C
@@ -451,8 +462,10 @@ int backward_impl(sbse_fno *f, int B, const float *x) {
   // projection: its weights' gradient with dy as the one row, the sum of dy is the bias's
   if ((rc = wgrad(f, f->dy, 1, Vl(f, L, B), C, B, f->grad + f->off_pw, f->grad + f->off_pb))) return rc;
   // the last layer has no activation: dU = dV
-  k_fno_project_back<<<dim3(nblk(ng), (unsigned)B), kT, 0, f->stream>>>(f->dy, f->par + f->off_pw, f->dU, C, ng);
-  count_launch(1);
+  over_batch(B, [&](int b0, int nb) {
+    k_fno_project_back<<<dim3(nblk(ng), (unsigned)nb), kT, 0, f->stream>>>(f->dy + b0 * ng, f->par + f->off_pw,
+                                                                          f->dU + b0 * C * ng, C, ng);
+  });
   for (int l = L - 1; l >= 0; --l) {
     if ((rc = wgrad(f, f->dU, C, Vl(f, l, B), C, B, f->grad + f->off_w[l], f->grad + f->off_b[l]))) return rc;
     // spectral: dG = c_kx / N^3 rfft(dU) on the kept modes (scaled as the mix reads it), dR, dF

@@ -406,3 +406,30 @@ def test_spectrum_of_a_diverged_surrogate_is_refused(B):
             with pytest.raises(B.SbseError) as e:
                 c.spectrum(5, vectors=vectors)
             assert e.value.code == B.SBSE_ERR_NUMERIC
+
+
+def test_fno_batch_beyond_a_grid_dimension(B):
+    """More batch entries than blocks in gridDim.y (65535): outputs and gradients are those of the same entries
+    in two parts (gradients: FP32 sums of 65605 terms in another grouping, sqrt(65605) 2^-24 = 1.5e-5 and a margin)."""
+    torch = pytest.importorskip("torch")
+    N, C, m, L, batch, part = 4, 2, 2, 2, 65535 + 70, 40000
+    gen = torch.Generator(device="cuda").manual_seed(1)
+    xd = torch.randn((batch, 2, N, N, N), generator=gen, device="cuda")
+    dyd = 1.0 + torch.randn((batch, N, N, N), generator=gen, device="cuda")
+    vec = _pack(ofno.init_params(C, m, L, seed=2))
+
+    def run(first, count):
+        net = B.FNO(N, width=C, modes=m, layers=L, max_batch=count)
+        net.set_params(vec)
+        x, dy, y = xd[first:first + count], dyd[first:first + count], torch.empty((count, N, N, N), device="cuda")
+        torch.cuda.synchronize()
+        net.forward(count, x.data_ptr(), y.data_ptr())
+        net.gradients(count, x.data_ptr(), dy.data_ptr())
+        g = net.get_params()[1].astype(np.float64)
+        net.close()
+        return y, g
+
+    y, g = run(0, batch)
+    (y0, g0), (y1, g1) = run(0, part), run(part, batch - part)
+    assert torch.equal(y, torch.cat([y0, y1]))
+    assert rel_err(g, g0 + g1) < 1e-4
