@@ -207,8 +207,8 @@ void launch_pair_norms(const double *phi, const int2 *pairs, int n_pairs, long l
 
 // ---- mixed hole-grid representation of A (mixed.cu), FP64; f, out: n_o rows of ng points
 void launch_exciton_density(const double *phi_o, const double *f, int n_o, long long ng, double *dn, cudaStream_t s);
-// out_j = tf_j + (v + scissor - eps_j - shift) f_j + dv phi_j - sum_i f_i W_ij
-void launch_abar(const double *tf, const double *f, const double *v, const double *eps_o, double scissor, double shift,
+// out_j += (v + scissor - eps_j - shift) f_j + dv phi_j - sum_i f_i W_ij
+void launch_abar(const double *f, const double *v, const double *eps_o, double scissor, double shift,
                  const double *dv, const double *phi_o, const double *W, int n_o, long long ng, double *out,
                  cudaStream_t s);
 // keep = 0: out_j -= sum_s <basis_s|out_j> basis_s; keep = 1: out_j = sum_s <basis_s|out_j> basis_s

@@ -23,15 +23,15 @@ __global__ void k_exciton_density(const double *phi_o, const double *f, int n_o,
   }
 }
 
-// out_j = tf_j + (v + scissor - eps_j - shift) f_j + dv phi_j - sum_i f_i W_ij (W in canonical slots)
-__global__ void k_abar(const double *tf, const double *f, const double *v, const double *eps_o, double scissor,
+// out_j += (v + scissor - eps_j - shift) f_j + dv phi_j - sum_i f_i W_ij (W in canonical slots)
+__global__ void k_abar(const double *f, const double *v, const double *eps_o, double scissor,
                        double shift, const double *dv, const double *phi_o, const double *W, int n_o, long long ng,
                        double *out) {
   const long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y;
   if (r >= ng) return;
   const long long o = (long long)j * ng + r;
-  double acc = tf[o] + (v[r] + scissor - eps_o[j] - shift) * f[o] + dv[r] * phi_o[o];
+  double acc = out[o] + (v[r] + scissor - eps_o[j] - shift) * f[o] + dv[r] * phi_o[o];
   for (int i = 0; i < n_o; ++i) {
     const int lo = i < j ? i : j, hi = i < j ? j : i;
     const int p = lo * n_o - lo * (lo - 1) / 2 + (hi - lo);
@@ -144,11 +144,11 @@ void launch_exciton_density(const double *phi_o, const double *f, int n_o, long 
   count_launch(1);
 }
 
-void launch_abar(const double *tf, const double *f, const double *v, const double *eps_o, double scissor, double shift,
+void launch_abar(const double *f, const double *v, const double *eps_o, double scissor, double shift,
                  const double *dv, const double *phi_o, const double *W, int n_o, long long ng, double *out,
                  cudaStream_t s) {
   dim3 grid((unsigned)((ng + kMxT - 1) / kMxT), n_o);
-  k_abar<<<grid, kMxT, 0, s>>>(tf, f, v, eps_o, scissor, shift, dv, phi_o, W, n_o, ng, out);
+  k_abar<<<grid, kMxT, 0, s>>>(f, v, eps_o, scissor, shift, dv, phi_o, W, n_o, ng, out);
   count_launch(1);
 }
 

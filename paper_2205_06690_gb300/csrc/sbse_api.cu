@@ -1063,24 +1063,23 @@ template <typename T> int run_direct_block(sbse_ctx *ctx, const std::vector<int>
 
 // ---- mixed hole-grid representation (Sec. II.C): A = Q A-bar on f_j(r), FP64 on the device
 struct MixedBufs {
-  double *tf;  // kinetic terms of the rows, padded to full slots, then the potential of the exciton density
   double *pwork, *dwork;
   C2<double> *pw;
 };
 
-int mixed_bufs(sbse_ctx *ctx, int n_extra_fields, MixedBufs *mb, double **extra) {
+// *extra: n_extra_vectors of n_o ng doubles. The last one is mixed_apply's `out`: it is followed by the fields
+// that the round trip writes beyond it (n_o odd: the empty half of its last slot; the exciton potential)
+int mixed_bufs(sbse_ctx *ctx, int n_extra_vectors, MixedBufs *mb, double **extra) {
   const long long ng = ctx->ng;
   const int n_o = ctx->n_o;
   // (not monotonic in the number of basis rows: fewer rows are cut into more chunks)
   const size_t pwd = std::max(project_work_doubles(n_o, ctx->n_occ, ng), project_work_doubles(n_o, ctx->n_c, ng));
-  const size_t slots = (size_t)(n_o + 1) / 2 + 1;
-  const size_t doubles = (2 * slots - 1) * ng + dot_work_doubles() + (size_t)n_extra_fields * n_o * ng;
+  const size_t slots = (size_t)(n_o + 1) / 2 + 1, beyond = 2 * slots - 1 - n_o;
+  const size_t doubles = dot_work_doubles() + ((size_t)n_extra_vectors * n_o + beyond) * ng;
   void *vp;
   int rc;
   if ((rc = ensure(ctx, WS_MIX, doubles * sizeof(double), &vp))) return rc;
-  double *p = (double *)vp;
-  mb->tf = p;
-  mb->dwork = mb->tf + (2 * slots - 1) * ng;
+  mb->dwork = (double *)vp;
   *extra = mb->dwork + dot_work_doubles();
   // the packed slots, and the projections' partial sums when the slots are done with
   if ((rc = ensure(ctx, WS_PW, std::max(slots * (size_t)ng * sizeof(C2<double>), pwd * sizeof(double)), &vp))) return rc;
@@ -1089,8 +1088,8 @@ int mixed_bufs(sbse_ctx *ctx, int n_extra_fields, MixedBufs *mb, double **extra)
   return SBSE_OK;
 }
 
-// out = Q (A-bar - shift) f for the n_o window rows f (device); projector 0: Q = 1 - P_occ, 1: onto
-// the conduction states
+// out = Q (A-bar - shift) f for the n_o window rows f (device; out: the last vector of mixed_bufs); projector
+// 0: Q = 1 - P_occ, 1: onto the conduction states
 int mixed_apply(sbse_ctx *ctx, int projector, const double *f, double *out, double shift, const MixedBufs &mb) {
   const long long ng = ctx->ng;
   const int n_o = ctx->n_o;
@@ -1099,8 +1098,8 @@ int mixed_apply(sbse_ctx *ctx, int projector, const double *f, double *out, doub
   XfwdArgs<double> xa{};
   xa.mode = XF_PACK_DN;
   // One round trip for the kinetic terms of the rows and the potential of the exciton density (held in `out`
-  // until the operator writes it): the passes of a few slots leave most SMs idle, so the density's slot is
-  // free (4 rows of 32^3: 106 us per term of the expansion, 159 with two trips).
+  // until the round trip has read it): the passes of a few slots leave most SMs idle, so the density's slot
+  // is free (4 rows of 32^3: 106 us per term of the expansion, 159 with two trips).
   launch_exciton_density(phi_o, f, n_o, ng, out, st);
   const int slots = (n_o + 1) / 2 + 1;
   xa.n_items = slots;
@@ -1108,9 +1107,9 @@ int mixed_apply(sbse_ctx *ctx, int projector, const double *f, double *out, doub
   xa.dn = f;
   xa.n_dn = n_o;
   xa.dn_last = out;
-  round_trip_poisson<double>(ctx, ctx->g64, xa, PoissonOut{2 * slots - 1, 1.0, 0.0, 0.0}, mb.tf, nullptr, nullptr, Z_HOLE_GRID);
-  const double *dv = mb.tf + (long long)(2 * slots - 2) * ng;
-  launch_abar(mb.tf, f, ctx->v64, ctx->eps_dev, ctx->scissor, shift, dv, phi_o, ctx->W, n_o, ng, out, st);
+  round_trip_poisson<double>(ctx, ctx->g64, xa, PoissonOut{2 * slots - 1, 1.0, 0.0, 0.0}, out, nullptr, nullptr, Z_HOLE_GRID);
+  const double *dv = out + (long long)(2 * slots - 2) * ng;
+  launch_abar(f, ctx->v64, ctx->eps_dev, ctx->scissor, shift, dv, phi_o, ctx->W, n_o, ng, out, st);
   if (projector == 0)
     launch_project(out, n_o, ctx->phi64, ctx->n_occ, ng, ctx->dV, 0, mb.pwork, st);
   else

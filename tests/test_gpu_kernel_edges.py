@@ -433,3 +433,35 @@ def test_fno_batch_beyond_a_grid_dimension(B):
     (y0, g0), (y1, g1) = run(0, part), run(part, batch - part)
     assert torch.equal(y, torch.cat([y0, y1]))
     assert rel_err(g, g0 + g1) < 1e-4
+
+
+def test_hole_grid_operator_at_a_memory_limit(B):
+    """At 4 rows the operator holds at most 18 FP64 fields (2 MiB each on 64^3) besides the context's own: six for
+    the operator, two vectors and two packed slots of two. Counted from the four fields of the boundary
+    potential."""
+    N, box, n_o, n_c = 64, 16.0, 4, 1
+    v, phi, eps = _orbitals(N, box, n_o + n_c, 5)
+    pairs = tdh.pair_list(n_o)
+    w = np.random.default_rng(2).standard_normal((len(pairs), N ** 3))
+    f = np.random.default_rng(3).standard_normal((n_o, N ** 3))
+
+    def least(call):
+        with B.Context(0, B.SBSE_FP64) as c:
+            c.set_grid(N, box, v)
+            c.set_orbitals(n_o, n_o, n_c, phi, eps, 0.5)
+            B.sbse_set_W(c.h, pairs, w)
+            for limit in range(1, 400):
+                B.sbse_set_option(c.h, B.SBSE_OPT_MEM_LIMIT_MB, limit)
+                try:
+                    return limit, call(c.h)
+                except B.SbseError as e:
+                    assert e.code == B.SBSE_ERR_OOM
+
+    first, _ = least(B.sbse_boundary_potential)
+    operator, at_limit = least(lambda h: B.sbse_apply_A_mixed(h, B.SBSE_Q_OCCUPIED, f))
+    assert operator - first <= 2 * (18 - 4) + 1
+    with B.Context(0, B.SBSE_FP64) as c:
+        c.set_grid(N, box, v)
+        c.set_orbitals(n_o, n_o, n_c, phi, eps, 0.5)
+        B.sbse_set_W(c.h, pairs, w)
+        assert np.array_equal(at_limit, B.sbse_apply_A_mixed(c.h, B.SBSE_Q_OCCUPIED, f))
