@@ -465,3 +465,50 @@ def test_hole_grid_operator_at_a_memory_limit(B):
         c.set_orbitals(n_o, n_o, n_c, phi, eps, 0.5)
         B.sbse_set_W(c.h, pairs, w)
         assert np.array_equal(at_limit, B.sbse_apply_A_mixed(c.h, B.SBSE_Q_OCCUPIED, f))
+
+
+@pytest.mark.parametrize("N,n_occ,n_o", [(16, 5, 1), (16, 6, 4), (32, 5, 3), (40, 5, 4), (48, 3, 2),  # four lanes per pencil
+                                         (9, 4, 2), (15, 4, 3), (54, 3, 1),                   # runtime radix
+                                         (18, 4, 3), (20, 6, 4), (45, 3, 2), (32, 8, 8)])     # a thread per pencil
+def test_hole_grid_operator_of_every_round_trip(B, N, n_occ, n_o):
+    """Kinetic multiplier of the rows' slots and Coulomb kernel of the last slot in each of the z passes, with
+    odd and even row counts."""
+    box = 0.4 * N
+    v, phi, eps = _orbitals(N, box, n_occ + 1, N + n_o)
+    g = tdh.Grid(N, box)
+    po = phi[n_occ - n_o:n_occ]
+    pairs = tdh.pair_list(n_o)
+    W = {(i, j): tdh.coulomb_periodic(po[i] * po[j], g) for i, j in pairs}
+    op = mixed.MixedA(g, v, phi, eps, n_occ, n_o, 1, W, 0.5, conduction_only=False)
+    f = op.Q(np.random.default_rng(N).standard_normal((n_o, N, N, N)))
+    with B.Context(0, B.SBSE_FP64) as c:
+        c.set_grid(N, box, v)
+        c.set_orbitals(n_occ, n_o, 1, phi, eps, 0.5)
+        B.sbse_bare_W(c.h, pairs)
+        got = B.sbse_apply_A_mixed(c.h, B.SBSE_Q_OCCUPIED, f.reshape(n_o, -1)).reshape(f.shape)
+    assert rel_err(got, op(f)) < 1e-10
+
+
+@pytest.mark.parametrize("scale", [1e-150, 1e-100, 1e100])
+@pytest.mark.parametrize("n", [2, 3, 40, 257])
+def test_eigenvalues_of_scaled_matrices(B, n, scale):
+    """Relative to the matrix's own norm, however small: a solver that returns zeros does not pass."""
+    a = scale * _sym(n, "dense")
+    ref = np.linalg.eigvalsh(a)
+    assert np.max(np.abs(_eig_noalloc(B, a, min(n, 12)) - ref[:12])) <= 10 * n * 2.2e-16 * np.max(np.abs(ref))
+
+
+def test_eigenvalues_of_the_zero_matrix(B):
+    assert np.array_equal(_eig_noalloc(B, np.zeros((40, 40)), 12), np.zeros(12))
+
+
+@pytest.mark.parametrize("N,n_pairs", [(32, 18), (32, 19), (48, 8), (48, 9), (64, 4), (64, 5), (80, 3), (80, 4), (96, 3)])
+def test_streamed_z_sweep_gives_the_bits_of_plain_loads(B, N, n_pairs):
+    """The z sweep fed by bulk copies (from 608 blocks of a pair's 32 columns on) and the one with plain loads
+    sum the same density terms in the same order; below the rule both options take the plain sweep."""
+    n_o, box = 6, 0.4 * N
+    pairs = tdh.pair_list(n_o)[:n_pairs]
+    v, phi, eps = _orbitals(N, box, n_o + 1, N)
+    prm = B.TDHParams(n_s=3, n_steps=5, clean_every=3, dt=0.05, gamma=0.1, alpha=1e-4, seed=3)
+    w = [_apply(B, B.SBSE_MIXED, N, box, v, phi, eps, n_o, n_o, 1, prm, pairs, SBSE_OPT_TMA_PLANES=tma) for tma in (0, 1)]
+    assert np.array_equal(w[0], w[1])
