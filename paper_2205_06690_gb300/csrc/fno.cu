@@ -268,7 +268,7 @@ struct sbse_fno {
   float2 *tw = nullptr, *fold = nullptr;
   float *kx_herm = nullptr;  // c_kx / N^3
   float *V = nullptr, *U = nullptr, *S = nullptr, *dV = nullptr, *dU = nullptr;
-  float2 *F = nullptr, *C1 = nullptr, *C2b = nullptr, *G = nullptr;
+  float2 *F = nullptr, *C1 = nullptr, *C2b = nullptr, *G = nullptr;  // (C1: direct sums only)
   float *y = nullptr, *dy = nullptr;
   double *red = nullptr, *gpart = nullptr, *gout = nullptr;
   size_t gpart_cap = 0;
@@ -299,7 +299,8 @@ template <typename X> int falloc(sbse_fno *f, X **p, size_t bytes) {
   return SBSE_OK;
 }
 
-// shared memory of the plane kernels beyond which the direct sums are used (planes of edge 200 and more)
+// shared memory of the plane kernels beyond which the direct sums are used: with every mode kept (m = N / 2) from
+// edge 144 on, with 12 modes from 507
 constexpr size_t kFoSmemMax = 200 * 1024;
 
 // spectral transform of the real fields [bc][z][y][x] -> F[bc][kz][ky][kx]
@@ -508,6 +509,7 @@ int sbse_fno_create(sbse_fno **out, int device, int n, int width, int modes, int
   f->maxB = max_batch;
   f->ng = (long long)n * n * n;
   f->modes = 4 * modes * modes * modes;
+  f->folded = fo_fwd_smem(n, modes) <= kFoSmemMax && fo_inv_smem(n, modes) <= kFoSmemMax;
   if (cudaSetDevice(device) != cudaSuccess || cudaStreamCreateWithFlags(&f->stream, cudaStreamNonBlocking) != cudaSuccess) {
     sbse::set_thread_error("FNO: CUDA setup failed");
     delete f;
@@ -549,7 +551,7 @@ int sbse_fno_create(sbse_fno **out, int device, int n, int width, int modes, int
   rc = rc ? rc : falloc(f, &f->dU, act * sizeof(float));
   rc = rc ? rc : falloc(f, &f->F, (size_t)layers * B * width * f->modes * sizeof(float2));
   rc = rc ? rc : falloc(f, &f->G, (size_t)B * width * f->modes * sizeof(float2));
-  rc = rc ? rc : falloc(f, &f->C1, (size_t)B * width * n * n * modes * sizeof(float2) + 64);
+  if (!f->folded) rc = rc ? rc : falloc(f, &f->C1, (size_t)B * width * n * n * modes * sizeof(float2) + 64);
   rc = rc ? rc : falloc(f, &f->C2b, (size_t)B * width * n * 2 * modes * modes * sizeof(float2) + 64);
   rc = rc ? rc : falloc(f, &f->y, B * f->ng * sizeof(float));
   rc = rc ? rc : falloc(f, &f->dy, B * f->ng * sizeof(float));
@@ -572,7 +574,6 @@ int sbse_fno_create(sbse_fno **out, int device, int n, int width, int modes, int
       fold[(size_t)p * (modes + 1) + k] = make_float2((float)cos(a), (float)sin(a));
     }
   cudaMemcpy(f->fold, fold.data(), fold.size() * sizeof(float2), cudaMemcpyHostToDevice);
-  f->folded = fo_fwd_smem(n, modes) <= kFoSmemMax && fo_inv_smem(n, modes) <= kFoSmemMax;
   if (f->folded) {
     raise_smem_limit((const void *)k_fo_fwd_xy, fo_fwd_smem(n, modes));
     raise_smem_limit((const void *)k_fo_inv_xy, fo_inv_smem(n, modes));

@@ -512,3 +512,21 @@ def test_streamed_z_sweep_gives_the_bits_of_plain_loads(B, N, n_pairs):
     prm = B.TDHParams(n_s=3, n_steps=5, clean_every=3, dt=0.05, gamma=0.1, alpha=1e-4, seed=3)
     w = [_apply(B, B.SBSE_MIXED, N, box, v, phi, eps, n_o, n_o, 1, prm, pairs, SBSE_OPT_TMA_PLANES=tma) for tma in (0, 1)]
     assert np.array_equal(w[0], w[1])
+
+
+def test_fno_holds_no_fields_of_the_direct_sums(B):
+    """A network whose transforms are folded allocates nothing for the direct sums (34 MB here): parameters and
+    their copies, activations, spectra and one field of the z transform."""
+    torch = pytest.importorskip("torch")
+    N, C, m, L, batch = 64, 32, 8, 1, 4
+    warm = B.FNO(8, width=2, modes=2, layers=1, max_batch=1)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    net = B.FNO(N, width=C, modes=m, layers=L, max_batch=batch)
+    used = free - torch.cuda.mem_get_info()[0]
+    act, modes, direct = batch * C * N ** 3 * 4, 4 * m ** 3, batch * C * N * N * m * 8
+    need = (L + 1 + L + 3) * act + (L + 1) * batch * C * modes * 8 + batch * C * N * 2 * m * m * 8 + 18 * net.n_params + \
+        2 * batch * N ** 3 * 4
+    assert used < need + direct // 2
+    net.close()
+    warm.close()
