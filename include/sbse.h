@@ -289,14 +289,16 @@ int sbse_get_stream(const sbse_ctx *ctx, void **stream);
  * per term, FP32 accumulation); 0 uses FP32 CUDA-core arithmetic. Errors: INVALID_ARG. */
 #define SBSE_OPT_TENSOR_CORES 1
 /* SBSE_OPT_CHUNK_MB (default 0): sbse_apply_W advances the pairs in chunks holding about this many
- * MiB of propagated orbitals, so that the three passes of a split-operator step find a chunk in the
- * L2 cache; 0 advances all pairs at once (fastest as separate launches: small launches leave
- * SMs idle). Results do not depend on it. */
+ * MiB of propagated orbitals, so that the passes of a split-operator step (two sweeps in SBSE_MIXED on
+ * grids with a register-pencil FFT, else three or five) find a chunk in the L2 cache; 0 advances all
+ * pairs at once (fastest as separate launches: small launches leave SMs idle). Results do not depend
+ * on it. */
 #define SBSE_OPT_CHUNK_MB 2
 /* SBSE_OPT_PERSISTENT (default 0): advance the eta0 set and all pairs by one split-operator step in
- * a single persistent kernel whose blocks pull tiles from a dependency-ordered queue (grids with a
- * register-pencil FFT); 0 uses three separate pass kernels, which are faster on GB300 (the merged
- * kernel is register-limited to fewer resident warps). Results do not depend on it. */
+ * a single persistent kernel whose blocks pull tiles from a dependency-ordered queue (grids of 8, 10, 12,
+ * 16, 20, 24, 32, 40, 48 and, in SBSE_MIXED, 64 points per axis); 0 uses separate pass kernels, which are
+ * faster on GB300 (the merged kernel is register-limited to fewer resident warps). Results do not depend
+ * on it. */
 #define SBSE_OPT_PERSISTENT 3
 /* SBSE_OPT_TMA_PLANES (default 1): in SBSE_MIXED on grids of 32, 48, 64, 80 or 96 points per axis, the
  * z sweep of a large pair batch (with the induced density of Eq. 11) is fed by bulk asynchronous
@@ -327,9 +329,11 @@ int sbse_kernel_launches(long long *count);
  * number of launches of one phase since the last reset (enable resets the counters).
  * phase: 0 = orbital propagation step (phase + 3D FFT + kinetic + inverse FFT + induced density),
  *        1 = Poisson solve and time-integral accumulation, 2 = cleaning, 3 = contractions (K, D),
- *        4 = A assembly + eigensolve; inside phase 0, the three passes over the pair batch on
- *        grids with the register-pencil FFT: 5 = forward plane pass (potential phase + x, y FFTs),
- *        6 = z-column pass (z FFT, kinetic phase, inverse z FFT), 7 = inverse plane pass (+ density).
+ *        4 = A assembly + eigensolve; inside phase 0, the passes over the pair batch on grids with
+ *        the register-pencil FFT. SBSE_MIXED: 5 = plane sweep (potential phase, x and y kinetic
+ *        operators), 7 = z sweep (z kinetic operator + density); SBSE_FP64: 5 = forward plane pass
+ *        (potential phase + x, y FFTs), 6 = z-column pass (z FFT, kinetic phase, inverse z FFT),
+ *        7 = inverse plane pass + density.
  *        Errors: INVALID_ARG, CUDA. */
 int sbse_profile(sbse_ctx *ctx, int enable);
 int sbse_phase_time(sbse_ctx *ctx, int phase, double *ms, long long *launches);

@@ -8,7 +8,7 @@ run of a batch goes one system at a time: under CUDA's lazy module loading the f
 kernel loads its module, which would invalidate another thread's graph capture in progress; after
 one run every kernel is loaded and every graph captured.
 `autotune` picks, per grid size and pair count, the fastest split-operator variant that the grid
-supports (three pass kernels or the persistent step kernel; plain or bulk-copy streamed passes;
+supports (separate pass kernels or the persistent step kernel; plain or bulk-copy streamed passes;
 all pairs per pass or L2-sized chunks of pairs) from a short timed trial, and caches the choice.
 """
 from __future__ import annotations

@@ -7,6 +7,8 @@
 
 namespace sbse {
 
+constexpr int kSMs = 152;  // streaming multiprocessors of a GB300 (four sub-partitions each), for launch rules
+
 template <typename T> struct Vec2;
 template <> struct Vec2<float> { using type = float2; };
 template <> struct Vec2<double> { using type = double2; };

@@ -226,10 +226,11 @@ template <typename T, int N> void few_attrs() {
 // 32^3, 160 warps: 11.3 + 4.6 + 5.1 -> 8.7 + 3.7 + 3.4 us). In FP64 the quartered pencils' extra
 // instructions (about 1.5 times as many) count once a quarter of the sub-partitions are busy: 2 slots of
 // 32^3, 64 warps: 32 + 31 + 41 -> 16 + 16 + 17 us; 5 slots of 40^3, 250 warps, were slower (fwd 62 -> 90,
-// inv 165 -> 220 us).
+// inv 165 -> 220 us). Edges: a warp holds 8 pencils, so multiples of 8, with a register transform of N / 4
+// points (that leaves out 24, a 6-point transform, and 56, 72, 80 and 96, whose slots are seldom few).
 template <typename T> bool few_items(int N, long long n_items) {
   if (N != 16 && N != 32 && N != 40 && N != 48 && N != 64) return false;
-  return n_items * N * N / 32 < (sizeof(T) == 8 ? 152 : 608);
+  return n_items * N * N / 32 < (sizeof(T) == 8 ? kSMs : 4 * kSMs);
 }
 
 int upload_few_twiddles() {

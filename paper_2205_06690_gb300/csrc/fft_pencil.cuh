@@ -223,7 +223,7 @@ template <typename T, int N> constexpr int kFew = few_ppb(N, kPPB<T, N>);
 template <typename T, int N> constexpr size_t few_plane_smem() {
   return (size_t)kFew<T, N> * N * (N + 1) * sizeof(C2<T>);
 }
-constexpr long long kFewBlocks = 76;
+constexpr long long kFewBlocks = kSMs / 2;
 template <typename T, int N> constexpr bool few_planes(long long planes) {
   return kFew<T, N> < kPPB<T, N> && planes / kPPB<T, N> < kFewBlocks;
 }
@@ -503,7 +503,8 @@ constexpr bool lane_pairs(int N) { return N == 32 || N == 48 || N == 64; }
 // queue; a tile waits (bounded) for the tiles it reads, whose queue positions are always earlier,
 // so every awaited tile is held by a running block and the launch cannot deadlock. The queue
 // pipelines pairs (forward tiles of pair j, z tiles of pair j-1, inverse tiles of pair j-2) so that
-// the orbitals in flight stay in L2 between the three passes.
+// the orbitals in flight stay in L2 between the passes (FP32: no z tiles of the pairs; the inverse tiles take
+// the z operator).
 
 __device__ __forceinline__ unsigned ld_acquire(const unsigned *p) {
   unsigned v;
@@ -770,11 +771,11 @@ template <typename T> struct FastOps {
       constexpr long long per_unit = (N * N + kZkT - 1) / kZkT;
       // the density summed in the sweep needs one block per pair and 128 columns, working through L orbitals
       // in turn: below two blocks per SM a second kernel sums it from the stored orbitals
-      if (dens && n_items / L * per_unit >= 304) {
+      if (dens && n_items / L * per_unit >= 2 * kSMs) {
         k_zkin<N, true><<<(unsigned)(n_items / L * per_unit), kZkT, 0, s>>>(view(g), d, a_next, dens, n_items / L, L);
         return;
       }
-      const int nt = n_items * per_unit < 152 ? 32 : kZkT;
+      const int nt = n_items * per_unit < kSMs ? 32 : kZkT;
       k_zkin<N, false><<<(unsigned)((long long)n_items * ((N * N + nt - 1) / nt)), nt, 0, s>>>(view(g), d, nullptr, nullptr,
                                                                                           n_items, 1);
       if (dens) launch_density<float>(g, d, a_next, n_items / L, L, dens, s);
@@ -784,7 +785,7 @@ template <typename T> struct FastOps {
     if constexpr (!(sizeof(T) == 8 && N > 48)) {
       // threads per block: 128, or one warp where 128 would leave SMs without a block
       const long long cols = (long long)n_items * N * N;
-      const int nt = cols < 128ll * 152 ? 32 : 128;
+      const int nt = cols < 128ll * kSMs ? 32 : 128;
       k_zcol<T, N><<<(unsigned)((cols + nt - 1) / nt), nt, 0, s>>>(view(g), d, cols, mult);
     }
   }

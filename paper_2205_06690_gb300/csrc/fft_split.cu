@@ -87,9 +87,13 @@ __global__ void __launch_bounds__(2 * N, N == 96 ? 2 : 3) k_plane_fwd2(GView<flo
 // one-dimensional operators F_a^-1 K_a F_a, one per axis, which commute. This pass applies the
 // potential phase (the pre-operation) and the x and y operators to one z-plane held in shared
 // memory (kin_roundtrip along each axis); the second sweep applies the z operator. One HBM round trip
-// per sweep: two per step instead of the three of a 3D FFT round trip. 36 pairs of 48^3 x 16 orbitals:
+// per sweep: two per step instead of the three of a 3D FFT round trip. 36 pairs of 48^3 x 10 orbitals:
 // 160 + 119 us (three thread-per-pencil sweeps: 147 + 113 + 113; the same two sweeps with a thread per pencil:
 // 208 + 157, held by 12 warps per SM); 10 pairs of 32^3: 14.1 us for the planes.
+
+// Mixed grids that took three thread-per-pencil sweeps before and two since (W of 10 pairs x 10 orbitals, three
+// against two): 20^3 6.5 -> 4.1 ms per 100 steps, 24^3 7.1 -> 4.6, 40^3 (streamed before) 13.1 -> 11.2; with lane
+// pairs 32^3 8.0 -> 5.5, 64^3 46.8 -> 33.4.
 
 // blocks per SM that the registers should allow: N points of a lane pair per thread pair
 constexpr int kin2_blocks(int N) { return N == 96 ? 2 : N == 80 ? 3 : N == 64 ? 5 : N == 48 ? 8 : 12; }
@@ -426,7 +430,7 @@ template <int N>
 void zkin2(const GridTables<float> &g, float2 *d, int n_items, const float2 *a_next, int L, float *dens,
            cudaStream_t s, int *err) {
   const int units = dens ? n_items / L : n_items;
-  if (dens && (long long)units * (N * N / kZtCw) < 608) {
+  if (dens && (long long)units * (N * N / kZtCw) < 4 * kSMs) {
     // a block works through its pair's L orbitals in turn: where that leaves most of the SMs' schedulers
     // without a warp, a second kernel sums the density from the stored orbitals (10 pairs x 4 orbitals of 32^3:
     // 5.5 + 5.7 us; 36 pairs of 48^3 take 119 us in one sweep)

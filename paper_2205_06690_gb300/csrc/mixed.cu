@@ -90,7 +90,7 @@ constexpr int kPrM = 4, kPrN = 8, kPrWarps = 4;
 
 long long project_chunk(long long ng, int n_o, int n_b) {
   const long long tiles = (long long)((n_o + kPrM - 1) / kPrM) * ((n_b + kPrN - 1) / kPrN);
-  const long long want = (152 * 16 + tiles - 1) / tiles;  // about 16 warps per SM
+  const long long want = (kSMs * 16 + tiles - 1) / tiles;  // about 16 warps per SM
   long long c = ((ng + want - 1) / want + 31) / 32 * 32;
   if (c > 4096) c = 4096;
   while ((ng + c - 1) / c > 4096) c *= 2;

@@ -640,7 +640,7 @@ int run_apply_W(sbse_ctx *ctx, const sbse_tdh_params *p, const std::vector<int> 
   }
   C *acur = a0, *anext = a1;
   // persistent step kernel: dependency-ordered tile queue and completion counters
-  // (the persistent step kernel exists for the thread-per-pencil sizes only, not for 80 and 96)
+  // (not for 80 and 96, nor for the further edges of fft_more.cu)
   const bool persistent = ctx->persistent && step_supported<T>(ctx->N);
   StepQueue sq{};
   int step_grid = 0;
@@ -755,7 +755,7 @@ int run_apply_W(sbse_ctx *ctx, const sbse_tdh_params *p, const std::vector<int> 
     // (which needs the new eta0) waits for it
     if (!eta0_issued && (rc = eta0_step(acur, anext, xa.pv))) return rc;
     eta0_issued = false;
-    // the three passes run over chunks of pairs (SBSE_OPT_CHUNK_MB, default: all pairs at once)
+    // the passes run over chunks of pairs (SBSE_OPT_CHUNK_MB, default: all pairs at once)
     for (int p0 = 0; p0 < P; p0 += chunk_pairs) {
       const int pc = std::min(chunk_pairs, P - p0);
       C *dc = d + (long long)p0 * L * ng;

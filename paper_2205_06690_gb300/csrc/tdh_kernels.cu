@@ -558,7 +558,7 @@ __global__ void k_density(long long ng, const C2<T> *d, const C2<T> *a, int L, T
 
 template <typename T>
 void launch_density(const GridTables<T> &g, const C2<T> *d, const C2<T> *a, int P, int L, T *dens, cudaStream_t s) {
-  const int nt = g.ng * P < 256ll * 304 ? 64 : 256;
+  const int nt = g.ng * P < 256ll * 2 * kSMs ? 64 : 256;
   dim3 grid((unsigned)((g.ng + nt - 1) / nt), P);
   k_density<T><<<grid, nt, 0, s>>>(g.ng, d, a, L, dens);
   count_launch(1);
@@ -646,7 +646,7 @@ constexpr int kOdC = 4, kOdS = 4, kOdWarps = 4;
 // warps of points
 static long long ov64_chunk(long long ng, int n_cols, int n_occ) {
   const long long tiles = (long long)((n_cols + kOdC - 1) / kOdC) * ((n_occ + kOdS - 1) / kOdS);
-  const long long want = (152 * 16 + tiles - 1) / tiles;
+  const long long want = (kSMs * 16 + tiles - 1) / tiles;
   long long c = ((ng + want - 1) / want + 31) / 32 * 32;
   if (c > 4096) c = 4096;  // a chunk's rows of d and phi stay in L2 while every tile reads them
   while ((ng + c - 1) / c > 4096) c *= 2;

@@ -606,7 +606,7 @@ static int umma_nt(int Nn) {
 
 static long long umma_kchunk(long long ng, int tiles) {
   // about two CTAs per SM across all tiles, whole stages per chunk
-  long long target = 304 / (tiles > 0 ? tiles : 1);
+  long long target = 2 * kSMs / (tiles > 0 ? tiles : 1);
   if (target < 1) target = 1;
   long long c = (ng + target - 1) / target;
   c = ((c + kUmBK - 1) / kUmBK) * kUmBK;
@@ -938,7 +938,7 @@ __global__ void __launch_bounds__(kOvThreads, 1)
 // grid of the streamed overlaps: (m tiles, chunks); about one CTA per SM, whole stages per chunk
 static void ov_grid(int n_cols, long long ng, int *m_tiles, long long *kc, long long *chunks) {
   *m_tiles = (n_cols + kOvCols - 1) / kOvCols;
-  long long target = 152 / *m_tiles;
+  long long target = kSMs / *m_tiles;
   if (target < 1) target = 1;
   long long c = (ng + target - 1) / target;
   c = ((c + kOvKS - 1) / kOvKS) * kOvKS;
