@@ -79,7 +79,7 @@ template <int N, int SIGN> __device__ __forceinline__ void fft2_dif(float2 (&v)[
 // leaving registers: on entry lane s holds x[2m + s], on return y[2m + s] (y = F^-1 K F x / N). Each
 // lane takes the half-length transform of its samples (E for the even ones, O for the odd ones),
 // receives the other lane's, forms E Kp + O M1 (lane 0: even outputs) or O Kp + E M2 (lane 1: odd
-// outputs), and transforms back. tab = [Kp | M1 | M2], N/2 entries each (see set_kinetic).
+// outputs), and transforms back. tab = [Kp | M1 | M2], N/2 entries each (kin_tables.h).
 template <int N>
 __device__ __forceinline__ void kin_roundtrip(float2 (&v)[N / 2], int s, const float2 *tab) {
   constexpr int H = N / 2;

@@ -74,17 +74,16 @@ template <typename T, int N> constexpr size_t plane_smem() {
 
 // ------------------------------------------------------------------------------------------
 
-// One-dimensional kinetic operator F^-1 diag(kt) F of a pencil in registers (kt = kin / N)
+// One-dimensional kinetic operator F^-1 diag(kt) F of a pencil in registers (kt: a table of kin_tables.h)
 template <int N> __device__ __forceinline__ void kin_pencil(float2 (&v)[N], const float2 *kt) {
   fft_reg<float, N, -1, TwP<float>>(v);
 #pragma unroll
   for (int k = 0; k < N; ++k) v[k] = cmul(v[k], kt[k]);
   fft_reg<float, N, +1, TwP<float>>(v);
 }
-// kt of the block, K / N rounded once (a rounded 1 / N would scale every transform of every step by the same
-// error); the caller synchronises
-template <int N> __device__ __forceinline__ void load_kin(float2 *kt, const GView<float> &g) {
-  for (int i = threadIdx.x; i < N; i += blockDim.x) kt[i] = g.kin[N + 3 * (N / 2) + i];
+// the table of a sweep (`at`: kin_xy(N) or kin_z(N)); the caller synchronises
+template <int N> __device__ __forceinline__ void load_kin(float2 *kt, const GView<float> &g, int at) {
+  for (int i = threadIdx.x; i < N; i += blockDim.x) kt[i] = g.kin[at + i];
 }
 
 // The PPB planes starting at plane offset `off` (= z0 N^2) of `item`: the fused pre-operation, then the
@@ -250,7 +249,7 @@ __global__ void __launch_bounds__(PPB * N) k_plane_kin(GView<float> g, XfwdArgs<
   constexpr int NN = N * N;
   extern __shared__ unsigned char smem_raw[];
   __shared__ float2 kt[N];
-  load_kin<N>(kt, g);  // (read after the pre-operation's barrier)
+  load_kin<N>(kt, g, kin_xy(N));  // (read after the pre-operation's barrier)
   const long long p0 = (long long)blockIdx.x * PPB;
   const long long item = p0 / N;
   (void)SBSE_IDX(p0 + PPB - 1, planes_total);
@@ -289,7 +288,7 @@ __global__ void __launch_bounds__(kZkT)
   constexpr int NN = N * N;
   __shared__ C kt[N];
   __shared__ float D[DENS ? N * kZkT : 1];
-  load_kin<N>(kt, g);
+  load_kin<N>(kt, g, kin_z(N));
   __syncthreads();
   const long long cols = (NN + blockDim.x - 1) / blockDim.x;  // blocks per unit
   const long long unit = blockIdx.x / cols;
@@ -526,7 +525,7 @@ __device__ __forceinline__ bool wait_geq(const unsigned *p, unsigned target, uns
 template <int N>
 __device__ __forceinline__ void step_tile_pairs(const GView<float> &g, const XfwdArgs<float> &fa, const XfwdArgs<float> &fp,
                                                 float2 *a_next, float2 *d, float *dens, int L, int4 it, float2 *S,
-                                                const float2 *tab) {
+                                                const float2 *tab, const float2 *ztab) {
   using C = float2;
   constexpr int PPB = kPPB<float, N>, NN = N * N, NT = PPB * N, H = N / 2;
   static_assert(PPB % 2 == 0, "two halves of PPB / 2 planes");
@@ -556,7 +555,7 @@ __device__ __forceinline__ void step_tile_pairs(const GView<float> &g, const Xfw
       C v[H];
 #pragma unroll
       for (int m = 0; m < H; ++m) v[m] = __ldcg(base + (long long)(2 * m + s) * NN);
-      kin_roundtrip<N>(v, s, tab);
+      kin_roundtrip<N>(v, s, ztab);
 #pragma unroll
       for (int m = 0; m < H; ++m) base[(long long)(2 * m + s) * NN] = v[m];
       if (pair) {
@@ -590,11 +589,13 @@ __global__ void __launch_bounds__(kPPB<T, N> * N)
   // with lane pairs where the sweeps take them
   constexpr bool KIN = sizeof(T) == 4;
   constexpr bool LP = KIN && lane_pairs(N);
-  __shared__ C kt[LP ? 3 * N / 2 : KIN ? N : 1];
-  if constexpr (LP) {  // (read after the first tile's barrier)
-    for (int i = threadIdx.x; i < 3 * N / 2; i += blockDim.x) kt[i] = g.kin[N + i];
-  } else if constexpr (KIN) {
-    load_kin<N>(kt, g);
+  constexpr int NK = LP ? 3 * N / 2 : KIN ? N : 1;
+  __shared__ C kt[2 * NK];  // of the planes, and from NK of the z operator (read after the first tile's barrier)
+  if constexpr (KIN) {
+    for (int i = threadIdx.x; i < NK; i += blockDim.x) {
+      kt[i] = g.kin[kin_xy(N) + i];
+      kt[NK + i] = g.kin[kin_z(N) + i];
+    }
   }
   const unsigned tgt = (q.epoch + 1) * (unsigned)G;
   for (;;) {
@@ -623,7 +624,7 @@ __global__ void __launch_bounds__(kPPB<T, N> * N)
     if (it.x < 0) break;
     if (go) {
       if constexpr (LP) {
-        step_tile_pairs<N>(g, fa, fp, a_next, d, dens, L, it, S, kt);
+        step_tile_pairs<N>(g, fa, fp, a_next, d, dens, L, it, S, kt, kt + NK);
       } else if constexpr (KIN) {
         const int rem = it.z * NT + threadIdx.x;
         switch (it.x) {
@@ -638,7 +639,7 @@ __global__ void __launch_bounds__(kPPB<T, N> * N)
               C v[N];
 #pragma unroll
               for (int z = 0; z < N; ++z) v[z] = __ldcg(base + (long long)z * NN);
-              kin_pencil<N>(v, kt);
+              kin_pencil<N>(v, kt + NK);
 #pragma unroll
               for (int z = 0; z < N; ++z) base[(long long)z * NN] = v[z];
               if (pair) add_density<N, true>(v, a_next + (long long)l * g.ng + rem, D + threadIdx.x, NT, l == 0);

@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(2 * N, kin2_blocks(N)) k_plane_kin2(GView<floa
   const int z = (int)(blockIdx.x / (unsigned)n_items);
   const long long item = (long long)blockIdx.x - (long long)z * n_items;
   __shared__ float2 tab[3 * H];
-  for (int i = threadIdx.x; i < 3 * H; i += blockDim.x) tab[i] = g.kin[N + i];
+  for (int i = threadIdx.x; i < 3 * H; i += blockDim.x) tab[i] = g.kin[kin_xy(N) + i];
   kin2_plane<N, PAIR>(g, a, item, (long long)z * NN, reinterpret_cast<float2 *>(smem_raw), tab, threadIdx.x);
 }
 
@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(128, N >= 80 ? 3 : DENS || N == 64 ? 4 : 6) k_
   constexpr int NN = N * N, H = N / 2, UB = 16;
   __shared__ float D[DENS ? N * kZDPitch : 1];
   __shared__ C tab[3 * H];
-  for (int i = threadIdx.x; i < 3 * H; i += blockDim.x) tab[i] = g.kin[N + i];
+  for (int i = threadIdx.x; i < 3 * H; i += blockDim.x) tab[i] = g.kin[kin_z(N) + i];
   __syncthreads();
   const int cs = (int)(blockIdx.x / (unsigned)n_units);
   const int unit = (int)blockIdx.x - cs * n_units;
@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(2 * kZtCw, N >= 80 ? 5 : N == 64 ? 7 : 10)
     tma_bar_expect(&bar, kStage);
     tma_load_3d(St, &dmap, 2 * cs * kZtCw, 0, (int)item0, &bar);
   }
-  for (int i = threadIdx.x; i < 3 * H; i += blockDim.x) tab[i] = g.kin[N + i];
+  for (int i = threadIdx.x; i < 3 * H; i += blockDim.x) tab[i] = g.kin[kin_z(N) + i];
   __syncthreads();
   const int lane = threadIdx.x & 31, s = lane >> 4, cw = (threadIdx.x >> 5) * 16 + (lane & 15);
   const int rem = cs * kZtCw + cw;

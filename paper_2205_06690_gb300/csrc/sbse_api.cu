@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "kernels.h"
+#include "kin_tables.h"
 #include "sbse.h"
 #include "smem_limit.h"
 
@@ -298,9 +299,7 @@ template <typename T> int build_tables(sbse_ctx *ctx, GridTables<T> &g, const do
   }
   int rc;
   if ((rc = dalloc(ctx, &g.tw, N * sizeof(C2<T>)))) return rc;
-  // per-axis kinetic factors (N), then for even N the lane-pair round-trip multipliers (3 N / 2), then the
-  // factors over N
-  if ((rc = dalloc(ctx, &g.kin, (2 * N + 3 * (N / 2)) * sizeof(C2<T>)))) return rc;
+  if ((rc = dalloc(ctx, &g.kin, kin_entries(N) * sizeof(C2<T>)))) return rc;
   if ((rc = dalloc(ctx, &g.k2, N * sizeof(T)))) return rc;
   if ((rc = dalloc(ctx, &g.v_loc, ctx->ng * sizeof(T)))) return rc;
   if ((rc = dalloc(ctx, &g.pv_dt, ctx->ng * sizeof(C2<T>)))) return rc;
@@ -314,31 +313,26 @@ template <typename T> int build_tables(sbse_ctx *ctx, GridTables<T> &g, const do
   return SBSE_OK;
 }
 
-// kinetic propagator per axis: exp(-i k_m^2 dt / 2); the 3D factor is the product over axes
+// kinetic propagator per axis: exp(-i k_m^2 dt / 2); the 3D factor is the product over axes. FP32 grids whose step
+// has two sweeps also get the tables of these (kin_tables.h), weighted for orbitals with momenta of about one
+// (a Gaussian in k of that width squared, bohr).
 template <typename T> int set_kinetic(sbse_ctx *ctx, GridTables<T> &g, double dt) {
-  const int N = ctx->N, H = N / 2;
-  std::vector<C2<T>> kin(2 * N + 3 * H);
-  std::vector<double> kr(N), ki(N);
+  const int N = ctx->N;
+  std::vector<C2<T>> kin(kin_entries(N));
+  std::vector<Cd> K(N);
+  std::vector<double> weight(N);
   for (int m = 0; m < N; ++m) {
     const double kk = kval(m, N, ctx->box);
     const double ph = -0.5 * dt * kk * kk;
-    kr[m] = cos(ph);
-    ki[m] = sin(ph);
-    kin[m] = C2<T>{(T)kr[m], (T)ki[m]};
-    kin[N + 3 * H + m] = C2<T>{(T)(kr[m] / N), (T)(ki[m] / N)};
+    K[m] = Cd(cos(ph), sin(ph));
+    weight[m] = exp(-0.5 * kk * kk);
+    kin[m] = C2<T>{(T)K[m].real(), (T)K[m].imag()};
   }
-  // The one-dimensional kinetic operator F^-1 diag(K) F on the even and odd samples (one per lane
-  // of a lane pair): with E, O the half-length transforms, the even outputs are the inverse
-  // half-length transform of E Kp + O M1 and the odd ones of O Kp + E M2, where
-  // Kp = (K_k + K_k+H) / N, M1 = W^k (K_k - K_k+H) / N, M2 = W^-k (K_k - K_k+H) / N, W = exp(-2 pi i / N).
-  if (N % 2 == 0) {
-    for (int k = 0; k < H; ++k) {
-      const double pr = (kr[k] + kr[k + H]) / N, pi = (ki[k] + ki[k + H]) / N;
-      const double mr = (kr[k] - kr[k + H]) / N, mi = (ki[k] - ki[k + H]) / N;
-      const double wr = cos(-2.0 * M_PI * k / N), wi = sin(-2.0 * M_PI * k / N);
-      kin[N + k] = C2<T>{(T)pr, (T)pi};
-      kin[N + H + k] = C2<T>{(T)(wr * mr - wi * mi), (T)(wr * mi + wi * mr)};
-      kin[N + 2 * H + k] = C2<T>{(T)(wr * mr + wi * mi), (T)(wr * mi - wi * mr)};
+  if (sizeof(T) == 4 && fast_supported<T>(N)) {
+    const KinAxes axes = kin_axes(K, weight, pair_size(N) || split_size(N));
+    for (size_t i = 0; i < axes.xy.size(); ++i) {
+      kin[kin_xy(N) + i] = C2<T>{(T)axes.xy[i].real(), (T)axes.xy[i].imag()};
+      kin[kin_z(N) + i] = C2<T>{(T)axes.z[i].real(), (T)axes.z[i].imag()};
     }
   }
   CK(cudaMemcpyAsync(g.kin, kin.data(), kin.size() * sizeof(C2<T>), cudaMemcpyHostToDevice, ctx->stream));

@@ -10,15 +10,19 @@
 
 namespace sbse {
 
+__host__ __device__ constexpr int kin_xy(int N) { return N; }
+__host__ __device__ constexpr int kin_z(int N) { return 2 * N + N / 2; }
+__host__ __device__ constexpr int kin_entries(int N) { return 4 * N; }
+
 // Device tables of one grid, in working precision T.
 template <typename T> struct GridTables {
   int N = 0;
   long long ng = 0;
   FftPlan plan{};
   C2<T> *tw = nullptr;      // exp(-2 pi i k / N), k < N
-  C2<T> *kin = nullptr;     // exp(-i k_m^2 dt / 2) per axis index m (rebuilt per dt); for even N
-                            // followed by the lane-pair round-trip multipliers Kp, M1, M2 (N/2 each),
-                            // then the factors over N
+  C2<T> *kin = nullptr;     // exp(-i k_m^2 dt / 2) per axis index m (rebuilt per dt), then the FP32
+                            // tables of the two sweeps at kin_xy(N) and kin_z(N): N entries, or the
+                            // lane-pair multipliers Kp, M1, M2 (N / 2 each)
   T *k2 = nullptr;          // k_m^2 per axis index m
   T *v_loc = nullptr;       // V_loc(r), ng
   C2<T> *pv_dt = nullptr;   // exp(-i V_loc dt), ng (rebuilt per dt)
