@@ -229,11 +229,10 @@ void launch_sigma_from_residues(const double *R, int K, const double *cw, const 
 
 // ---- absorption spectrum by a Chebyshev expansion of A (spectrum.cu)
 struct SpectrumBufs {
-  double *f0, *cw, *hist, *R, *D, *omega, *sigma, *squares;
+  double *f0, *cw, *hist, *R, *D, *omega, *sigma;
 };
-// squares: with room for T_2 and T_4 of the matrix where rounds of four terms pay; without it, single terms
-size_t spectrum_work_bytes(int n, int n_terms, int n_omega, bool squares);
-SpectrumBufs spectrum_bufs(double *work, int n, int n_terms, int n_omega, bool squares);
+size_t spectrum_work_bytes(int n, int n_terms, int n_omega);
+SpectrumBufs spectrum_bufs(double *work, int n, int n_terms, int n_omega);
 // the caller fills b.omega (n_omega frequencies) before; b.sigma and b.R (n_terms residues) after
 // *err is set if a bounded wait between the terms runs out; false: the launch failed
 bool launch_absorption(const SpectrumBufs &b, const double *phi_o, const double *phi_c, int n_o, int n_c, int N,

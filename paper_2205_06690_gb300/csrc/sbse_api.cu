@@ -2045,16 +2045,8 @@ int sbse_absorption(sbse_ctx *ctx, int axis, int n_terms, double broadening, int
   const int n = ctx->n_o * ctx->n_c;
   void *vp;
   int rc;
-  // where the squares of the matrix don't fit, the recursion advances by single terms
-  bool squares = true;
-  rc = ensure(ctx, WS_SPEC, spectrum_work_bytes(n, n_terms, n_omega, true), &vp);
-  if (rc == SBSE_ERR_OOM) {
-    squares = false;
-    ctx->err.clear();
-    rc = ensure(ctx, WS_SPEC, spectrum_work_bytes(n, n_terms, n_omega, false), &vp);
-  }
-  if (rc) return rc;
-  const SpectrumBufs b = spectrum_bufs((double *)vp, n, n_terms, n_omega, squares);
+  if ((rc = ensure(ctx, WS_SPEC, spectrum_work_bytes(n, n_terms, n_omega), &vp))) return rc;
+  const SpectrumBufs b = spectrum_bufs((double *)vp, n, n_terms, n_omega);
   cudaStream_t st = ctx->stream;
   CK(cudaMemcpyAsync(b.omega, omega, (size_t)n_omega * sizeof(double), cudaMemcpyHostToDevice, st));
   const double *phi_o = ctx->phi64 + (long long)(ctx->n_occ - ctx->n_o) * ctx->ng;

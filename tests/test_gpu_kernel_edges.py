@@ -530,3 +530,25 @@ def test_fno_holds_no_fields_of_the_direct_sums(B):
     assert used < need + direct // 2
     net.close()
     warm.close()
+
+
+def test_absorption_residues_keep_64_bits(B):
+    """Residues of many terms against the recursion in extended precision, on the library's own A: within one
+    rounding (2^-53) per term, root mean square."""
+    N, box, n_o, n_c, terms = 12, 6.0, 10, 11, 2048
+    v, phi, eps = _orbitals(N, box, n_o + n_c, 7)
+    with B.Context(0, B.SBSE_FP64) as c:
+        c.set_grid(N, box, v)
+        c.set_orbitals(n_o, n_o, n_c, phi, eps, 0.5)
+        A = c.build_A(B.SBSE_EXCHANGE)
+        _, res = c.absorption(0, terms, 0.2, np.linspace(0.1, 4.0, 5))
+    f0 = spectrum.dipoles(tdh.Grid(N, box), phi[:n_o], phi[n_o:], 0).astype(np.longdouble)
+    mid, half = spectrum.scaling(A)
+    m = (A.astype(np.longdouble) - np.longdouble(mid) * np.eye(len(A))) / np.longdouble(half)
+    prev, cur = f0, m @ f0
+    ref = [f0 @ prev, f0 @ cur]
+    for _ in range(2, terms):
+        prev, cur = cur, 2 * (m @ cur) - prev
+        ref.append(f0 @ cur)
+    ref = np.array(ref)
+    assert np.sqrt(np.sum((res - ref) ** 2) / np.sum(ref ** 2)) <= terms * 2.0 ** -53
