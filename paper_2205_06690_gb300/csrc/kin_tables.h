@@ -9,8 +9,8 @@
 // (about 0.5 ms, once per grid and time step). The sum over three axes stays near 3e-8 per step; with K / N rounded
 // on every axis it was up to 2.4e-7, and on 20, 30 and 40 points W of 60 steps was 2 to 3 times as far from 64 bits as
 // with 3D transforms. Error of W against 64 bits (200 steps; 3D transforms, or one table for the lane pairs of
-// 80 and 96, against these): 20^3 2.3e-6, 4.8e-7; 30^3 8.1e-7, 6.9e-7; 40^3 1.8e-6, 8.1e-7; 48^3 9.4e-6, 1.4e-6;
-// 64^3 4.5e-6, 3.0e-6; 96^3 1.1e-5, 6.8e-6. (60^3 2.1e-6, 3.3e-6: there the former errors happened to cancel.)
+// 80 and 96, against these): 20^3 2.3e-6, 6.1e-7; 30^3 8.1e-7, 7.9e-7; 40^3 1.8e-6, 8.1e-7; 48^3 9.4e-6, 1.1e-6;
+// 60^3 2.3e-6, 2.1e-6; 64^3 4.5e-6, 3.3e-6; 96^3 1.1e-5, 6.8e-6.
 #pragma once
 
 #include <math.h>

@@ -314,8 +314,8 @@ template <typename T> int build_tables(sbse_ctx *ctx, GridTables<T> &g, const do
 }
 
 // kinetic propagator per axis: exp(-i k_m^2 dt / 2); the 3D factor is the product over axes. FP32 grids whose step
-// has two sweeps also get the tables of these (kin_tables.h), weighted for orbitals with momenta of about one
-// (a Gaussian in k of that width squared, bohr).
+// has two sweeps also get the tables of these (kin_tables.h), weighted with exp(-k^2) (bohr), the momenta of
+// orbitals in wells of about one bohr.
 template <typename T> int set_kinetic(sbse_ctx *ctx, GridTables<T> &g, double dt) {
   const int N = ctx->N;
   std::vector<C2<T>> kin(kin_entries(N));
@@ -325,7 +325,7 @@ template <typename T> int set_kinetic(sbse_ctx *ctx, GridTables<T> &g, double dt
     const double kk = kval(m, N, ctx->box);
     const double ph = -0.5 * dt * kk * kk;
     K[m] = Cd(cos(ph), sin(ph));
-    weight[m] = exp(-0.5 * kk * kk);
+    weight[m] = exp(-kk * kk);
     kin[m] = C2<T>{(T)K[m].real(), (T)K[m].imag()};
   }
   if (sizeof(T) == 4 && fast_supported<T>(N)) {
